@@ -193,7 +193,9 @@ dem_status dem_stats(dem_ctx *ctx, dem_stats_t *out);
 
 /* Capture dem_step in CUDA graphs of `steps_per_graph` steps (0 disables).
  * The neighbour-list rebuild sits in a conditional node set by the step
- * kernel, so a captured run needs no host round trip. */
+ * kernel, so a captured run needs no host round trip.  dem_step runs the graph
+ * as often as it fits and for a remainder of at least a quarter of its steps
+ * (fused steps: for any remainder); the rest it launches step by step. */
 dem_status dem_set_graph(dem_ctx *ctx, int32_t steps_per_graph);
 
 /* Threads per block of the step kernel (the fused force and integration of Eqs. 1-6):
@@ -222,7 +224,8 @@ dem_status dem_set_step_block(dem_ctx *ctx, int32_t threads);
 dem_status dem_set_step_lanes(dem_ctx *ctx, int32_t lanes);
 
 /* How a captured graph (dem_set_graph) runs its steps.  1: one step-kernel launch per step,
- * each preceded by a conditional list-build node.  2: fused steps: one cooperative launch
+ * with a conditional list-build node before every fifth (a kernel that finds a list build
+ * due leaves its step to the loop at the graph's end).  2: fused steps: one cooperative launch
  * (one block per 128-slot tile, or as many blocks as are resident at once, each walking a
  * range of tiles) runs every step up to the next list build, with a grid barrier
  * between steps (the last block to arrive ends the step for every instance); the graph loops
@@ -253,7 +256,7 @@ dem_status dem_set_list_build(dem_ctx *ctx, int32_t staged);
 dem_status dem_test_stall_barrier(dem_ctx *ctx);
 
 /* CUDA-event time of step kernels of the most recent graph launch: every fifth
- * step kernel of the graph (the first, the sixth, ...) is bracketed by event
+ * step kernel of the graph (the first, the sixth, ... that its steps reach) is bracketed by event
  * nodes; total_ms = the sum over those, count = their number (total_ms / count is
  * the mean duration of a step kernel).  Synchronises the stream.  DEM_ERR_STATE if
  * no graph was built. */

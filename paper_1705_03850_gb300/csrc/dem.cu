@@ -1293,14 +1293,36 @@ __device__ __forceinline__ void step_finish_instances(const Dev& d)
     }
 }
 
+// What a step kernel inside a graph does besides its step.  Step kernels of a graph are launched
+// in runs of several behind one conditional list build: a kernel that finds a list build pending,
+// or no step left to do, does nothing (the graph's loop at the end makes up for the steps left
+// out), so that no step runs on lists that are out of date.
+struct StepCtl {
+    int counted;                           // 0: a launch of its own (no graph): always steps
+    int set_rb, set_loop;                  // set the condition h_rb (a list build is due) / h_loop (steps remain)
+    cudaGraphConditionalHandle h_rb, h_loop;
+};
+
 template <int MODE, bool WALLS, int BS = TILE, int LPP = 1>
-__global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int prime, cudaGraphConditionalHandle hnext, int use_cond)
+__global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int prime, StepCtl ctl)
 {
     __shared__ InstC sc;
     __shared__ InstD sd;
     __shared__ float smax[BS / 32];
     __shared__ bool am_last;
     int kstaged = -1;
+    if (MODE == 0 && ctl.counted) {
+        // written only by the ends of earlier kernels, so every block decides alike
+        const unsigned any = __ldcg(&d.g->any);
+        const long long rem = __ldcg(&d.g->remain);
+        if (any != 0u || rem <= 0) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                if (ctl.set_rb) cudaGraphSetConditional(ctl.h_rb, any != 0u && rem > 0 ? 1u : 0u);
+                if (ctl.set_loop) cudaGraphSetConditional(ctl.h_loop, rem > 0 ? 1u : 0u);
+            }
+            return;
+        }
+    }
     step_pass<MODE, WALLS, BS, LPP>(d, prime, sc, sd, smax, kstaged);
     if (MODE == 0) {
         // the last block to finish accumulates the bound per instance and decides on rebuilds
@@ -1317,7 +1339,13 @@ __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int 
             if (threadIdx.x == 0) {
                 d.g->counter = 0u;
                 d.g->pool = 0u;                 // every block has left its claim loop
-                if (use_cond) cudaGraphSetConditional(hnext, atomicOr(&d.g->any, 0u) ? 1u : 0u);
+                if (ctl.counted) {
+                    const long long rem = __ldcg(&d.g->remain) - 1;
+                    d.g->remain = rem;
+                    if (ctl.set_rb)
+                        cudaGraphSetConditional(ctl.h_rb, rem > 0 && atomicOr(&d.g->any, 0u) ? 1u : 0u);
+                    if (ctl.set_loop) cudaGraphSetConditional(ctl.h_loop, rem > 0 ? 1u : 0u);
+                }
             }
         }
     }
@@ -1411,13 +1439,19 @@ __global__ void __launch_bounds__(TILE, 5) k_steps(Dev d, cudaGraphConditionalHa
     }
 }
 
-// the start of a fused graph launch: S steps to do, a list build first if one is pending
-__global__ void k_steps_init(Dev d, long long S, cudaGraphConditionalHandle h_rb, cudaGraphConditionalHandle h_loop)
+// the start of a graph launch: S steps to do (or the number set for this launch), a list build
+// first if one is pending
+__global__ void k_steps_init(Dev d, long long S, cudaGraphConditionalHandle h_rb, cudaGraphConditionalHandle h_loop,
+                             int set_loop)
 {
-    d.g->remain = S;
+    const long long t = d.g->todo > 0 ? d.g->todo : S;
+    d.g->todo = 0;
+    d.g->remain = t;
     cudaGraphSetConditional(h_rb, d.g->any ? 1u : 0u);
-    cudaGraphSetConditional(h_loop, S > 0 ? 1u : 0u);
+    if (set_loop) cudaGraphSetConditional(h_loop, t > 0 ? 1u : 0u);
 }
+
+__global__ void k_set_todo(Dev d, long long n) { d.g->todo = n; }
 
 __global__ void k_set_cond(Dev d, cudaGraphConditionalHandle h)
 {
@@ -2332,11 +2366,29 @@ dem_status launch_rebuild(dem_ctx* ctx, cudaStream_t st)
     return DEM_OK;
 }
 
+// Lists valid for the current state, on the context's stream: nothing to do when nothing ran since
+// the last build that could ask for one; the chain when a state was written; otherwise the chain
+// behind one condition, where a graph holds it (one launch instead of eleven kernels that find
+// nothing to do), else the chain.
+dem_status ensure_lists(dem_ctx* ctx)
+{
+    if (ctx->lists_ok) return DEM_OK;
+    if (ctx->rb_if && !ctx->must_build) {
+        CU(cudaGraphLaunch(ctx->rb_if, ctx->stream));
+    } else {
+        dem_status st = launch_rebuild(ctx, ctx->stream);
+        if (st) return st;
+    }
+    ctx->lists_ok = true;
+    ctx->must_build = false;
+    return DEM_OK;
+}
+
 dem_status launch_eval(dem_ctx* ctx)
 {
-    dem_status st = launch_rebuild(ctx, ctx->stream);
+    dem_status st = ensure_lists(ctx);
     if (st) return st;
-    k_step<1, true><<<ctx->grid1, TILE, 0, ctx->stream>>>(ctx->dev, ctx->fresh ? 1 : 0, 0, 0);
+    k_step<1, true><<<ctx->grid1, TILE, 0, ctx->stream>>>(ctx->dev, ctx->fresh ? 1 : 0, StepCtl{});
     CU(cudaGetLastError());
     return DEM_OK;
 }
@@ -2359,9 +2411,14 @@ void destroy_graph(dem_ctx* ctx)
     ctx->ev0.clear();
     ctx->ev1.clear();
     if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
+    if (ctx->rb_if) cudaGraphExecDestroy(ctx->rb_if);
     if (ctx->graph) cudaGraphDestroy(ctx->graph);
+    if (ctx->rb_if_graph) cudaGraphDestroy(ctx->rb_if_graph);
     if (ctx->rb_graph) cudaGraphDestroy(ctx->rb_graph);
     ctx->gexec = nullptr;
+    ctx->rb_if = nullptr;
+    ctx->rb_if_graph = nullptr;
+    ctx->last_graph_steps = 0;
     ctx->graph = nullptr;
     ctx->rb_graph = nullptr;
 }
@@ -2410,14 +2467,14 @@ int step_grid(const dem_ctx* ctx)
 dem_status launch_step(dem_ctx* ctx, int prime)
 {
     Dev dv = ctx->dev;
-    cudaGraphConditionalHandle h = 0;
-    int use_cond = 0;
-    void* args[] = {&dv, &prime, &h, &use_cond};
+    StepCtl ctl{};
+    void* args[] = {&dv, &prime, &ctl};
     CU(cudaLaunchKernel(step_func(ctx), dim3(step_grid(ctx)), dim3(step_block(ctx)), args, step_smem(ctx), ctx->stream));
     return DEM_OK;
 }
 
-constexpr int EV_EVERY = 5;    // step kernels per timed one in a graph
+constexpr int EV_EVERY = 5;    // step kernels per run of a graph (one conditional list build, one of them timed)
+constexpr int GRAPH_PART = 4;  // a graph also runs a remainder of at least 1/GRAPH_PART of its steps
 
 // the fused step kernel for the context's walls and lanes per particle
 void* fused_func(const dem_ctx* ctx)
@@ -2442,7 +2499,8 @@ dem_status build_fused_graph(dem_ctx* ctx, cudaGraph_t g, int S)
     long long SS = S;
     cudaGraphNode_t init;
     {
-        void* args[] = {&dv, &SS, &h_rb, &h_loop};
+        int set_loop = 1;
+        void* args[] = {&dv, &SS, &h_rb, &h_loop, &set_loop};
         cudaKernelNodeParams kp{};
         kp.func = (void*)k_steps_init;
         kp.gridDim = dim3(1);
@@ -2505,6 +2563,31 @@ dem_status build_graph(dem_ctx* ctx, int S)
     if (st) return st;
     if (ce != cudaSuccess) return fail(ctx, DEM_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(ce));
     ctx->rb_graph = rb;
+    {
+        // the chain behind one condition (ensure_lists)
+        cudaGraph_t c;
+        CU(cudaGraphCreate(&c, 0));
+        ctx->rb_if_graph = c;
+        cudaGraphConditionalHandle h;
+        CU(cudaGraphConditionalHandleCreate(&h, c, 0, 0));
+        Dev dv = ctx->dev;
+        void* args[] = {&dv, &h};
+        cudaKernelNodeParams kp{};
+        kp.func = (void*)k_set_cond;
+        kp.gridDim = dim3(1);
+        kp.blockDim = dim3(1);
+        kp.kernelParams = args;
+        cudaGraphNode_t kn, cn, child;
+        CU(cudaGraphAddKernelNode(&kn, c, nullptr, 0, &kp));
+        cudaGraphNodeParams cp{};
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = h;
+        cp.conditional.type = cudaGraphCondTypeIf;
+        cp.conditional.size = 1;
+        CU(cudaGraphAddNode(&cn, c, &kn, nullptr, 1, &cp));
+        CU(cudaGraphAddChildGraphNode(&child, cp.conditional.phGraph_out[0], nullptr, 0, rb));
+        CU(cudaGraphInstantiate(&ctx->rb_if, c, 0));
+    }
     cudaGraph_t g;
     CU(cudaGraphCreate(&g, 0));
     ctx->graph = g;
@@ -2525,60 +2608,89 @@ dem_status build_graph(dem_ctx* ctx, int S)
         if (ctx->graph_mode == 2 || (ctx->graph_mode == 0 && can && live * ctx->step_lanes <= ctx->grid_fused))
             return build_fused_graph(ctx, g, S);
     }
-    std::vector<cudaGraphConditionalHandle> h(S);
-    for (int i = 0; i < S; ++i) CU(cudaGraphConditionalHandleCreate(&h[i], g, 0, 0));
+    // S steps in runs of EV_EVERY step kernels, each run behind one conditional list build, then a
+    // loop of (conditional list build, step kernel) for the steps that kernels left out because a
+    // loop of (conditional list build, step kernel) for the steps that kernels left out because a
+    // build became due within their run.  A condition per run instead of per step: the node costs
+    // about 5 us between two kernels, and builds are hundreds of steps apart (100 steps of a
+    // 187,504-sphere silo: 3536 against 4058 us, of the 1M bed 10149 against 10730 us).
+    const int runs = (S + EV_EVERY - 1) / EV_EVERY;
+    std::vector<cudaGraphConditionalHandle> h(runs);
+    cudaGraphConditionalHandle h_rb, h_loop;
+    for (int i = 0; i < runs; ++i) CU(cudaGraphConditionalHandleCreate(&h[i], g, 0, 0));
+    CU(cudaGraphConditionalHandleCreate(&h_rb, g, 0, 0));
+    CU(cudaGraphConditionalHandleCreate(&h_loop, g, 0, 0));
     Dev dv = ctx->dev;
     cudaGraphNode_t prev;
     {
         cudaKernelNodeParams kp{};
-        void* args[] = {&dv, &h[0]};
-        kp.func = (void*)k_set_cond;
+        long long SS = S;
+        int set_loop = 0;
+        void* args[] = {&dv, &SS, &h[0], &h_loop, &set_loop};
+        kp.func = (void*)k_steps_init;
         kp.gridDim = dim3(1);
         kp.blockDim = dim3(1);
         kp.kernelParams = args;
         CU(cudaGraphAddKernelNode(&prev, g, nullptr, 0, &kp));
     }
-    // CUDA events around every EV_EVERY-th step kernel (each pair of event nodes adds a few
-    // microseconds to the step, so the timing is sampled)
-    const int nev = (S + EV_EVERY - 1) / EV_EVERY;
-    ctx->ev0.resize(nev);
-    ctx->ev1.resize(nev);
-    for (int i = 0; i < nev; ++i) {
+    // CUDA events around the first step kernel of every run (it always steps unless none is left)
+    ctx->ev0.resize(runs);
+    ctx->ev1.resize(runs);
+    for (int i = 0; i < runs; ++i) {
         CU(cudaEventCreate(&ctx->ev0[i]));
         CU(cudaEventCreate(&ctx->ev1[i]));
     }
-    for (int i = 0; i < S; ++i) {
+    // a conditional node (if or while) after `after` (nullptr: first), holding the rebuild chain if asked
+    auto cond_node = [&](cudaGraph_t in, cudaGraphNode_t* node, cudaGraphNode_t* after, cudaGraphConditionalHandle hh,
+                         bool loop, bool chain, cudaGraph_t* body) -> cudaError_t {
         cudaGraphNodeParams cp{};
         cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = h[i];
-        cp.conditional.type = cudaGraphCondTypeIf;
+        cp.conditional.handle = hh;
+        cp.conditional.type = loop ? cudaGraphCondTypeWhile : cudaGraphCondTypeIf;
         cp.conditional.size = 1;
-        cudaGraphNode_t cn;
-        CU(cudaGraphAddNode(&cn, g, &prev, nullptr, 1, &cp));
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
+        cudaError_t e = cudaGraphAddNode(node, in, after, nullptr, after ? 1 : 0, &cp);
+        if (e != cudaSuccess) return e;
+        if (body) *body = cp.conditional.phGraph_out[0];
         cudaGraphNode_t child;
-        CU(cudaGraphAddChildGraphNode(&child, body, nullptr, 0, rb));
+        return chain ? cudaGraphAddChildGraphNode(&child, cp.conditional.phGraph_out[0], nullptr, 0, rb) : cudaSuccess;
+    };
+    auto step_node = [&](cudaGraph_t in, cudaGraphNode_t* node, cudaGraphNode_t* after, StepCtl ctl) -> cudaError_t {
         int prime = 0;
-        int use_cond = i + 1 < S ? 1 : 0;
-        cudaGraphConditionalHandle hn = i + 1 < S ? h[i + 1] : h[i];
-        void* args[] = {&dv, &prime, &hn, &use_cond};
+        void* args[] = {&dv, &prime, &ctl};
         cudaKernelNodeParams kp{};
         kp.func = step_func(ctx);
         kp.gridDim = dim3(step_grid(ctx));
         kp.blockDim = dim3(step_block(ctx));
         kp.sharedMemBytes = step_smem(ctx);
         kp.kernelParams = args;
+        return cudaGraphAddKernelNode(node, in, after, 1, &kp);
+    };
+    for (int i = 0; i < S; ++i) {
         cudaGraphNode_t kn;
+        const int run = i / EV_EVERY;
         if (i % EV_EVERY == 0) {
-            cudaGraphNode_t e0, e1;
-            CU(cudaGraphAddEventRecordNode(&e0, g, &cn, 1, ctx->ev0[i / EV_EVERY]));
-            CU(cudaGraphAddKernelNode(&kn, g, &e0, 1, &kp));
-            CU(cudaGraphAddEventRecordNode(&e1, g, &kn, 1, ctx->ev1[i / EV_EVERY]));
-            prev = e1;
-        } else {
-            CU(cudaGraphAddKernelNode(&kn, g, &cn, 1, &kp));
-            prev = kn;
+            cudaGraphNode_t cn, e0;
+            CU(cond_node(g, &cn, &prev, h[run], false, true, nullptr));
+            CU(cudaGraphAddEventRecordNode(&e0, g, &cn, 1, ctx->ev0[run]));
+            prev = e0;
         }
+        StepCtl ctl{1, 0, 0, 0, 0};
+        if (i + 1 == S) ctl = StepCtl{1, 1, 1, h_rb, h_loop};
+        else if ((i + 1) % EV_EVERY == 0) ctl = StepCtl{1, 1, 0, h[run + 1], 0};
+        CU(step_node(g, &kn, &prev, ctl));
+        prev = kn;
+        if (i % EV_EVERY == 0) {
+            cudaGraphNode_t e1;
+            CU(cudaGraphAddEventRecordNode(&e1, g, &prev, 1, ctx->ev1[run]));
+            prev = e1;
+        }
+    }
+    {
+        cudaGraphNode_t loop, ifn, kn;
+        cudaGraph_t body;
+        CU(cond_node(g, &loop, &prev, h_loop, true, false, &body));
+        CU(cond_node(body, &ifn, nullptr, h_rb, false, true, nullptr));
+        CU(step_node(body, &kn, &ifn, StepCtl{1, 1, 1, h_rb, h_loop}));
     }
     CU(cudaGraphInstantiate(&ctx->gexec, g, 0));
     ctx->graph_steps = S;
@@ -2859,7 +2971,7 @@ dem_status dem_write(dem_ctx* ctx, int32_t field, const void* src, int64_t n)
         dsrc = ctx->dev.stage;
     }
     if (field == DEM_F_WALL_XI) {            // the floor histories of the lists of this state: build them first
-        dem_status st = launch_rebuild(ctx, ctx->stream);
+        dem_status st = ensure_lists(ctx);
         if (st) return st;
     }
     k_write_field<<<nblk(n, 256), 256, 0, ctx->stream>>>(ctx->dev, field, dsrc, n, ctx->d_hl);
@@ -2870,6 +2982,8 @@ dem_status dem_write(dem_ctx* ctx, int32_t field, const void* src, int64_t n)
         CU(cudaGetLastError());
         ctx->fresh = true;
         ctx->have_state = true;
+        ctx->lists_ok = false;
+        ctx->must_build = true;
     }
     if (dsrc == ctx->dev.stage) CU(cudaStreamSynchronize(ctx->stream));
     return DEM_OK;
@@ -2925,7 +3039,7 @@ dem_status dem_read_neighbors(dem_ctx* ctx, int32_t* partner, int32_t width, int
     if (dem_status st = refresh_count(ctx)) return st;
     if (n != total_count(ctx) || width < 1 || !partner) return fail(ctx, DEM_ERR_ARG, "bad neighbour arguments");
     if (!is_device_ptr(partner)) return fail(ctx, DEM_ERR_ARG, "neighbour buffer must be device memory");
-    dem_status st = launch_rebuild(ctx, ctx->stream);
+    dem_status st = ensure_lists(ctx);
     if (st) return st;
     k_read_neighbors<<<nblk(ctx->ncap, 256), 256, 0, ctx->stream>>>(ctx->dev, partner, width);
     CU(cudaGetLastError());
@@ -2940,7 +3054,7 @@ dem_status dem_write_contacts(dem_ctx* ctx, const int32_t* partner, const double
     if (dem_status st = refresh_count(ctx)) return st;
     if (n != total_count(ctx) || width < 1 || !partner || !xi) return fail(ctx, DEM_ERR_ARG, "bad contacts arguments");
     if (!is_device_ptr(partner) || !is_device_ptr(xi)) return fail(ctx, DEM_ERR_ARG, "contacts buffers must be device memory");
-    dem_status st = launch_rebuild(ctx, ctx->stream);
+    dem_status st = ensure_lists(ctx);
     if (st) return st;
     k_write_contacts<<<nblk(ctx->ncap, 256), 256, 0, ctx->stream>>>(ctx->dev, partner, xi, width);
     CU(cudaGetLastError());
@@ -2955,16 +3069,26 @@ dem_status dem_step(dem_ctx* ctx, int64_t nsteps)
     if (!ctx->have_state) return fail(ctx, DEM_ERR_STATE, "write the state before stepping");
     int64_t done = 0;
     while (done < nsteps) {
-        if (!ctx->fresh && ctx->gexec && nsteps - done >= ctx->graph_steps) {
+        // the graph, also for a remainder of at least 1/GRAPH_PART of its steps (the step kernels
+        // beyond it find none left and end at once, about 4 us each with their share of the graph's
+        // other nodes, where a step launched alone comes with the eleven kernels of the rebuild
+        // chain, 25 us); fused steps run any number
+        const int64_t left = nsteps - done;
+        if (!ctx->fresh && ctx->gexec && (ctx->graph_fused || left * GRAPH_PART >= ctx->graph_steps)) {
+            const int64_t now = std::min<int64_t>(left, ctx->graph_steps);
+            if (now < ctx->graph_steps) k_set_todo<<<1, 1, 0, ctx->stream>>>(ctx->dev, (long long)now);
             CU(cudaGraphLaunch(ctx->gexec, ctx->stream));
-            done += ctx->graph_steps;
+            ctx->last_graph_steps = (int)now;
+            ctx->lists_ok = false;
+            done += now;
             continue;
         }
-        dem_status st = launch_rebuild(ctx, ctx->stream);
+        dem_status st = ensure_lists(ctx);
         if (st) return st;
         st = launch_step(ctx, ctx->fresh ? 1 : 0);
         if (st) return st;
         ctx->fresh = false;
+        ctx->lists_ok = false;
         ++done;
     }
     ctx->steps += nsteps;
@@ -3132,13 +3256,16 @@ dem_status dem_graph_step_kernel_ms(dem_ctx* ctx, double* total_ms, int32_t* cou
     if (!ctx->gexec) return fail(ctx, DEM_ERR_STATE, "no step graph has been built");
     CU(cudaStreamSynchronize(ctx->stream));
     double t = 0.0;
-    for (size_t i = 0; i < ctx->ev0.size(); ++i) {
+    // the runs that the last launch's steps reached
+    const int ls = ctx->last_graph_steps > 0 ? ctx->last_graph_steps : ctx->graph_steps;
+    const size_t nev = ctx->graph_fused ? ctx->ev0.size() : std::min(ctx->ev0.size(), (size_t)((ls + EV_EVERY - 1) / EV_EVERY));
+    for (size_t i = 0; i < nev; ++i) {
         float ms = 0.f;
         CU(cudaEventElapsedTime(&ms, ctx->ev0[i], ctx->ev1[i]));
         t += ms;
     }
     *total_ms = t;
-    *count = ctx->graph_fused ? (int32_t)ctx->graph_steps : (int32_t)ctx->ev0.size();
+    *count = ctx->graph_fused ? (int32_t)ls : (int32_t)nev;
     return DEM_OK;
 }
 
@@ -3382,8 +3509,9 @@ dem_status dem_rollout_forward(dem_ctx* ctx, int64_t nsteps, int64_t checkpoint_
     ro.K = checkpoint_every;
     ro.ncp = (int)ro.ck.size();
     ro.prime0 = ctx->fresh;
-    dem_status st = launch_rebuild(ctx, ctx->stream);       // the lists the whole rollout uses
+    dem_status st = ensure_lists(ctx);                      // the lists the whole rollout uses
     if (st) return st;
+    ctx->lists_ok = false;
     if ((st = set_frozen(ctx, 1u))) return st;
     for (long long s = 0; s < nsteps; ++s) {
         if (s % ro.K == 0 && (st = snap(ctx, ro.ck[s / ro.K], true))) return st;

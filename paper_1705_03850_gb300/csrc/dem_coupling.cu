@@ -1406,9 +1406,9 @@ dem_status dem_couple(dem_coupler* cp)
     if (ctx->status) return check_status(ctx);
     // both levels must be current and their lists valid; work on the fine level's stream,
     // after everything queued on the coarse level's (an event, no host wait)
-    dem_status st = launch_rebuild(coarse, coarse->stream);
+    dem_status st = ensure_lists(coarse);
     if (st) return st;
-    if ((st = launch_rebuild(ctx, ctx->stream))) return st;
+    if ((st = ensure_lists(ctx))) return st;
     cudaStream_t s = ctx->stream;
     if (coarse->stream != s) {
         CU(cudaEventRecord(cp->ready, coarse->stream));
@@ -1440,6 +1440,7 @@ dem_status dem_couple(dem_coupler* cp)
     // no host wait: the device updated the count and the offsets (k_cp_append) and reports an
     // overflow in the status word; the host copy of the count is refreshed when next needed
     ctx->count_stale = true;
+    ctx->lists_ok = false;         // rows that did not fit fall back to a list build
     return DEM_OK;
 }
 

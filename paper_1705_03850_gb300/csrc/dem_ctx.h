@@ -44,6 +44,10 @@ struct dem_ctx {
     bool walls = false;               // some instance has axisymmetric walls (step kernel variant)
     bool count_stale = false;         // a coupling call changed the IDs handed out on the device
     bool have_state = false;
+    // host knowledge of the lists: lists_ok, no list build can be pending on the device (nothing
+    // ran since the last one that could ask for one); must_build, one certainly is (a written state)
+    bool lists_ok = false;
+    bool must_build = true;
     long long steps = 0;
     unsigned status = 0;
     std::string err;
@@ -53,9 +57,12 @@ struct dem_ctx {
     bool graph_fused = false;         // the current graph runs its steps in fused cooperative launches
     int grid_fused = 0;               // co-resident blocks of the fused step kernel (0: unknown)
     cudaGraph_t rb_graph = nullptr;
+    cudaGraph_t rb_if_graph = nullptr;   // the rebuild chain behind one condition, for calls that need valid
+    cudaGraphExec_t rb_if = nullptr;     // lists (reads, coupling): a launch instead of the chain's eleven
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
-    std::vector<cudaEvent_t> ev0, ev1;   // around each step kernel of the graph
+    std::vector<cudaEvent_t> ev0, ev1;   // around every EV_EVERY-th step kernel of the graph
+    int last_graph_steps = 0;            // steps of the most recent graph launch
     std::vector<double> nu;              // Poisson ratio per instance (for material updates)
     std::vector<double> rmax;            // largest radius per instance [m]
     struct Rollout {
@@ -74,6 +81,7 @@ dem_status fail(dem_ctx* c, dem_status st, const std::string& msg);
 dem_status check_status(dem_ctx* ctx);
 dem_status refresh_count(dem_ctx* ctx);
 dem_status launch_rebuild(dem_ctx* ctx, cudaStream_t st);
+dem_status ensure_lists(dem_ctx* ctx);
 dem_status launch_eval(dem_ctx* ctx);
 long long total_count(const dem_ctx* ctx);
 void set_thread_error(const std::string& msg);

@@ -143,7 +143,8 @@ struct Glob {
     int err_pad;               //  4 contact pass of the step kernel)
     unsigned bar_gen;          // fused steps: grid-barrier generation (bumped by each release)
     unsigned bar_pad;
-    long long remain;          // fused steps: steps still to do in the current graph launch
+    long long remain;          // steps still to do in the current graph launch
+    long long todo;            // steps of the next graph launch (0: as many as the graph was built for)
     int nlive;                 // entries of live_tiles
     unsigned test_stall;       // 1: the next fused launch's first block skips its first barrier
     unsigned pool;             // SM-wide step blocks: slices claimed from the shared pool this launch
