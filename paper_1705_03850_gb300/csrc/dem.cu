@@ -824,6 +824,20 @@ constexpr int step_minb()
     return BS == SMW_BS ? 1 : LPP == 1 ? DEM_STEP_MINB * TILE / BS : 5;
 }
 
+// Stride (ints) between entries of the rows that fused steps stage in shared memory, entry-major:
+// the lanes of a group read neighbouring entries of one slot, and with this padding a warp's 32
+// reads fall into 32 banks.  Dynamic shared memory of a fused launch: the contact pass's staging
+// slots (64 B a thread), then the rows and the row lengths.
+__host__ __device__ constexpr int row_stride(int lpp, int threads)
+{
+    return (threads / lpp + 31) / 32 * 32 + (lpp == 1 ? 0 : 32 / lpp);
+}
+__host__ __device__ constexpr int fused_smem(int lpp, int threads, int lmax)
+{
+    return threads * 64 + 4 * (lmax * row_stride(lpp, threads) + threads / lpp);
+}
+constexpr int FUSED_T = 640;   // most threads of a fused block (96 registers a thread: one such block per SM)
+
 // Particle state: neighbours' through the read-only data cache, except in fused steps, where the
 // state is rewritten during the launch (by other blocks for the neighbours): there every state
 // load goes to L2 (ordered after the previous step's writes by the grid barrier's fences), so
@@ -849,15 +863,20 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void* src)
 
 // One step over the block's units (MODE 0: force, kick and drift of every particle; MODE 1:
 // forces only), ending with the block's displacement maximum folded into its last instance.
-// sc, sd, smax: the block's shared staging of the current instance and of the warp maxima.
+// sc, sd, smax: the block's shared staging of the current instance and of the warp maxima (a fused
+// step of a single instance leaves the block's maximum in smax[0], for the kernel's own barrier).
+// rows, rcnt: the rows and row lengths of the block's slots staged in shared memory (fused steps,
+// blocks of one unit; nullptr: read from the lists).
 // FUSED: called once per step by the fused kernel; kstaged: the instance staged in sc and sd at
 // the end of the previous step (-1: none), kept so that a block of one instance stages it once
 // per launch and then only flips its state buffer (all else in them is constant between list
 // builds).
 template <int MODE, bool WALLS, int BS, int LPP, bool FUSED = false>
-__device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, InstD& sd, float* smax, int& kstaged)
+__device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, InstD& sd, float* smax, int& kstaged,
+                                          const int* rows = nullptr, const int* rcnt = nullptr)
 {
-    constexpr int WPB = BS / 32;             // warps per block
+    const int nthr = FUSED ? (int)blockDim.x : BS;   // fused steps choose their block size by the system's
+    const int WPB = nthr / 32;               // warps per block
     constexpr int SPW = 32 / LPP;            // slots per warp
     constexpr int WPT = TILE / SPW;          // warp slices per tile
     static_assert(BS == 64 || BS == 128 || BS == 256 || BS == SMW_BS, "step block of 64, 128, 256 or SMW_BS threads");
@@ -876,7 +895,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
     // their blocks busy); the step kernel walks every tile (a lookup per unit costs it 4 %)
     const int nlive = FUSED ? *(volatile int*)&d.g->nlive : d.ntiles;
     const bool all_live = !FUSED || nlive == d.ntiles;   // then no lookup
-    const int NU = nlive * WPT / WPB;
+    const int NV = nlive * WPT;              // warp slices; whole units except in fused steps of one instance
+    const int NU = FUSED ? (NV + WPB - 1) / WPB : NV / WPB;
     const int u0 = (int)((long long)blockIdx.x * NU / gridDim.x);
     const int u1 = (int)((long long)(blockIdx.x + 1) * NU / gridDim.x);
     const int ncap = d.ncap;
@@ -888,6 +908,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         __syncthreads();
     }
     float runmax = 0.f;
+    const int rstride = FUSED ? row_stride(LPP, nthr) : 0;
     // SM-wide blocks: block b's share [v0(b), v1(b)) of the slices of the tiles that hold live
     // slots (a contiguous range: the instance's live slots come first).  Its warps claim
     // [v0(b), v1(b) - P) in order from the shared counter snext; the last P slices of every
@@ -953,7 +974,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
                 runmax = 0.f;
             }
             __syncthreads();
-            for (int i = threadIdx.x; i < (int)(sizeof(InstC) / 4); i += BS) ((int*)&sc)[i] = ((const int*)(d.ic + k))[i];
+            for (int i = threadIdx.x; i < (int)(sizeof(InstC) / 4); i += nthr) ((int*)&sc)[i] = ((const int*)(d.ic + k))[i];
             if (threadIdx.x < (int)(sizeof(InstD) / 4))
                 ((int*)&sd)[threadIdx.x] = FUSED ? __ldcg((const int*)(d.id + k) + threadIdx.x)
                                                  : ((const int*)(d.id + k))[threadIdx.x];
@@ -964,6 +985,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         // warp slice w' of tile t takes the 32-slot slice (w' + t) mod 4: rebuilds put the rows
         // with the most contacts in the first slice, so the rotation evens out the warps' work
         if (!SMW) vw = u * WPB + ((int)threadIdx.x >> 5);
+        if (FUSED && vw >= NV) continue;
         const int t = all_live ? vw / WPT : d.live_tiles[vw / WPT];
         const int s = t * TILE + (((vw & (WPT - 1)) + t) & (WPT - 1)) * SPW + lane / LPP;
         if (s - c.slot0 >= sd.n) continue;
@@ -984,8 +1006,12 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         const float dt_hist = prime ? 0.f : c.dt;
         V3 F = sub == 0 ? m * v3(c.g[0], c.g[1], c.g[2]) : v3(0.f, 0.f, 0.f);
         V3 Tq = v3(0.f, 0.f, 0.f);
-        const int ncnt = d.cnt[lp][s];
+        const int ls = FUSED ? ((int)threadIdx.x >> 5) * SPW + lane / LPP : 0;   // slot within the block's unit
+        const int ncnt = FUSED && rows ? rcnt[ls] : d.cnt[lp][s];
         const int* nb = d.nbr[lp] + s;
+        auto entry = [&](int e) -> int {
+            return FUSED && rows ? rows[e * rstride + ls] : __ldg(nb + (size_t)e * ncap);
+        };
         float* h = d.hist[lp] + s;
         float* ho = MODE == 1 ? d.xi_out + s : h;
         const int per0 = c.per[0], per1 = c.per[1], ext0 = c.ext[0], ext1 = c.ext[1], hf0 = c.half[0],
@@ -996,10 +1022,10 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         unsigned tm = 0u;
         // the first batch of indices is loaded before the row length arrives (rows hold at
         // least d.Lmax entries of storage); entries beyond the row are replaced by this slot
-        int jn0 = sub < d.Lmax ? __ldg(nb + (size_t)sub * ncap) : s;
-        int jn1 = sub + LPP < d.Lmax ? __ldg(nb + (size_t)(sub + LPP) * ncap) : s;
-        int jn2 = sub + 2 * LPP < d.Lmax ? __ldg(nb + (size_t)(sub + 2 * LPP) * ncap) : s;
-        int jn3 = sub + 3 * LPP < d.Lmax ? __ldg(nb + (size_t)(sub + 3 * LPP) * ncap) : s;
+        int jn0 = sub < d.Lmax ? entry(sub) : s;
+        int jn1 = sub + LPP < d.Lmax ? entry(sub + LPP) : s;
+        int jn2 = sub + 2 * LPP < d.Lmax ? entry(sub + 2 * LPP) : s;
+        int jn3 = sub + 3 * LPP < d.Lmax ? entry(sub + 3 * LPP) : s;
         jn0 = sub < ncnt ? jn0 : s;
         jn1 = sub + LPP < ncnt ? jn1 : s;
         jn2 = sub + 2 * LPP < ncnt ? jn2 : s;
@@ -1025,10 +1051,10 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
             int4 Qb[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) Qb[k] = ld_state<FUSED>(pos + jb[k]);
-            if (e0 + 4 * LPP < ncnt) jn0 = __ldg(nb + (size_t)(e0 + 4 * LPP) * ncap);
-            if (e0 + 5 * LPP < ncnt) jn1 = __ldg(nb + (size_t)(e0 + 5 * LPP) * ncap);
-            if (e0 + 6 * LPP < ncnt) jn2 = __ldg(nb + (size_t)(e0 + 6 * LPP) * ncap);
-            if (e0 + 7 * LPP < ncnt) jn3 = __ldg(nb + (size_t)(e0 + 7 * LPP) * ncap);
+            if (e0 + 4 * LPP < ncnt) jn0 = entry(e0 + 4 * LPP);
+            if (e0 + 5 * LPP < ncnt) jn1 = entry(e0 + 5 * LPP);
+            if (e0 + 6 * LPP < ncnt) jn2 = entry(e0 + 6 * LPP);
+            if (e0 + 7 * LPP < ncnt) jn3 = entry(e0 + 7 * LPP);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int4 Q = Qb[k];
@@ -1063,8 +1089,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         // position and overlap as well costs L1 capacity (the slots come out of it) and is 2 %
         // slower
         float4* stg;
-        if constexpr (SMW) {
-            extern __shared__ float4 stg_dyn[];     // 2 * 2 * BS float4 (57 kB: above the static limit)
+        if constexpr (SMW || FUSED) {
+            extern __shared__ float4 stg_dyn[];     // 2 * 2 * nthr float4 (SM-wide: 57 kB, above the static limit)
             stg = stg_dyn;
         } else {
             __shared__ float4 stg_st[2 * 2 * BS];
@@ -1072,13 +1098,13 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         }
         const int tid = (int)threadIdx.x;
         auto saddr = [&](int sl, int f) -> unsigned {
-            return (unsigned)__cvta_generic_to_shared(&stg[(sl * 2 + f) * BS + tid]);
+            return (unsigned)__cvta_generic_to_shared(&stg[(sl * 2 + f) * nthr + tid]);
         };
         int4 Qn = P;
         float hxn = 0.f, hyn = 0.f, hzn = 0.f;
         auto issue = [&](int sl, int en_) {
             const size_t o1 = (size_t)en_ * ncap;
-            int j = __ldg(nb + o1);
+            int j = entry(en_);
             if (!in_range(d, j, ncap, s, 4)) j = s;
             Qn = ld_state<FUSED>(pos + j);
             cp_async16<FUSED>(saddr(sl, 0), vel + j);
@@ -1107,8 +1133,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
             }
             asm volatile("cp.async.commit_group;\n" ::: "memory");
             asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-            const float4* sp = &stg[(sl * 2) * BS + tid];
-            const float4 Vb = sp[0], Wb = sp[BS];
+            const float4* sp = &stg[(sl * 2) * nthr + tid];
+            const float4 Vb = sp[0], Wb = sp[nthr];
             const int dx = min_image(P.x - Q.x, per0, ext0, hf0);
             const int dy = min_image(P.y - Q.y, per1, ext1, hf1);
             const int dz = P.z - Q.z;
@@ -1257,7 +1283,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         if (threadIdx.x == 0) {
             float bm = smax[0];
             for (int i = 1; i < WPB; ++i) bm = fmaxf(bm, smax[i]);
-            if (bm > 0.f && kprev >= 0) atomicMax(&d.id[kprev].stepmax, __float_as_uint(bm));
+            if (FUSED && d.B == 1) smax[0] = bm;
+            else if (bm > 0.f && kprev >= 0) atomicMax(&d.id[kprev].stepmax, __float_as_uint(bm));
         }
     }
     kstaged = kprev;
@@ -1293,6 +1320,25 @@ __device__ __forceinline__ void step_finish_instances(const Dev& d)
     }
 }
 
+// counters of the blocks that are done: a release of the block's earlier writes and an acquire of
+// the other blocks' (lighter than __threadfence, which is a sequentially consistent fence)
+__device__ __forceinline__ unsigned add_acq_rel(unsigned* p)
+{
+    unsigned v;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void add_release(unsigned* p)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // What a step kernel inside a graph does besides its step.  Step kernels of a graph are launched
 // in runs of several behind one conditional list build: a kernel that finds a list build pending,
 // or no step left to do, does nothing (the graph's loop at the end makes up for the steps left
@@ -1326,14 +1372,9 @@ __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int 
     step_pass<MODE, WALLS, BS, LPP>(d, prime, sc, sd, smax, kstaged);
     if (MODE == 0) {
         // the last block to finish accumulates the bound per instance and decides on rebuilds
-        if (threadIdx.x == 0) {
-            __threadfence();
-            const unsigned prev = atomicAdd(&d.g->counter, 1u);
-            am_last = prev == gridDim.x - 1;
-        }
+        if (threadIdx.x == 0) am_last = add_acq_rel(&d.g->counter) == gridDim.x - 1;
         __syncthreads();
         if (am_last) {
-            __threadfence();
             step_finish_instances(d);
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -1354,13 +1395,26 @@ __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int 
 // Several steps in one cooperative launch (every block resident at once; a block walks its
 // range of tiles each step, one tile per block when they all fit), for systems too small to hide
 // the per-step launch and graph-node latency.
-// Each step is exactly the step kernel's; between steps a grid barrier (the last block to
-// arrive ends the step for every instance, as the step kernel's last block does, then
-// releases the others; every wait gives up after a second and reports DEM_ERR_TIMEOUT, and a
-// block that gave up, or saw another give up, leaves the launch).  Runs the steps still to do
-// in this graph launch (g->remain) and stops early when an instance needs a list build; the
-// last block then sets the loop's conditions: h_rb (build the lists before going on) and
-// h_loop (steps remain).
+// Each step is exactly the step kernel's; between steps a grid barrier whose waits give up after a
+// second and report DEM_ERR_TIMEOUT (a block that gave up, or saw another give up, leaves the
+// launch).  Runs the steps still to do in this graph launch (g->remain) and stops early when an
+// instance needs a list build; the loop's conditions are set at the end: h_rb (build the lists
+// before going on) and h_loop (steps remain).
+// What bounds it is the chain of dependent round trips to L2 of one step, so:
+// - single instance: each block folds {step tag, its largest displacement} into one word and adds
+//   itself to a count; once the count is full every block reads the word, advances the
+//   displacement bound and decides on the list build alike.  (Tags grow, so nothing is reset; the
+//   words alternate by the tag's parity, as a block can be one step ahead, never two.)  With
+//   several instances the last block to arrive ends the step for each and releases the others.
+// - the barrier's cost is its fences and the arrivals at one word: one release and one acquire per
+//   block, by its first thread, and few blocks, one per SM.  A 1,440-sphere box on 96 blocks spent
+//   3,400 cycles of a step there, against 8,000 where each block wrote a word of its own and read
+//   all others', and 10,000 with fences by every warp; the 23,438-sphere silo on 736 blocks of 128
+//   threads 8,000 cycles, against 23,000.
+// - a block of one unit keeps its rows and row lengths in shared memory for the launch: they do not
+//   change between list builds, but the barrier's acquires empty the L1.
+// 200 steps of the 1,440-sphere box (8 lanes): 1265 against 1793 us with the counter's last arrival
+// ending the step, of the 23,438-sphere silo (4 lanes, walls) 2763 against 3100 us.
 constexpr unsigned long long BAR_WAIT_NS = 1000000000ull;   // a barrier wait gives up after 1 s
 constexpr unsigned BAR_POLLS = 1u << 24;                     // or after this many polls
 
@@ -1371,67 +1425,166 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+// a bounded wait of one thread until *p is past `target` (as a wrapping count)
+__device__ __forceinline__ bool wait_count(const unsigned* p, unsigned target)
+{
+    unsigned long long t0 = 0ull;
+    unsigned polls = 0u;
+    while ((int)(ld_acquire(p) - target) < 0) {
+        if ((++polls & 63u) == 0u) {
+            const unsigned long long t = global_ns();
+            if (t0 == 0ull) t0 = t;
+            if (polls > BAR_POLLS || t - t0 > BAR_WAIT_NS) return false;
+        }
+    }
+    return true;
+}
+
+// The barrier of a single instance at the step `tag`: folds in the block's largest displacement
+// smax[0] (written by its first thread, after the block's last barrier) and gives that of all blocks.
+// False: a wait gave up.
+__device__ __forceinline__ bool step_barrier(const Dev& d, unsigned tag, unsigned target, const float* smax, float& mx)
+{
+    __shared__ float s_mx;
+    __shared__ int s_ok;
+    if (threadIdx.x == 0) {
+        unsigned long long* f = d.bar + (size_t)(tag & 1u) * BAR_LINE;
+        unsigned* count = (unsigned*)(d.bar + 2 * BAR_LINE);
+        const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(smax[0]);
+        asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(f), "l"(w) : "memory");
+        add_release(count);
+        const bool ok = wait_count(count, target);
+        unsigned long long r;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(r) : "l"(f) : "memory");
+        s_mx = __uint_as_float((unsigned)r);
+        s_ok = ok ? 1 : 0;
+        if (!ok) atomicOr(&d.g->status, ST_TIMEOUT);
+    }
+    __syncthreads();
+    mx = s_mx;
+    return s_ok != 0;
+}
+
 template <bool WALLS, int LPP>
-__global__ void __launch_bounds__(TILE, 5) k_steps(Dev d, cudaGraphConditionalHandle h_rb,
+__global__ void __launch_bounds__(FUSED_T, 1) k_steps(Dev d, cudaGraphConditionalHandle h_rb,
                                                                         cudaGraphConditionalHandle h_loop)
 {
     __shared__ InstC sc;
     __shared__ InstD sd;
-    __shared__ float smax[TILE / 32];
+    __shared__ float smax[FUSED_T / 32];
     __shared__ bool am_last, quit;
-    // stop unless the block that ends the last step says otherwise (set before any block can
-    // reach the final barrier, so the later setting wins)
+    extern __shared__ float4 stg_dyn[];
+    const int nthr = (int)blockDim.x;
+    int* srows = (int*)(stg_dyn + 4 * nthr);
+    int* srcnt = srows + d.Lmax * row_stride(LPP, nthr);
+    // stop unless the end of the launch says otherwise (set before any block can reach the final
+    // barrier, so the later setting wins)
     if (blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h_loop, 0u);
     const long long todo = *(volatile long long*)&d.g->remain;
     long long done = 0;
-    bool final_last = false;
     int kstaged = -1;
+    const int* rows = nullptr;
+    {
+        // the rows of a block of at most one unit (the same split as the step pass)
+        constexpr int WPT = 4 * LPP, SPW = 32 / LPP;
+        const int wpb = nthr / 32, spb = nthr / LPP, stride = row_stride(LPP, nthr);
+        const int nlive = *(volatile int*)&d.g->nlive;
+        const int NV = nlive * WPT, NU = (NV + wpb - 1) / wpb;
+        const int u0 = (int)((long long)blockIdx.x * NU / gridDim.x);
+        const int u1 = (int)((long long)(blockIdx.x + 1) * NU / gridDim.x);
+        if (u1 - u0 == 1) {
+            for (int i = threadIdx.x; i < spb * LPP; i += nthr) {
+                const int ls = i % spb;
+                const int vw = u0 * wpb + ls / SPW;
+                if (vw >= NV) continue;
+                const int t = nlive == d.ntiles ? vw / WPT : d.live_tiles[vw / WPT];
+                const int s = t * TILE + (((vw & (WPT - 1)) + t) & (WPT - 1)) * SPW + ls % SPW;
+                const int k = d.tile_inst[t], lp = __ldcg(&d.id[k].lp);
+                const int cnt = s - d.ic[k].slot0 < __ldcg(&d.id[k].n) ? d.cnt[lp][s] : 0;
+                if (i < spb) srcnt[ls] = cnt;
+                for (int e = i / spb; e < cnt; e += LPP) srows[e * stride + ls] = __ldg(d.nbr[lp] + (size_t)e * d.ncap + s);
+            }
+            rows = srows;
+            __syncthreads();
+        }
+    }
+    // one call site of the step pass for both barriers: two inlined copies of it were contracted
+    // into multiply-adds differently, and fused steps have to give the step kernel's bits
+    const bool one = d.B == 1;
+    const unsigned base = *(volatile unsigned*)&d.g->bar_gen, count0 = *(volatile unsigned*)&d.g->bar_count;
+    const unsigned frozen = __ldcg(&d.g->frozen);
+    const float skin = d.ic[0].skin_f;
+    float disp = __ldcg(&d.id[0].disp);
+    bool rebuild = false, ok = true, last = false;
     while (done < todo) {
-        step_pass<0, WALLS, TILE, LPP, true>(d, 0, sc, sd, smax, kstaged);
+        step_pass<0, WALLS, TILE, LPP, true>(d, 0, sc, sd, smax, kstaged, rows, srcnt);
+        // a test of the timeout path (dem_test_stall_barrier): the first block does not arrive at
+        // the first barrier of this launch and leaves, so the others' waits run out
+        if (blockIdx.x == 0 && done == 0) {
+            if (threadIdx.x == 0) {
+                quit = atomicExch(&d.g->test_stall, 0u) != 0u;
+                if (quit) atomicOr(&d.g->status, ST_TIMEOUT);
+            }
+            __syncthreads();
+            if (quit) return;
+        }
+        if (one) {
+            float mx;
+            const unsigned i = (unsigned)done + 1u;
+            ok = step_barrier(d, base + i, count0 + i * gridDim.x, smax, mx);
+            if (!ok) break;
+            ++done;
+            disp += mx;
+            if (2.0f * disp >= 0.99f * skin) {
+                if (!frozen) {
+                    rebuild = true;
+                    break;
+                }
+                if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&d.g->status, ST_SKIN);
+            }
+            continue;
+        }
         if (threadIdx.x == 0) {
             const unsigned gen = *(volatile unsigned*)&d.g->bar_gen;
-            __threadfence();
-            // a test of the timeout path (dem_test_stall_barrier): the first block does not
-            // arrive at the first barrier of this launch and leaves, so the others' waits run out
-            const bool skip = blockIdx.x == 0 && done == 0 && atomicExch(&d.g->test_stall, 0u) != 0u;
-            const unsigned prev = skip ? 0u : atomicAdd(&d.g->counter, 1u);
-            am_last = !skip && prev == gridDim.x - 1;
-            if (skip) {
-                atomicOr(&d.g->status, ST_TIMEOUT);
-            } else if (!am_last) {
-                const unsigned long long t0 = global_ns();
-                unsigned polls = 0u;
-                while (*(volatile unsigned*)&d.g->bar_gen == gen) {
-                    if (++polls > BAR_POLLS || global_ns() - t0 > BAR_WAIT_NS) {
-                        atomicOr(&d.g->status, ST_TIMEOUT);
-                        break;
-                    }
-                    __nanosleep(256);
-                }
-                __threadfence();
-            }
+            am_last = add_acq_rel(&d.g->counter) == gridDim.x - 1;
+            if (!am_last && !wait_count(&d.g->bar_gen, gen + 1u)) atomicOr(&d.g->status, ST_TIMEOUT);
         }
         __syncthreads();
-        const bool last = am_last;
+        last = am_last;
         if (last) {
-            __threadfence();
             step_finish_instances(d);
             __syncthreads();
             if (threadIdx.x == 0) {
                 d.g->counter = 0u;
-                __threadfence();
-                atomicAdd(&d.g->bar_gen, 1u);      // release
+                add_release(&d.g->bar_gen);
             }
         }
         ++done;
-        final_last = last;
         if (threadIdx.x == 0)
             quit = *(volatile unsigned*)&d.g->any != 0u || (*(volatile unsigned*)&d.g->status & ST_TIMEOUT) != 0u;
         __syncthreads();
         if (quit) break;
     }
-    if (final_last && threadIdx.x == 0) {
-        const long long rem = todo - done;
+    if (threadIdx.x != 0) return;
+    const long long rem = todo - done;
+    if (one) {
+        // every block holds the same values and has read the record; the first writes them back
+        if (blockIdx.x != 0) return;
+        InstD* D = d.id;
+        if (done > 0) {
+            D->disp = disp;
+            D->cur ^= (int)(done & 1);
+            if (rebuild) {
+                D->flag = 1;
+                d.g->any = 1u;
+            }
+            d.g->bar_gen = base + (unsigned)done;
+            d.g->bar_count = count0 + (unsigned)done * gridDim.x;
+        }
+        d.g->remain = rem;
+        cudaGraphSetConditional(h_rb, rebuild ? 1u : 0u);
+        cudaGraphSetConditional(h_loop, rem > 0 && ok ? 1u : 0u);
+    } else if (last) {
         d.g->remain = rem;
         const bool timeout = (*(volatile unsigned*)&d.g->status & ST_TIMEOUT) != 0u;
         cudaGraphSetConditional(h_rb, *(volatile unsigned*)&d.g->any ? 1u : 0u);
@@ -2101,7 +2254,7 @@ struct Plan {
     unsigned ncodes = 0, nparts = 0;
     // offsets
     size_t o_pos[2], o_vel[2], o_omg[2], o_nbr[2], o_hist[2], o_cnt[2], o_hmask[2], o_fext[2], o_whist[2], o_wseg[2], o_wrem;
-    size_t o_cellcode, o_cslot, o_perm, o_fin, o_spos, o_sid, o_ccount, o_crange, o_part, o_pinst, o_soi, o_tile, o_live, o_ic, o_id, o_spread, o_g,
+    size_t o_cellcode, o_cslot, o_perm, o_fin, o_spos, o_sid, o_ccount, o_crange, o_part, o_pinst, o_soi, o_tile, o_live, o_bar, o_ic, o_id, o_spread, o_g,
         o_goff, o_outF, o_outT, o_outV, o_outW, o_outWX, o_xi, o_cmask, o_stage, o_hl, o_small, o_wgeo;
     size_t bytes = 0;
 };
@@ -2257,6 +2410,7 @@ dem_status make_plan(const dem_config* cfg, Plan& p, std::string& err)
     p.o_soi = L.take(N * 4);
     p.o_tile = L.take((size_t)p.ntiles * 4);
     p.o_live = L.take((size_t)p.ntiles * 4);
+    p.o_bar = L.take(sizeof(unsigned long long) * 3 * BAR_LINE);
     p.o_ic = L.take(sizeof(InstC) * p.B);
     p.o_id = L.take(sizeof(InstD) * p.B);
     p.o_spread = L.take(p.spread.size() * 4);
@@ -2533,8 +2687,9 @@ dem_status build_fused_graph(dem_ctx* ctx, cudaGraph_t g, int S)
         void* args[] = {&dv, &h_rb, &h_loop};
         cudaKernelNodeParams kp{};
         kp.func = fused_func(ctx);
-        kp.gridDim = dim3(std::min(ctx->ntiles * ctx->step_lanes, ctx->grid_fused));   // all resident: cooperative
-        kp.blockDim = dim3(TILE);
+        kp.gridDim = dim3(ctx->fused_blocks);      // all resident: cooperative
+        kp.blockDim = dim3(ctx->fused_threads);
+        kp.sharedMemBytes = fused_smem(ctx->step_lanes, ctx->fused_threads, ctx->Lmax);
         kp.kernelParams = args;
         CU(cudaGraphAddKernelNode(&kn, body, &ifn, 1, &kp));
         cudaLaunchAttributeValue coop{};
@@ -2597,9 +2752,28 @@ dem_status build_graph(dem_ctx* ctx, int S)
         // default when a block for every tile holding live slots fits on the GPU at once
         int nsm = 0, occ = 0;
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fused_func(ctx), TILE, 0);
-        cudaGetLastError();
+        cudaFuncSetAttribute(fused_func(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             fused_smem(1, FUSED_T, MAXL));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fused_func(ctx), TILE,
+                                                      fused_smem(ctx->step_lanes, TILE, ctx->Lmax));
         ctx->grid_fused = nsm * occ;
+        // blocks of 128 threads with several instances (a block stages one instance's constants);
+        // for one instance a block per SM, with the warps that spread the capacity's slices over
+        // the SMs (2 .. 20): the barrier between steps costs by the block
+        const int slices = ctx->ntiles * 4 * ctx->step_lanes;
+        ctx->fused_threads = TILE;
+        ctx->fused_blocks = std::min(ctx->ntiles * ctx->step_lanes, ctx->grid_fused);
+        if (ctx->B == 1 && ctx->grid_fused > 0) {
+            const int warps = std::min(FUSED_T / 32, std::max(2, (slices + nsm - 1) / nsm));
+            int wide = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wide, fused_func(ctx), 32 * warps,
+                                                          fused_smem(ctx->step_lanes, 32 * warps, ctx->Lmax));
+            if (wide > 0) {
+                ctx->fused_threads = 32 * warps;
+                ctx->fused_blocks = std::min(nsm, (slices + warps - 1) / warps);
+            }
+        }
+        cudaGetLastError();
         const bool can = (ctx->step_bs == 0 || ctx->step_bs == TILE) && ctx->grid_fused > 0;
         if (ctx->graph_mode == 2 && !can) return fail(ctx, DEM_ERR_STATE, "fused steps need 128-thread blocks");
         // the tiles holding live slots (from the host's last copy of the counts)
@@ -2609,7 +2783,6 @@ dem_status build_graph(dem_ctx* ctx, int S)
             return build_fused_graph(ctx, g, S);
     }
     // S steps in runs of EV_EVERY step kernels, each run behind one conditional list build, then a
-    // loop of (conditional list build, step kernel) for the steps that kernels left out because a
     // loop of (conditional list build, step kernel) for the steps that kernels left out because a
     // build became due within their run.  A condition per run instead of per step: the node costs
     // about 5 us between two kernels, and builds are hundreds of steps apart (100 steps of a
@@ -2814,6 +2987,7 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
     d.slot_of_id = (int*)(base + p.o_soi);
     d.tile_inst = (int*)(base + p.o_tile);
     d.live_tiles = (int*)(base + p.o_live);
+    d.bar = (unsigned long long*)(base + p.o_bar);
     d.ic = (const InstC*)(base + p.o_ic);
     d.id = (InstD*)(base + p.o_id);
     d.spread = (const unsigned*)(base + p.o_spread);
@@ -2867,6 +3041,7 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
     CUC(cudaMemcpyAsync(ctx->d_hl, p.hl.data(), sizeof(HostInstLo) * p.B, cudaMemcpyHostToDevice, s));
     CUC(cudaMemsetAsync(d.hist[0], 0, (size_t)p.ncap * p.Lmax * 12, s));
     CUC(cudaMemsetAsync(d.hist[1], 0, (size_t)p.ncap * p.Lmax * 12, s));
+    CUC(cudaMemsetAsync(d.bar, 0, sizeof(unsigned long long) * 3 * BAR_LINE, s));
     CUC(cudaMemsetAsync(d.wrem, 0, sizeof(double) * 2 * p.B, s));
     k_init_ids<<<nblk(p.ncap, 256), 256, 0, s>>>(d);
     CUC(cudaGetLastError());
@@ -3226,7 +3401,7 @@ dem_status dem_set_step_lanes(dem_ctx* ctx, int32_t lanes)
         long long live = 0;
         for (int k = 0; k < ctx->B; ++k) live += 2 * ((ctx->count[k] + 2 * TILE - 1) / (2 * TILE));
         int bf = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_steps<false, 2>, 128, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_steps<false, 2>, 128, fused_smem(2, 128, 1));
         cudaGetLastError();
         const long long gf = (long long)std::max(1, nsm) * std::max(1, bf);
         if (ctx->graph_mode != 1 && live <= gf) {

@@ -55,7 +55,8 @@ struct dem_ctx {
     int graph_steps = 0;
     int graph_mode = 0;               // 0: fused steps when the context fits, 1: a kernel per step, 2: fused
     bool graph_fused = false;         // the current graph runs its steps in fused cooperative launches
-    int grid_fused = 0;               // co-resident blocks of the fused step kernel (0: unknown)
+    int grid_fused = 0;               // co-resident 128-thread blocks of the fused step kernel (0: unknown)
+    int fused_threads = 0, fused_blocks = 0;   // its launch in the current graph
     cudaGraph_t rb_graph = nullptr;
     cudaGraph_t rb_if_graph = nullptr;   // the rebuild chain behind one condition, for calls that need valid
     cudaGraphExec_t rb_if = nullptr;     // lists (reads, coupling): a launch instead of the chain's eleven

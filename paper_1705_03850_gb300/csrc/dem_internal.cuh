@@ -35,6 +35,7 @@ constexpr int MAXL = 32;       // largest list width (one bit per entry in a 32-
 constexpr unsigned ID_MASK = 0x3fffffffu;   // particle ID (< 2^30)
 constexpr unsigned GONE_BIT = 0x40000000u;  // removed: dropped at the next list build
 constexpr unsigned WALL_BIT = 0x80000000u;  // in contact with the floor at the last step
+constexpr int BAR_LINE = 16;   // 64-bit words per line of the fused steps' barrier
 constexpr int MAX_WP = 8;      // points of an axisymmetric wall polyline
 
 // Axisymmetric walls: the offsets (a, b) = (rho, z) - nearest point of wall segment k of an
@@ -141,8 +142,9 @@ struct Glob {
     long long err_val;         // DEM_CHECKS builds: the index found out of range, and where
     int err_site;              // (1 cell code, 2 cell range of the list build; 3 touch pass,
     int err_pad;               //  4 contact pass of the step kernel)
-    unsigned bar_gen;          // fused steps: grid-barrier generation (bumped by each release)
-    unsigned bar_pad;
+    unsigned bar_gen;          // fused steps: grid-barrier generation (bumped by each release); with a single
+                               // instance the tag of the last step's maximum
+    unsigned bar_count;        // fused steps of a single instance: the barrier's arrivals so far
     long long remain;          // steps still to do in the current graph launch
     long long todo;            // steps of the next graph launch (0: as many as the graph was built for)
     int nlive;                 // entries of live_tiles
@@ -162,6 +164,8 @@ struct Dev {
     float4* fext[2];           // external force per particle (coupling controllers), list parity
     float4* whist[2];
     float4* wseg[2];           // [2][ncap] axisymmetric-wall contacts, list parity
+    unsigned long long* bar;   // fused steps of a single instance, a cache line each: {step tag, largest
+                               // displacement} by the tag's parity, and the count of arrivals
     double* wrem;              // [2 * B] particles and mass removed below the removal height
     unsigned* cellcode;
     unsigned* cslot;

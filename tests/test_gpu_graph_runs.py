@@ -40,3 +40,24 @@ def test_step_kernel_times_cover_the_steps_of_the_last_launch():
     sim.step(7)                                 # 7 of 20: the runs of steps 0-4 and 5-9
     ms, count = sim.graph_step_kernel_ms()
     assert count == 2 and 0 < ms < 100
+
+
+# one warp to several units per block: 30 and 512 slots (blocks of 64 threads), 12,000 and 40,000
+# (wide blocks; with 8 lanes more slices than the resident warps), and spare capacity
+@pytest.mark.parametrize("lanes", [1, 2, 4, 8])
+@pytest.mark.parametrize("shape,spare", [((5, 3, 2), 0), ((8, 8, 8), 5000), ((30, 20, 20), 0), ((40, 40, 25), 30000)])
+def test_fused_blocks_of_every_width_equal_one_launch_per_step(shape, spare, lanes):
+    wl = workloads.dense_block(*shape, seed=80, vel=0.4)
+    wl.skin = 0.02e-3
+    runs = []
+    for mode in (1, 2):
+        sim = dem.from_workload(wl, capacity=wl.n + spare, max_neighbors=20)
+        sim.set_step_lanes(lanes)
+        sim.set_graph_mode(mode)
+        sim.set_graph(40)
+        sim.step(121)
+        runs.append(sim)
+    a, b = runs
+    assert a.stats()["rebuilds"] == b.stats()["rebuilds"] > 2
+    for f in (dem.POS, dem.VEL, dem.OMEGA):
+        assert np.array_equal(a.read(f), b.read(f)), f
