@@ -42,10 +42,10 @@ def test_step_kernel_times_cover_the_steps_of_the_last_launch():
     assert count == 2 and 0 < ms < 100
 
 
-# one warp to several units per block: 30 and 512 slots (blocks of 64 threads), 12,000 and 40,000
+# one warp to several units per block: 40 and 512 slots (blocks of 64 threads), 12,000 and 40,000
 # (wide blocks; with 8 lanes more slices than the resident warps), and spare capacity
 @pytest.mark.parametrize("lanes", [1, 2, 4, 8])
-@pytest.mark.parametrize("shape,spare", [((5, 3, 2), 0), ((8, 8, 8), 5000), ((30, 20, 20), 0), ((40, 40, 25), 30000)])
+@pytest.mark.parametrize("shape,spare", [((5, 4, 2), 0), ((8, 8, 8), 5000), ((30, 20, 20), 0), ((40, 40, 25), 30000)])
 def test_fused_blocks_of_every_width_equal_one_launch_per_step(shape, spare, lanes):
     wl = workloads.dense_block(*shape, seed=80, vel=0.4)
     wl.skin = 0.02e-3
