@@ -679,6 +679,9 @@ __device__ __forceinline__ Coef<float> coef_of(const InstC& c)
 // MODE 0: one velocity-Verlet step (force at x^n with v^{n-1/2}, merged kick,
 // drift to x^{n+1}, displacement bound, rebuild decision by the last block).
 // MODE 1: forces at the current state only, written to the output arrays.
+// MODE 2: one step from a saved state to another (rollouts): Dev's buffers 0 hold the state before
+// the step and receive nothing, buffers 1 receive the state after it, with its overlaps and their
+// mask; lists come from the instance's parity.  No displacement bound, no end of step.
 //
 // Persistent grid: block b owns the contiguous tile range [b T / G, (b+1) T / G)
 // (neighbouring tiles share neighbours, which then hit in L1), one thread per
@@ -884,6 +887,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
     static_assert(!SMW || (LPP == 1 && !FUSED), "SM-wide blocks: one lane per particle, per-step launches");
     static_assert(LPP == 1 || LPP == 2 || LPP == 4 || LPP == 8, "1, 2, 4 or 8 lanes per particle");
     static_assert(LPP == 1 || MODE == 0, "several lanes per particle only for the step");
+    static_assert(MODE != 2 || (!WALLS && !FUSED), "rollouts have no walls and are not fused");
     static_assert((WPT & (WPT - 1)) == 0, "warps per tile must be a power of two");
     // entries of a lane's share of a row: bits e with e mod LPP == sub
     constexpr unsigned SUBBITS = LPP == 1 ? 0xffffffffu : LPP == 2 ? 0x55555555u : LPP == 4 ? 0x11111111u : 0x01010101u;
@@ -989,7 +993,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         const int t = all_live ? vw / WPT : d.live_tiles[vw / WPT];
         const int s = t * TILE + (((vw & (WPT - 1)) + t) & (WPT - 1)) * SPW + lane / LPP;
         if (s - c.slot0 >= sd.n) continue;
-        const int cur = sd.cur, lp = sd.lp;
+        const int cur = MODE == 2 ? 0 : sd.cur, lp = sd.lp;
+        const int hin = MODE == 2 ? 0 : lp, hout = MODE == 2 ? 1 : lp;   // overlaps, mask and floor overlap
         const int4* __restrict__ pos = d.pos[cur];
         const float4* __restrict__ vel = d.vel[cur];
         const float4* __restrict__ omg = d.omg[cur];
@@ -1012,13 +1017,13 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         auto entry = [&](int e) -> int {
             return FUSED && rows ? rows[e * rstride + ls] : __ldg(nb + (size_t)e * ncap);
         };
-        float* h = d.hist[lp] + s;
-        float* ho = MODE == 1 ? d.xi_out + s : h;
+        float* h = d.hist[hin] + s;
+        float* ho = MODE == 1 ? d.xi_out + s : MODE == 2 ? d.hist[hout] + s : h;
         const int per0 = c.per[0], per1 = c.per[1], ext0 = c.ext[0], ext1 = c.ext[1], hf0 = c.half[0],
                   hf1 = c.half[1];
 
         // ---- pass 1: positions of every entry, touch mask (independent loads)
-        const unsigned hm = d.hmask[lp][s];
+        const unsigned hm = d.hmask[hin][s];
         unsigned tm = 0u;
         // the first batch of indices is loaded before the row length arrives (rows hold at
         // least d.Lmax entries of storage); entries beyond the row are replaced by this slot
@@ -1032,7 +1037,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         jn3 = sub + 3 * LPP < ncnt ? jn3 : s;
         // removed below the removal height: parked until the next list build drops it (tested
         // here, after the row's first loads are in flight, so that live rows do not wait on it)
-        if (idw & GONE_BIT) {
+        if (MODE != 2 && (idw & GONE_BIT)) {
             if (MODE == 0 && sub == 0) {
                 d.pos[cur ^ 1][s] = P;
                 d.vel[cur ^ 1][s] = Vv;
@@ -1072,7 +1077,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         for (int o = 1; o < LPP; o <<= 1) tm |= __shfl_xor_sync(gmask, tm, o);
         // entries that left contact (or, for the read-out, every non-contact) get no history
         const unsigned rowmask = ncnt >= 32 ? 0xffffffffu : ((1u << ncnt) - 1u);
-        unsigned clr = (MODE == 1 ? rowmask : hm) & ~tm & submask;
+        unsigned clr = MODE == 2 ? 0u : (MODE == 1 ? rowmask : hm) & ~tm & submask;
         while (clr) {
             const int e = __ffs(clr) - 1;
             clr &= clr - 1u;
@@ -1171,7 +1176,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
             Tq.z += __shfl_xor_sync(gmask, Tq.z, o);
         }
         if (LPP > 1 && sub != 0) continue;      // the group's first lane finishes the particle
-        if (MODE == 0) d.hmask[lp][s] = cm;
+        if (MODE != 1) d.hmask[hout][s] = cm;
         if (sd.fext) {   // coupling controllers' force, held over the coupling interval
             const float4 fe = d.fext[lp][s];
             F = F + v3(fe.x, fe.y, fe.z);
@@ -1184,7 +1189,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
             if (dw > 0) {
                 wall_now = true;
                 if (wall_prev) {
-                    const float4 hw = d.whist[lp][s];
+                    const float4 hw = d.whist[hin][s];
                     wxi = v3(hw.x, hw.y, hw.z);
                 }
                 const V3 n = v3(0.f, 0.f, 1.f);
@@ -1195,7 +1200,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
                                                        v3(0.f, 0.f, 0.f), wxi, dt_hist, ft, slip);
                 F = F + fa;
                 Tq = Tq - r * cross(n, ft);
-                if (MODE == 0) d.whist[lp][s] = make_float4(wxi.x, wxi.y, wxi.z, 0.f);
+                if (MODE != 1) d.whist[hout][s] = make_float4(wxi.x, wxi.y, wxi.z, 0.f);
             }
         }
         int nseg = 0;
@@ -1249,14 +1254,14 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
                 const long long z = (long long)P.z + iz;
                 if (z > 2000000000ll || z < -2000000000ll) bad = true;
                 Pn = make_int4(x, y, (int)z, P.w);
-                runmax = fmaxf(runmax, sqrtf((float)ix * (float)ix + (float)iy * (float)iy + (float)iz * (float)iz));
+                if (MODE == 0) runmax = fmaxf(runmax, sqrtf((float)ix * (float)ix + (float)iy * (float)iy + (float)iz * (float)iz));
             }
             if (bad) {
                 atomicOr(&d.g->status, ST_ESCAPED);
                 d.g->err_slot = s;
             }
             unsigned gone = 0u;
-            if (Pn.z < c.zrem) {
+            if (MODE == 0 && Pn.z < c.zrem) {
                 // fell below the removal height: parked two cell heights lower with no radius
                 // (every live particle lies above the removal height, so none can touch it)
                 // and frozen until the next list build drops it; no rebuild is forced
@@ -1961,31 +1966,32 @@ __global__ void __launch_bounds__(TILE) k_snap(Dev d, Snap S)
     }
 }
 
-// F-bar, T-bar of this step from the velocity adjoints (and the drift)
-__global__ void __launch_bounds__(TILE) k_adj_prep(Dev d, AdjBufs a, float kick, int drift)
+// F-bar, T-bar of the evaluation at the last step from the seeds (no drift)
+__global__ void __launch_bounds__(TILE) k_adj_prep(Dev d, AdjBufs a, float kick)
 {
     for_live_slots(d, [&](int s, int k, const InstD& D) {
         const InstC& c = d.ic[k];
         const float dt = c.dt;
-        float4 vb = a.vb[s];
-        if (drift) {
-            const float4 xb = a.xb[s];
-            vb.x += dt * xb.x;
-            vb.y += dt * xb.y;
-            vb.z += dt * xb.z;
-            a.vb[s] = vb;
-        }
-        const float4 wb = a.wb[s];
+        const float4 vb = a.vb[s], wb = a.wb[s];
         const float m = d.omg[D.cur][s].w;
         const float r = (float)d.pos[D.cur][s].w * c.q;
         const float fk = kick * dt / m, tk = kick * dt / (0.4f * m * r * r);
-        a.Fb[s] = make_float4(fk * vb.x, fk * vb.y, fk * vb.z, 0.f);
-        a.Tb[s] = make_float4(tk * wb.x, tk * wb.y, tk * wb.z, 0.f);
+        a.Fb[0][s] = make_float4(fk * vb.x, fk * vb.y, fk * vb.z, 0.f);
+        a.Tb[0][s] = make_float4(tk * wb.x, tk * wb.y, tk * wb.z, 0.f);
     });
 }
 
-// pull the force adjoints back to x^n, v^{n-1/2}, w^{n-1/2}, xi^{n-1} and (E, e, mu)
-__global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, int prime)
+// Pulls the force adjoints (buffers par) back to x^n, v^{n-1/2}, w^{n-1/2}, xi^{n-1} and (E, e, mu),
+// then takes this particle one step further back (kick_next, its step's kick in dt): the drift and
+// the force adjoints of step n - 1 go to the other pair of buffers, so that the reverse step is one
+// kernel.  tmask: the contacts of x^n, which the forward step left in the mask of x^{n+1}
+// (nullptr: found from the positions, at the last step).
+// Bound by the latency of the gathers of a contact's four neighbour records and by registers (155:
+// three blocks of 128 an SM).  64 columns of 10,000 spheres, 100 steps forward and back: 37.4 ms
+// against 46.1 ms with a snapshot kernel before every recomputed step, a kernel of its own for the
+// force adjoints, a touch pass per reverse step and zeros written for every entry out of contact.
+__global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, const unsigned* __restrict__ tmask, int prime,
+                                                    int par, float kick_next)
 {
     const size_t plane = (size_t)d.Lmax * d.ncap;
     const int ncap = d.ncap;
@@ -2000,7 +2006,9 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, in
         const V3 vme = v3(Vv.x, Vv.y, Vv.z), wme = v3(Wv.x, Wv.y, Wv.z);
         const unsigned hm = S.hmask[s];
         const float dt_hist = prime ? 0.f : c.dt;
-        const float4 Fi = a.Fb[s], Ti = a.Tb[s];
+        const float4* Fb = a.Fb[par];
+        const float4* Tb = a.Tb[par];
+        const float4 Fi = Fb[s], Ti = Tb[s];
         float4 xb = a.xb[s], vb = a.vb[s], wb = a.wb[s];
         // the particle's share of d(loss)/d(E, e, mu) this step, summed over its few contacts in
         // float and added to the running double sums once (FP64 per contact is slow on this GPU)
@@ -2011,9 +2019,9 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, in
         const float* hs = S.hist + s;
         const int per0 = c.per[0], per1 = c.per[1], ext0 = c.ext[0], ext1 = c.ext[1], hf0 = c.half[0],
                   hf1 = c.half[1];
-        // pass 1: which entries touch (independent loads, four at a time)
-        unsigned tm = 0u;
-        for (int e0 = 0; e0 < ncnt; e0 += 4) {
+        // pass 1 (the last step only): which entries touch (independent loads, four at a time)
+        unsigned tm = tmask ? tmask[s] : 0u;
+        for (int e0 = tmask ? ncnt : 0; e0 < ncnt; e0 += 4) {
             int jb[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) jb[k] = e0 + k < ncnt ? __ldg(nb + (size_t)(e0 + k) * ncap) : s;
@@ -2028,14 +2036,7 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, in
                 if (e0 + k < ncnt && d2 < (long long)Sr * Sr) tm |= 1u << (e0 + k);
             }
         }
-        // the overlap adjoint of entries out of contact is zero
-        const unsigned rowmask = ncnt >= 32 ? 0xffffffffu : ((1u << ncnt) - 1u);
-        for (unsigned z = rowmask & ~tm; z; z &= z - 1u) {
-            const size_t o = (size_t)(__ffs(z) - 1) * ncap;
-            xbr[o] = 0.f;
-            xbr[plane + o] = 0.f;
-            xbr[2 * plane + o] = 0.f;
-        }
+        const unsigned xm = a.xmask[s];
         // pass 2: the contacts in row order
         for (unsigned rem = tm; rem; rem &= rem - 1u) {
             const int e = __ffs(rem) - 1;
@@ -2049,7 +2050,7 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, in
             const int Sr = P.w + Q.w;
             const long long S2 = (long long)Sr * Sr;
             const float4 Vj = S.vel[j], Wj = S.omg[j];
-            const float4 Fj = a.Fb[j], Tj = a.Tb[j];
+            const float4 Fj = Fb[j], Tj = Tb[j];
             const float d2f = (float)d2;
             const float inv = rsqrtf(d2f);
             const float dist = d2f * inv;
@@ -2059,7 +2060,7 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, in
             const V3 xio = ((hm >> e) & 1u) ? v3(hs[o], hs[plane + o], hs[2 * plane + o]) : v3(0.f, 0.f, 0.f);
             const V3 G = v3(Fi.x - Fj.x, Fi.y - Fj.y, Fi.z - Fj.z);
             const V3 H = v3(r * Ti.x + rj * Tj.x, r * Ti.y + rj * Tj.y, r * Ti.z + rj * Tj.z);
-            const V3 xibar = v3(xbr[o], xbr[plane + o], xbr[2 * plane + o]);
+            const V3 xibar = ((xm >> e) & 1u) ? v3(xbr[o], xbr[plane + o], xbr[2 * plane + o]) : v3(0.f, 0.f, 0.f);
             PairGrad<float> g;
             contact_vjp<float, false>(cf, delta, n, dist * q, r, rj, m, Wj.w, vme, v3(Vj.x, Vj.y, Vj.z), wme,
                                       v3(Wj.x, Wj.y, Wj.z), xio, dt_hist, G, H, xibar, g);
@@ -2098,8 +2099,17 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, in
         }
         a.wxib[s] = wx;
         a.xb[s] = xb;
-        a.vb[s] = vb;
         a.wb[s] = wb;
+        a.xmask[s] = tm;
+        // one step further back: the drift, then F-bar and T-bar (as k_adj_prep)
+        const float dt = c.dt;
+        vb.x += dt * xb.x;
+        vb.y += dt * xb.y;
+        vb.z += dt * xb.z;
+        a.vb[s] = vb;
+        const float fk = kick_next * dt / m, tk = kick_next * dt / (0.4f * m * r * r);
+        a.Fb[par ^ 1][s] = make_float4(fk * vb.x, fk * vb.y, fk * vb.z, 0.f);
+        a.Tb[par ^ 1][s] = make_float4(tk * wb.x, tk * wb.y, tk * wb.z, 0.f);
         a.thb[3 * (size_t)s] += (double)thE;
         a.thb[3 * (size_t)s + 1] += (double)the;
         a.thb[3 * (size_t)s + 2] += (double)thm;
@@ -2170,7 +2180,6 @@ __global__ void __launch_bounds__(256) k_obs(Dev d, const HostInstLo* __restrict
 // (small[16 k + 5..6] = weights), and zeroed history and parameter adjoints.
 __global__ void __launch_bounds__(TILE) k_adj_seed(Dev d, AdjBufs a, const HostInstLo* __restrict__ hl)
 {
-    const size_t plane = (size_t)d.Lmax * d.ncap;
     for_live_slots(d, [&](int s, int k, const InstD& D) {
         const double* sm = d.small + 16 * k;
         const float wke = (float)sm[5], wro = (float)sm[6];
@@ -2190,8 +2199,7 @@ __global__ void __launch_bounds__(TILE) k_adj_seed(Dev d, AdjBufs a, const HostI
         a.vb[s] = make_float4(wke * m * v.x, wke * m * v.y, wke * m * v.z, 0.f);
         a.wb[s] = make_float4(wke * I * w.x, wke * I * w.y, wke * I * w.z, 0.f);
         a.wxib[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int e = 0; e < d.Lmax; ++e)
-            for (int c3 = 0; c3 < 3; ++c3) a.xib[c3 * plane + (size_t)e * d.ncap + s] = 0.f;
+        a.xmask[s] = 0u;
         a.thb[3 * (size_t)s] = a.thb[3 * (size_t)s + 1] = a.thb[3 * (size_t)s + 2] = 0.0;
     });
 }
@@ -3088,6 +3096,8 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
         }
         ctx->grid1 = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * std::max(1, b1)));
         ctx->grid_rb = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * 8));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_adj_force, TILE, 0);
+        ctx->grid_adj = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * std::max(1, b1)));
         int bb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_build<false>, RB_T, 0);
         ctx->grid_build = std::max(1, std::min(ctx->ntiles * (TILE / RB_T), std::max(1, nsm) * std::max(1, bb)));
@@ -3499,7 +3509,7 @@ size_t rollout_layout(dem_ctx* ctx, long long nsteps, long long K, char* base)
 {
     Layout L;
     const int ncp = (int)((nsteps + K - 1) / K) + 1;
-    const int nseg = (int)std::min<long long>(K, nsteps);
+    const int nseg = (int)std::min<long long>(K, nsteps) - 1;   // a segment's first state is its checkpoint
     if (base) {
         ctx->ro.ck.assign(ncp, Snap{});
         ctx->ro.seg.assign(nseg, Snap{});
@@ -3508,14 +3518,18 @@ size_t rollout_layout(dem_ctx* ctx, long long nsteps, long long K, char* base)
     for (int i = 0; i < nseg; ++i) snap_layout(ctx, L, base ? &ctx->ro.seg[i] : nullptr, base);
     const size_t N = (size_t)ctx->ncap, Lm = (size_t)ctx->Lmax;
     size_t o_xb = L.take(N * 16), o_vb = L.take(N * 16), o_wb = L.take(N * 16), o_Fb = L.take(N * 16),
-           o_Tb = L.take(N * 16), o_xib = L.take(N * Lm * 12), o_wxib = L.take(N * 16), o_thb = L.take(N * 24);
+           o_Tb = L.take(N * 16), o_Fb1 = L.take(N * 16), o_Tb1 = L.take(N * 16), o_xib = L.take(N * Lm * 12),
+           o_xm = L.take(N * 4), o_wxib = L.take(N * 16), o_thb = L.take(N * 24);
     if (base) {
         AdjBufs& a = ctx->ro.a;
         a.xb = (float4*)(base + o_xb);
         a.vb = (float4*)(base + o_vb);
         a.wb = (float4*)(base + o_wb);
-        a.Fb = (float4*)(base + o_Fb);
-        a.Tb = (float4*)(base + o_Tb);
+        a.Fb[0] = (float4*)(base + o_Fb);
+        a.Tb[0] = (float4*)(base + o_Tb);
+        a.Fb[1] = (float4*)(base + o_Fb1);
+        a.Tb[1] = (float4*)(base + o_Tb1);
+        a.xmask = (unsigned*)(base + o_xm);
         a.xib = (float*)(base + o_xib);
         a.wxib = (float4*)(base + o_wxib);
         a.thb = (double*)(base + o_thb);
@@ -3541,6 +3555,24 @@ dem_status snap(dem_ctx* ctx, const Snap& S, bool save)
 dem_status step_once(dem_ctx* ctx, int prime)
 {
     if (dem_status st = launch_step(ctx, prime)) return st;   // rollouts refuse walls
+    CU(cudaGetLastError());
+    return DEM_OK;
+}
+
+// one step from the saved state A to B's buffers (lists frozen)
+dem_status step_between(dem_ctx* ctx, const Snap& A, const Snap& B, int prime)
+{
+    Dev d = ctx->dev;
+    const Snap* S[2] = {&A, &B};
+    for (int i = 0; i < 2; ++i) {
+        d.pos[i] = S[i]->pos;
+        d.vel[i] = S[i]->vel;
+        d.omg[i] = S[i]->omg;
+        d.hist[i] = S[i]->hist;
+        d.hmask[i] = S[i]->hmask;
+        d.whist[i] = S[i]->whist;
+    }
+    k_step<2, false><<<ctx->grid_bs[1], TILE, 0, ctx->stream>>>(d, prime, StepCtl{});
     CU(cudaGetLastError());
     return DEM_OK;
 }
@@ -3743,20 +3775,23 @@ dem_status dem_rollout_adjoint(dem_ctx* ctx, const double* weights, const double
     if ((st = set_frozen(ctx, 1u))) return st;
     const long long N = ro.nsteps, K = ro.K;
     // v^N = v^{N-1/2} + dt/2 F^N / m: the evaluation at N with a half kick and no drift
-    k_adj_prep<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, ro.a, 0.5f, 0);
-    k_adj_force<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, ro.a, ro.ck[ro.ncp - 1], 0);
+    auto prime_at = [&](long long t) { return t == 0 && ro.prime0; };
+    auto kick_at = [&](long long t) { return prime_at(t) ? 0.5f : 1.0f; };
+    int par = 0;
+    k_adj_prep<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, ro.a, 0.5f);
+    k_adj_force<<<ctx->grid_adj, TILE, 0, s>>>(ctx->dev, ro.a, ro.ck[ro.ncp - 1], nullptr, 0, par, kick_at(N - 1));
     CU(cudaGetLastError());
     for (int c = ro.ncp - 2; c >= 0; --c) {
         const long long s0 = (long long)c * K, s1 = std::min(s0 + K, N);
-        if ((st = snap(ctx, ro.ck[c], false))) return st;          // restore step s0
-        for (long long t = s0; t < s1; ++t) {                      // recompute the segment
-            if ((st = snap(ctx, ro.seg[t - s0], true))) return st;
-            if ((st = step_once(ctx, (t == 0 && ro.prime0) ? 1 : 0))) return st;
-        }
+        // the segment's states, recomputed from its checkpoint straight into their buffers (state t
+        // in at(t)); the last one's successor is the next checkpoint
+        auto at = [&](long long t) -> const Snap& { return t == s0 ? ro.ck[c] : t == s1 ? ro.ck[c + 1] : ro.seg[t - s0 - 1]; };
+        for (long long t = s0; t + 1 < s1; ++t)
+            if ((st = step_between(ctx, at(t), at(t + 1), prime_at(t) ? 1 : 0))) return st;
         for (long long t = s1 - 1; t >= s0; --t) {
-            const bool pr = t == 0 && ro.prime0;
-            k_adj_prep<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, ro.a, pr ? 0.5f : 1.0f, 1);
-            k_adj_force<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, ro.a, ro.seg[t - s0], pr ? 1 : 0);
+            par ^= 1;
+            k_adj_force<<<ctx->grid_adj, TILE, 0, s>>>(ctx->dev, ro.a, at(t), at(t + 1).hmask, prime_at(t) ? 1 : 0, par,
+                                                       t > 0 ? kick_at(t - 1) : 0.0f);
             CU(cudaGetLastError());
         }
     }

@@ -239,9 +239,10 @@ struct AdjBufs {
     float4* xb;        // adjoint of x^n [1/m units of the objective]
     float4* vb;        // adjoint of v^{n-1/2}
     float4* wb;        // adjoint of w^{n-1/2}
-    float4* Fb;        // adjoint of F^n
-    float4* Tb;        // adjoint of T^n
+    float4* Fb[2];     // adjoint of F^n, alternating by step (read by the neighbours while the
+    float4* Tb[2];     // next one is written); adjoint of T^n
     float* xib;        // adjoint of the stored overlaps, [3][Lmax][ncap], from each row's side
+    unsigned* xmask;   // bit e: entry e's overlap adjoint is non-zero (the others' are never read)
     float4* wxib;      // adjoint of the floor overlap
     double* thb;       // per slot: accumulated d/dE, d/de, d/dmu
 };
