@@ -217,6 +217,13 @@ __global__ void __launch_bounds__(TILE) k_rb_cellsort(Dev d)
     });
 }
 
+// The contact count that slots are ordered by: that of the last step, or for a build that only
+// orders a state that was just written (flag 3, order_slots) the contacts found by k_touch.
+__device__ __forceinline__ unsigned order_contacts(const Dev& d, const InstD& D, int old)
+{
+    return D.flag == 3 ? (unsigned)__popcll(d.cmask[old]) : (unsigned)__popc(d.hmask[D.lp][old]);
+}
+
 // Slots within each tile of TILE cell-order positions go to the particles in order
 // of decreasing contact count at the last step (then list length, then cell
 // order), so that the 32 rows a warp of the step kernel walks together have
@@ -242,7 +249,7 @@ __global__ void __launch_bounds__(TILE) k_rb_tilesort(Dev d)
             d.spos[p] = d.pos[D.cur][old];                    // cell-order copies for the list build
             d.sid[p] = (int)(__float_as_uint(d.vel[D.cur][old].w) & ID_MASK);
             if (D.flag != 2)
-                kk = ((unsigned)__popc(d.hmask[D.lp][old]) << 8) | (unsigned)min(d.cnt[D.lp][old], 255);
+                kk = (order_contacts(d, D, old) << 8) | (unsigned)min(d.cnt[D.lp][old], 255);
         }
         __syncthreads();                    // the previous tile's keys are no longer read
         key[threadIdx.x] = kk;
@@ -317,7 +324,7 @@ __global__ void __launch_bounds__(WS_T) k_rb_winsort(Dev d, int G)
                 d.sid[p] = (int)(__float_as_uint(d.vel[D.cur][old].w) & ID_MASK);
                 kk = 0;
                 if (D.flag != 2) {
-                    const int nc = min(__popc(d.hmask[D.lp][old]), MAXL), nl = min(d.cnt[D.lp][old], MAXL);
+                    const int nc = min((int)order_contacts(d, D, old), MAXL), nl = min(d.cnt[D.lp][old], MAXL);
                     kk = WS_KEYS - 1 - (nc * (MAXL + 1) + nl);    // more contacts, longer rows first
                 }
             }
@@ -630,11 +637,11 @@ __global__ void k_rb_finish(Dev d)
         if (D.flag) {
             D.cur ^= 1;
             D.lp ^= 1;
+            if (D.flag != 3) atomicAdd(&d.g->rebuilds, 1ull);
             D.flag = 0;
             D.n = D.n_new;
             D.nbin = D.n_new;
             D.disp = 0.f;
-            atomicAdd(&d.g->rebuilds, 1ull);
         }
     }
     __syncthreads();
@@ -862,6 +869,11 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void* src)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void cp_async4(unsigned dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
 }
 
 // One step over the block's units (MODE 0: force, kick and drift of every particle; MODE 1:
@@ -1915,6 +1927,19 @@ __device__ __forceinline__ void for_live_slots(const Dev& d, Fn fn)
     }
 }
 
+// the same by slices of 32 slots, for blocks of one warp
+template <typename Fn>
+__device__ __forceinline__ void for_live_slices(const Dev& d, Fn fn)
+{
+    for (int u = blockIdx.x; u < 4 * d.ntiles; u += gridDim.x) {
+        const int k = d.tile_inst[u >> 2];
+        const InstD D = d.id[k];
+        const int s = u * 32 + threadIdx.x;
+        if (s - d.ic[k].slot0 >= D.n) continue;
+        fn(s, k, D);
+    }
+}
+
 template <bool SAVE>
 __global__ void __launch_bounds__(TILE) k_snap(Dev d, Snap S)
 {
@@ -1966,6 +1991,39 @@ __global__ void __launch_bounds__(TILE) k_snap(Dev d, Snap S)
     }
 }
 
+// the contacts of the current positions, for ordering the slots (flag 3)
+__global__ void __launch_bounds__(TILE) k_touch(Dev d)
+{
+    for_live_slots(d, [&](int s, int k, const InstD& D) {
+        const InstC& c = d.ic[k];
+        const int4* __restrict__ pos = d.pos[D.cur];
+        const int* __restrict__ nb = d.nbr[D.lp] + s;
+        const int4 P = pos[s];
+        const int ncnt = d.cnt[D.lp][s], ncap = d.ncap;
+        unsigned tm = 0u;
+        for (int e0 = 0; e0 < ncnt; e0 += 4) {
+            int jb[4];
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4) jb[k4] = e0 + k4 < ncnt ? nb[(size_t)(e0 + k4) * ncap] : s;
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4) {
+                const int4 Q = pos[jb[k4]];
+                const long long dx = min_image(P.x - Q.x, c.per[0], c.ext[0], c.half[0]);
+                const long long dy = min_image(P.y - Q.y, c.per[1], c.ext[1], c.half[1]);
+                const long long dz = P.z - Q.z, S = P.w + Q.w;
+                if (e0 + k4 < ncnt && dx * dx + dy * dy + dz * dz < S * S) tm |= 1u << (e0 + k4);
+            }
+        }
+        d.cmask[s] = tm;
+    });
+}
+
+__global__ void k_mark_order(Dev d)
+{
+    for (int k = threadIdx.x; k < d.B; k += blockDim.x) d.id[k].flag = 3;
+    if (threadIdx.x == 0) d.g->any = 1u;
+}
+
 // F-bar, T-bar of the evaluation at the last step from the seeds (no drift)
 __global__ void __launch_bounds__(TILE) k_adj_prep(Dev d, AdjBufs a, float kick)
 {
@@ -1986,17 +2044,25 @@ __global__ void __launch_bounds__(TILE) k_adj_prep(Dev d, AdjBufs a, float kick)
 // the force adjoints of step n - 1 go to the other pair of buffers, so that the reverse step is one
 // kernel.  tmask: the contacts of x^n, which the forward step left in the mask of x^{n+1}
 // (nullptr: found from the positions, at the last step).
-// Bound by the latency of the gathers of a contact's four neighbour records and by registers (155:
-// three blocks of 128 an SM).  64 columns of 10,000 spheres, 100 steps forward and back: 37.4 ms
-// against 46.1 ms with a snapshot kernel before every recomputed step, a kernel of its own for the
-// force adjoints, a touch pass per reverse step and zeros written for every entry out of contact.
-__global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, const unsigned* __restrict__ tmask, int prime,
+// Bound by the latency of the gathers of a contact's five neighbour records: 154 registers leave 12
+// warps an SM.  So the next contact's records are copied asynchronously into shared memory while
+// one is evaluated, blocks are single warps (a 32-slot slice each, in the order of contact counts:
+// persistent blocks left the last of eight rounds nearly empty), and a rollout orders the slots by
+// contact count first (14 of 32 lanes were active without).  64 columns of 10,000 spheres, 100
+// steps forward and back: 31.3 ms against 37.4 ms without these (148 against about 180 us a reverse
+// step); 37.0 ms with the ordering alone, 32.1 ms at 128 registers (16 warps, 48 bytes spilled).
+__global__ void __launch_bounds__(32, 12) k_adj_force(Dev d, AdjBufs a, Snap S, const unsigned* __restrict__ tmask, int prime,
                                                     int par, float kick_next)
 {
     const size_t plane = (size_t)d.Lmax * d.ncap;
     const int ncap = d.ncap;
-    for_live_slots(d, [&](int s, int k, const InstD& D) {
+    // a block of one warp per 32-slot slice: the slices' contact counts differ, and what is resident
+    // is limited by registers, so blocks of one warp that come and go by themselves fill the SMs
+    for_live_slices(d, [&](int s, int k, const InstD& D) {
         const InstC& c = d.ic[k];
+        const int lane = (int)threadIdx.x;
+        __shared__ float4 stg[2][5][32];       // the next contact's position, velocity, spin, force adjoints,
+        __shared__ float stx[2][6][32];        // overlap and overlap adjoint
         const Coef<float> cf = coef_of(c);
         const int lp = D.lp;
         const float q = c.q;
@@ -2037,30 +2103,58 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, co
             }
         }
         const unsigned xm = a.xmask[s];
-        // pass 2: the contacts in row order
+        // pass 2: the contacts in row order, the next one's records copied to shared memory meanwhile
+        // (no registers held) and the index of the one after it loaded
+        auto issue = [&](int sl, int e, int j) {
+            auto sh = [](const void* p) -> unsigned { return (unsigned)__cvta_generic_to_shared(p); };
+            cp_async16<false>(sh(&stg[sl][0][lane]), S.pos + j);
+            cp_async16<false>(sh(&stg[sl][1][lane]), S.vel + j);
+            cp_async16<false>(sh(&stg[sl][2][lane]), S.omg + j);
+            cp_async16<false>(sh(&stg[sl][3][lane]), Fb + j);
+            cp_async16<false>(sh(&stg[sl][4][lane]), Tb + j);
+            const size_t o = (size_t)e * ncap;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                if ((hm >> e) & 1u) cp_async4(sh(&stx[sl][i][lane]), hs + o + i * plane);
+                if ((xm >> e) & 1u) cp_async4(sh(&stx[sl][3 + i][lane]), xbr + o + i * plane);
+            }
+        };
+        int sl = 0, jnext = s;
+        if (tm) {
+            const int e = __ffs(tm) - 1;
+            const unsigned r1 = tm & (tm - 1u);
+            const int j = __ldg(nb + (size_t)e * ncap);
+            if (r1) jnext = __ldg(nb + (size_t)(__ffs(r1) - 1) * ncap);
+            issue(0, e, j);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
         for (unsigned rem = tm; rem; rem &= rem - 1u) {
             const int e = __ffs(rem) - 1;
             const size_t o = (size_t)e * ncap;
-            const int j = __ldg(nb + o);
-            const int4 Q = __ldg(S.pos + j);
+            const unsigned r1 = rem & (rem - 1u), r2 = r1 & (r1 - 1u);
+            if (r1) issue(sl ^ 1, __ffs(r1) - 1, jnext);
+            if (r2) jnext = __ldg(nb + (size_t)(__ffs(r2) - 1) * ncap);
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+            const int4 Q = *reinterpret_cast<const int4*>(&stg[sl][0][lane]);
             const int dx = min_image(P.x - Q.x, per0, ext0, hf0);
             const int dy = min_image(P.y - Q.y, per1, ext1, hf1);
             const int dz = P.z - Q.z;
             const long long d2 = (long long)dx * dx + (long long)dy * dy + (long long)dz * dz;
             const int Sr = P.w + Q.w;
             const long long S2 = (long long)Sr * Sr;
-            const float4 Vj = S.vel[j], Wj = S.omg[j];
-            const float4 Fj = Fb[j], Tj = Tb[j];
+            const float4 Vj = stg[sl][1][lane], Wj = stg[sl][2][lane];
+            const float4 Fj = stg[sl][3][lane], Tj = stg[sl][4][lane];
             const float d2f = (float)d2;
             const float inv = rsqrtf(d2f);
             const float dist = d2f * inv;
             const float delta = __fdividef((float)(S2 - d2), (float)Sr + dist) * q;
             const V3 n = v3((float)dx * inv, (float)dy * inv, (float)dz * inv);
             const float rj = (float)Q.w * q;
-            const V3 xio = ((hm >> e) & 1u) ? v3(hs[o], hs[plane + o], hs[2 * plane + o]) : v3(0.f, 0.f, 0.f);
+            const V3 xio = ((hm >> e) & 1u) ? v3(stx[sl][0][lane], stx[sl][1][lane], stx[sl][2][lane]) : v3(0.f, 0.f, 0.f);
             const V3 G = v3(Fi.x - Fj.x, Fi.y - Fj.y, Fi.z - Fj.z);
             const V3 H = v3(r * Ti.x + rj * Tj.x, r * Ti.y + rj * Tj.y, r * Ti.z + rj * Tj.z);
-            const V3 xibar = ((xm >> e) & 1u) ? v3(xbr[o], xbr[plane + o], xbr[2 * plane + o]) : v3(0.f, 0.f, 0.f);
+            const V3 xibar = ((xm >> e) & 1u) ? v3(stx[sl][3][lane], stx[sl][4][lane], stx[sl][5][lane]) : v3(0.f, 0.f, 0.f);
             PairGrad<float> g;
             contact_vjp<float, false>(cf, delta, n, dist * q, r, rj, m, Wj.w, vme, v3(Vj.x, Vj.y, Vj.z), wme,
                                       v3(Wj.x, Wj.y, Wj.z), xio, dt_hist, G, H, xibar, g);
@@ -2074,6 +2168,7 @@ __global__ void __launch_bounds__(TILE) k_adj_force(Dev d, AdjBufs a, Snap S, co
             thE += 0.5f * (g.c_kn * c.c_kn + g.c_kt * c.c_kt) * c.inv_E;
             the += 0.5f * g.nbeta * c.dnb_de;
             thm += 0.5f * g.mu;
+            sl ^= 1;
         }
         float4 wx = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c.floor_on) {
@@ -2540,10 +2635,25 @@ dem_status ensure_lists(dem_ctx* ctx)
     } else {
         dem_status st = launch_rebuild(ctx, ctx->stream);
         if (st) return st;
+        if (ctx->must_build) ctx->written = true;
     }
     ctx->lists_ok = true;
     ctx->must_build = false;
     return DEM_OK;
+}
+
+// Orders the slots of a state that was just written by contact count: its list build could not,
+// knowing none, and the 32 rows of a warp are then of mixed lengths until the displacements call
+// for the next build (the reverse step of 40 columns ran 14 of 32 lanes).  A second build of the
+// same rows, for callers with enough steps ahead; results do not depend on the slots' order.
+dem_status order_slots(dem_ctx* ctx)
+{
+    if (!ctx->written) return DEM_OK;
+    ctx->written = false;
+    k_touch<<<ctx->grid_rb, TILE, 0, ctx->stream>>>(ctx->dev);
+    k_mark_order<<<1, 256, 0, ctx->stream>>>(ctx->dev);
+    CU(cudaGetLastError());
+    return launch_rebuild(ctx, ctx->stream);
 }
 
 dem_status launch_eval(dem_ctx* ctx)
@@ -2636,6 +2746,8 @@ dem_status launch_step(dem_ctx* ctx, int prime)
 }
 
 constexpr int EV_EVERY = 5;    // step kernels per run of a graph (one conditional list build, one of them timed)
+constexpr int ORDER_STEPS = 64;   // steps ahead from which a written state's slots are ordered first (order_slots)
+constexpr int ORDER_ROLLOUT = 6; // the same for a rollout, whose every step is walked three times
 constexpr int GRAPH_PART = 4;  // a graph also runs a remainder of at least 1/GRAPH_PART of its steps
 
 // the fused step kernel for the context's walls and lanes per particle
@@ -3096,8 +3208,6 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
         }
         ctx->grid1 = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * std::max(1, b1)));
         ctx->grid_rb = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * 8));
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_adj_force, TILE, 0);
-        ctx->grid_adj = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * std::max(1, b1)));
         int bb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_build<false>, RB_T, 0);
         ctx->grid_build = std::max(1, std::min(ctx->ntiles * (TILE / RB_T), std::max(1, nsm) * std::max(1, bb)));
@@ -3169,6 +3279,7 @@ dem_status dem_write(dem_ctx* ctx, int32_t field, const void* src, int64_t n)
         ctx->have_state = true;
         ctx->lists_ok = false;
         ctx->must_build = true;
+        ctx->written = false;
     }
     if (dsrc == ctx->dev.stage) CU(cudaStreamSynchronize(ctx->stream));
     return DEM_OK;
@@ -3270,8 +3381,10 @@ dem_status dem_step(dem_ctx* ctx, int64_t nsteps)
         }
         dem_status st = ensure_lists(ctx);
         if (st) return st;
+        if (left >= ORDER_STEPS && !ctx->graph_fused && (st = order_slots(ctx))) return st;
         st = launch_step(ctx, ctx->fresh ? 1 : 0);
         if (st) return st;
+        ctx->written = false;
         ctx->fresh = false;
         ctx->lists_ok = false;
         ++done;
@@ -3718,6 +3831,8 @@ dem_status dem_rollout_forward(dem_ctx* ctx, int64_t nsteps, int64_t checkpoint_
     ro.prime0 = ctx->fresh;
     dem_status st = ensure_lists(ctx);                      // the lists the whole rollout uses
     if (st) return st;
+    if (nsteps >= ORDER_ROLLOUT && (st = order_slots(ctx))) return st;
+    ctx->written = false;
     ctx->lists_ok = false;
     if ((st = set_frozen(ctx, 1u))) return st;
     for (long long s = 0; s < nsteps; ++s) {
@@ -3779,7 +3894,7 @@ dem_status dem_rollout_adjoint(dem_ctx* ctx, const double* weights, const double
     auto kick_at = [&](long long t) { return prime_at(t) ? 0.5f : 1.0f; };
     int par = 0;
     k_adj_prep<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, ro.a, 0.5f);
-    k_adj_force<<<ctx->grid_adj, TILE, 0, s>>>(ctx->dev, ro.a, ro.ck[ro.ncp - 1], nullptr, 0, par, kick_at(N - 1));
+    k_adj_force<<<4 * ctx->ntiles, 32, 0, s>>>(ctx->dev, ro.a, ro.ck[ro.ncp - 1], nullptr, 0, par, kick_at(N - 1));
     CU(cudaGetLastError());
     for (int c = ro.ncp - 2; c >= 0; --c) {
         const long long s0 = (long long)c * K, s1 = std::min(s0 + K, N);
@@ -3790,7 +3905,7 @@ dem_status dem_rollout_adjoint(dem_ctx* ctx, const double* weights, const double
             if ((st = step_between(ctx, at(t), at(t + 1), prime_at(t) ? 1 : 0))) return st;
         for (long long t = s1 - 1; t >= s0; --t) {
             par ^= 1;
-            k_adj_force<<<ctx->grid_adj, TILE, 0, s>>>(ctx->dev, ro.a, at(t), at(t + 1).hmask, prime_at(t) ? 1 : 0, par,
+            k_adj_force<<<4 * ctx->ntiles, 32, 0, s>>>(ctx->dev, ro.a, at(t), at(t + 1).hmask, prime_at(t) ? 1 : 0, par,
                                                        t > 0 ? kick_at(t - 1) : 0.0f);
             CU(cudaGetLastError());
         }

@@ -1440,6 +1440,7 @@ dem_status dem_couple(dem_coupler* cp)
     // no host wait: the device updated the count and the offsets (k_cp_append) and reports an
     // overflow in the status word; the host copy of the count is refreshed when next needed
     ctx->count_stale = true;
+    ctx->written = coarse->written = false;
     ctx->lists_ok = false;         // rows that did not fit fall back to a list build
     return DEM_OK;
 }

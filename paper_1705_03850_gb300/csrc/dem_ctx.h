@@ -33,7 +33,6 @@ struct dem_ctx {
     int grid_lanes[3] = {1, 1, 1};    // persistent step grids for 2, 4 and 8 lanes per particle
     bool list_staged = false;         // list build with the shared-memory window of cell-order positions
     int grid_build_staged = 1;
-    int grid_adj = 1;                 // one wave of the reverse step
     int grid_rb = 1;                  // persistent grid of the per-slot rebuild kernels
     int grid_build = 1;               // one wave of the list build (occupancy-sized)
     unsigned ncodes = 0, nparts = 0;
@@ -49,6 +48,7 @@ struct dem_ctx {
     // ran since the last one that could ask for one); must_build, one certainly is (a written state)
     bool lists_ok = false;
     bool must_build = true;
+    bool written = false;             // lists built for a written state, nothing but reads since
     long long steps = 0;
     unsigned status = 0;
     std::string err;

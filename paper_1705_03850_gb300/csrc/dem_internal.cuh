@@ -119,7 +119,7 @@ struct InstD {
     int n;               // live particles (slots slot0 .. slot0 + n - 1)
     int cur;             // state buffer holding the current step
     int lp;              // list buffer parity
-    int flag;            // 0 none, 1 rebuild pending, 2 rebuild with cleared history
+    int flag;            // 0 none, 1 rebuild pending, 2 rebuild with cleared history, 3 rebuild to order the slots
     float disp;          // accumulated per-step displacement bound since the last build [units]
     unsigned stepmax;    // this step's largest displacement (float bits)
     int nid;             // IDs handed out so far (n plus removed particles); IDs are never reused
