@@ -104,14 +104,30 @@ __global__ void __launch_bounds__(1024) k_scan_top(Dev d)
         if (threadIdx.x == 0) carry += tot;
         __syncthreads();
     }
+    // particles of every rebuilding instance after the build: those binned in its chunks (removed
+    // ones are not)
+    for (int k = threadIdx.x; k < d.B; k += blockDim.x) {
+        if (!d.id[k].flag) continue;
+        const InstC& c = d.ic[k];
+        const unsigned b0 = (unsigned)c.code0 / SCAN_TILE, b1 = b0 + ((unsigned)c.ncode + SCAN_TILE - 1) / SCAN_TILE;
+        d.id[k].n_new = (int)((b1 < d.nparts ? d.part[b1] : carry) - d.part[b0]);
+    }
 }
 
+// Also lists the cubes of CUBE codes that hold particles (the list build's units of work) and leaves
+// the counts zero for the next build.
+constexpr int CUBE = 64;       // 4 x 4 x 4 cells where each axis has at least four
 __global__ void __launch_bounds__(SCAN_T) k_scan_down(Dev d)
 {
     if (!d.g->any || !chunk_active(d, blockIdx.x)) return;
+    constexpr int TPC = CUBE / SCAN_V, NC = SCAN_TILE / CUBE;   // threads per cube, cubes per chunk
+    static_assert(32 % TPC == 0 && NC <= 32, "a cube within a warp, a chunk's cubes in one mask");
+    __shared__ unsigned held;
+    __shared__ int first;
     const unsigned base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
     unsigned v[SCAN_V];
     unsigned s = 0;
+    if (threadIdx.x == 0) held = 0u;
 #pragma unroll
     for (int k = 0; k < SCAN_V; ++k) {
         unsigned i = base + k;
@@ -120,12 +136,21 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_down(Dev d)
     }
     unsigned tot;
     unsigned ex = block_exclusive_scan(s, &tot) + d.part[blockIdx.x];
+    if (s) atomicOr(&held, 1u << (threadIdx.x / TPC));
 #pragma unroll
     for (int k = 0; k < SCAN_V; ++k) {
         unsigned i = base + k;
-        if (i < d.ncodes) d.crange[i] = make_uint2(ex, v[k]);
+        if (i < d.ncodes) {
+            d.crange[i] = make_uint2(ex, v[k]);
+            if (v[k]) d.ccount[i] = 0u;
+        }
         ex += v[k];
     }
+    __syncthreads();
+    if (threadIdx.x == 0) first = atomicAdd(&d.g->ncubes, __popc(held));
+    __syncthreads();
+    if (threadIdx.x < NC && ((held >> threadIdx.x) & 1u))
+        d.cubes[first + __popc(held & ((1u << threadIdx.x) - 1u))] = (int)(blockIdx.x * SCAN_TILE + threadIdx.x * CUBE);
 }
 
 // ==================================================================== cells
@@ -133,8 +158,8 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_down(Dev d)
 
 // ================================================================ rebuild
 // Triggered per instance by the displacement bound (flag != 0).  Sequence:
-// clear counts -> bin (atomic slot in cell) -> scan -> scatter -> order each
-// cell by particle ID -> count -> order the slots of each tile by contact count
+// bin (atomic slot in cell) -> scan -> scatter -> order each
+// cell by particle ID -> order the slots of each tile by contact count
 // (and copy positions and IDs in cell order) -> build lists, permute state,
 // carry histories -> finish.
 
@@ -151,16 +176,6 @@ __device__ __forceinline__ void for_rebuilding_slots(const Dev& d, Fn fn)
         const int s = t * TILE + threadIdx.x;
         if (s - c.slot0 >= D.n) continue;
         fn(s, D, c);
-    }
-}
-
-__global__ void k_rb_clear(Dev d)
-{
-    if (!d.g->any) return;
-    for (unsigned b = blockIdx.x; b < d.nparts; b += gridDim.x) {
-        if (!chunk_active(d, b)) continue;
-        for (unsigned i = b * SCAN_TILE + threadIdx.x; i < (b + 1) * SCAN_TILE && i < d.ncodes; i += blockDim.x)
-            d.ccount[i] = 0u;
     }
 }
 
@@ -200,7 +215,7 @@ __global__ void __launch_bounds__(TILE) k_rb_cellsort(Dev d)
     for_rebuilding_slots(d, [&](int s, const InstD& D, const InstC& c) {
         if (d.cslot[s] != 0u) return;   // not the first of its cell, or removed
         const unsigned code = d.cellcode[s];
-        const int cntc = (int)d.ccount[code];
+        const int cntc = (int)d.crange[code].y;
         if (cntc < 2) return;
         int* a = d.perm + c.slot0 + (int)(d.crange[code].x - d.crange[c.code0].x);
         const float4* v = d.vel[D.cur];
@@ -384,47 +399,401 @@ __global__ void __launch_bounds__(WS_T) k_rb_winsort(Dev d, int G)
     }
 }
 
-// One thread per particle: move it into its new slot of the other state buffer,
-// collect neighbours within r_i + r_j + skin (exact integer test), order the
-// row by overlap depth, and carry the tangential overlaps of pairs that were
-// already listed (found by ID in the particle's previous row).  The candidate
-// row is kept in shared memory, entry-major so that the threads of a warp hit
-// different banks.
-constexpr int RB_T = 64;                     // threads per block of the list build
+// One thread per particle: collect neighbours within r_i + r_j + skin (exact integer
+// test), order the row by overlap depth, move the particle into its new slot of the
+// other state buffer, and carry the tangential overlaps of pairs that were already
+// listed (found by ID in the particle's previous row).
 
-struct RowScratch {
-    float key[MAXL][RB_T];                   // d^2 - (r_i + r_j)^2 (rounded to float: monotone)
-    int pos[MAXL][RB_T];                     // partner's cell-order position
+// The particle `old` (cell-order position ps) with its list of nl <= N candidates, get(i, key, m):
+// key d^2 - (r_i + r_j)^2 (rounded to float: monotone) and cell-order position, the particle itself
+// among them or not.  The row goes out ordered by (key, ID) to the particle's new slot s, with the
+// state and the old row's overlaps.  The list is taken into registers: its places come from
+// comparing every two keys once, and the loads of all entries are in flight together (what this
+// costs otherwise is one chain of dependent loads per entry).
+template <int N, typename Get>
+__device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, const InstD& D, const InstC& c, int nl, bool overflow,
+                                        Get get)
+{
+    const int cur = D.cur, nxt = cur ^ 1, lp = D.lp, nlp = lp ^ 1;
+    const int ncap = d.ncap;
+    const bool fresh = D.flag == 2;          // a written state: no histories
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int ocnt = fresh ? 0 : d.cnt[lp][old];
+    unsigned ohm = fresh ? 0u : d.hmask[lp][old];
+    float key[N];
+    int m[N], r[N];
+    int nc = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        key[i] = INFINITY;                   // beyond the list, or the particle itself: after every neighbour
+        m[i] = ps;
+        r[i] = 0;
+        if (i < nl) {
+            get(i, key[i], m[i]);
+            if (m[i] == ps) key[i] = INFINITY;
+            else ++nc;
+        }
+    }
+    bool tie = false;
+#pragma unroll
+    for (int i = 1; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            const bool before = key[j] <= key[i];
+            r[i] += before ? 1 : 0;
+            r[j] += before ? 0 : 1;
+            tie |= key[j] == key[i] && key[i] < INFINITY;
+        }
+    // the new row (partner slots); the positions give way to the partner IDs
+    int* nrow = d.nbr[nlp] + s;
+    int id[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) id[i] = m[i] != ps ? d.sid[m[i]] : -2;
+    if (tie) {
+        // equal keys (rare) by ID, so that the row does not depend on the scan order
+#pragma unroll 1
+        for (int i = 1; i < N; ++i)
+#pragma unroll 1
+            for (int j = 0; j < i; ++j) {
+                float ki = 0.f, kj = 1.f;
+                int di = 0, dj = 0;
+#pragma unroll
+                for (int q = 0; q < N; ++q) {
+                    if (q == i) { ki = key[q]; di = id[q]; }
+                    if (q == j) { kj = key[q]; dj = id[q]; }
+                }
+                if (ki == kj && ki < INFINITY && dj > di) {   // counted the other way round above
+#pragma unroll
+                    for (int q = 0; q < N; ++q) {
+                        if (q == i) --r[q];
+                        if (q == j) ++r[q];
+                    }
+                }
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (m[i] != ps) nrow[(size_t)r[i] * ncap] = d.fin[m[i]];
+    if (overflow) {
+        atomicOr(&d.g->status, ST_CAPACITY);
+        d.g->err_slot = s;
+    }
+    // carry every non-zero stored overlap of the old row to the pair's new entry, four at a time.
+    // Overlaps are written only where carried: every reader of an entry's overlap first checks its
+    // bit in the history mask, so the other entries' storage is never read
+    const int* orow = d.nbr[lp] + old;
+    const float* ho = d.hist[lp] + old;
+    float* hn = d.hist[nlp] + s;
+    const size_t plane = (size_t)d.Lmax * ncap;
+    if (ocnt < 32) ohm &= (1u << ocnt) - 1u;
+    unsigned nhm = 0u;
+    while (ohm) {
+        int eo[4], oid[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            eo[k] = ohm ? __ffs(ohm) - 1 : -1;
+            ohm &= ohm - 1u;                 // stays zero once it is
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) oid[k] = eo[k] >= 0 ? orow[(size_t)eo[k] * ncap] : old;
+        float h[4][3];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const size_t o = (size_t)max(eo[k], 0) * ncap;
+            h[k][0] = eo[k] >= 0 ? ho[o] : 0.f;
+            h[k][1] = eo[k] >= 0 ? ho[plane + o] : 0.f;
+            h[k][2] = eo[k] >= 0 ? ho[2 * plane + o] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) oid[k] = (int)(__float_as_uint(d.vel[cur][oid[k]].w) & ID_MASK);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (h[k][0] == 0.f && h[k][1] == 0.f && h[k][2] == 0.f) continue;   // nothing to carry
+            int re = -1;
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                if (id[i] == oid[k]) re = r[i];
+            if (re >= 0) {
+                float* x = hn + (size_t)re * ncap;
+                x[0] = h[k][0];
+                x[plane] = h[k][1];
+                x[2 * plane] = h[k][2];
+                nhm |= 1u << re;
+            }
+        }
+    }
+    float4 v = d.vel[cur][old];
+    const int4 p = d.pos[cur][old];
+    const float4 w = d.omg[cur][old];
+    const float4 wh = fresh ? z4 : d.whist[lp][old];
+    const unsigned myid = __float_as_uint(v.w) & ID_MASK;
+    if (fresh) v.w = __uint_as_float(myid);  // no floor history
+    d.pos[nxt][s] = p;
+    d.vel[nxt][s] = v;
+    d.omg[nxt][s] = w;
+    d.slot_of_id[c.slot0 + (int)myid] = s;
+    d.cnt[nlp][s] = nc;
+    d.hmask[nlp][s] = nhm;
+    if (D.fext) d.fext[nlp][s] = d.fext[lp][old];      // held until overwritten, even across state writes
+    d.whist[nlp][s] = wh;
+    if (c.nwp >= 2) {
+        d.wseg[nlp][s] = fresh ? z4 : d.wseg[lp][old];
+        d.wseg[nlp][ncap + s] = fresh ? z4 : d.wseg[lp][ncap + old];
+    }
+}
+
+// The default list build: one block per cube of CUBE consecutive Morton codes (4 x 4 x 4 cells)
+// that holds particles.  The block copies the positions of the cube's cells and of the layer of
+// cells around them (6 x 6 x 6) into shared memory, x fastest, shifted to the image next to the
+// cube, so that the three cells of a row along x are one run: a particle scans nine runs there,
+// without image arithmetic, cell lookups or trips to L2.  The copy goes by windows of CB_CAP
+// positions, so that any occupancy fits; at ordinary densities (370 to 530 positions for 110 to
+// 155 particles) one window holds them all.  The distance test needs no check of the axes first:
+// in unsigned 64 bits three squares of 32-bit differences cannot overflow.
+// Bound by latency: of the 40,000 cycles a block spends on a cube of the 1M bed, half go to the
+// scan (16-byte shared loads at random, four candidates at a time) and a third to the row's way out.
+// One list build of a 1M bed adds 390 us to a step, of a 100,000-sphere bed 55 us, against 575 and
+// 78 us with a thread looking up and scanning its 27 cells in global memory; blocks of 192 threads
+// and 4 to 7 resident blocks of 128 came within 5 % of this.
+constexpr int CB_T = 128;                    // threads per block
+constexpr int CB_CAP = 640;                  // positions per window
+constexpr int CB_H = 600;                    // cells of a cube and around it: 216, at most 66 x 3 x 3
+constexpr int CB_OWN = 384;                  // particles of the cube whose cell is noted (the others' is computed)
+struct CubeScratch {
+    int4 pos[CB_CAP];
+    int m[CB_CAP];                           // their cell-order positions
+    unsigned char shift[CB_CAP];             // images: bits 0-1 x, 2-3 y (0 none, 1 from below, 2 from above)
+    unsigned short own[CB_OWN];              // the cell (as h) of the cube's particles
+    int off[CB_H + 1];                       // cell h's first position in the copied order
+    int wsum[CB_T / 32];
 };
+__host__ __device__ constexpr size_t cube_smem(int lmax) { return (size_t)(lmax + 1) * CB_T * 4; }
 
-// The staged variant of the list build: the block's 64 cell-order positions and RB_W on either
-// side (the cells around the block's particles, in Morton order) staged in shared memory;
-// candidates inside the window are read from there, the others from L2.
+__global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
+{
+    if (!d.g->any) return;
+    __shared__ CubeScratch C;
+    extern __shared__ int cube_rows[];       // candidates [Lmax + 1][CB_T]: the particle itself is among them
+    const int tx = threadIdx.x, lane = tx & 31, warp = tx >> 5;
+    const int Lmax = d.Lmax;
+    int* row = cube_rows + tx;
+    const int ncubes = d.g->ncubes;
+    for (int i = blockIdx.x; i < ncubes; i += gridDim.x) {
+        const int code = d.cubes[i];
+        const int k = d.B == 1 ? 0 : d.part_inst[code / SCAN_TILE];
+        const InstD D = d.id[k];
+        const InstC& c = d.ic[k];
+        const unsigned cbase = d.crange[c.code0].x;
+        const int last = min(code + CUBE, c.code0 + c.ncode) - 1;
+        const uint2 rl = d.crange[last];
+        const int first = (int)d.crange[code].x;
+        const int p0 = c.slot0 + first - (int)cbase, n = (int)(rl.x + rl.y) - first;
+        // the cube's first cell, from any of its particles
+        const int4 pf = d.spos[p0];
+        const int lgx = D.cube_lg & 15, lgy = (D.cube_lg >> 4) & 15, lgz = (D.cube_lg >> 8) & 15;
+        const int bx = axis_cell(c, 0, pf.x) >> lgx << lgx, by = axis_cell(c, 1, pf.y) >> lgy << lgy,
+                  bz = axis_cell(c, 2, pf.z) >> lgz << lgz;
+        const int HX = (1 << lgx) + 2, HY = (1 << lgy) + 2, HZ = (1 << lgz) + 2;
+        const int H = HX * HY * HZ;
+        __syncthreads();                     // the previous cube is done with the shared arrays
+        // the cells, each thread a run of them: starts, counts and images, then their offsets
+        constexpr int CHM = (CB_H + CB_T - 1) / CB_T;
+        const int CH = (H + CB_T - 1) / CB_T;
+        int cst[CHM], ccn[CHM], csh[CHM];
+        int sum = 0;
+#pragma unroll
+        for (int q = 0; q < CHM; ++q) {
+            const int h = tx * CH + q;
+            cst[q] = ccn[q] = csh[q] = 0;
+            if (q < CH && h < H) {
+                const int hx = h % HX, hy = (h / HX) % HY, hz = h / (HX * HY);
+                int cx = bx - 1 + hx, cy = by - 1 + hy;
+                const int cz = bz - 1 + hz;
+                int sh = 0;
+                if (c.per[0]) {
+                    if (cx < 0) { cx += c.nc[0]; sh |= 1; }
+                    else if (cx == c.nc[0]) { cx = 0; sh |= 2; }
+                }
+                if (c.per[1]) {
+                    if (cy < 0) { cy += c.nc[1]; sh |= 4; }
+                    else if (cy == c.nc[1]) { cy = 0; sh |= 8; }
+                }
+                if (cx >= 0 && cx < c.nc[0] && cy >= 0 && cy < c.nc[1] && cz >= 0 && cz < c.nc[2]) {
+                    const unsigned cd = cell_code(d, c, cx, cy, cz);
+                    bool ok = true;
+#if DEM_CHECKS
+                    ok = in_range(d, (long long)cd - c.code0, c.ncode, p0, 1);
+#endif
+                    if (ok) {
+                        const uint2 r = d.crange[cd];
+                        cst[q] = c.slot0 + (int)(r.x - cbase);
+                        ccn[q] = (int)r.y;
+                        csh[q] = sh;
+#if DEM_CHECKS
+                        if (ccn[q] > 0 && !(in_range(d, cst[q] - c.slot0, c.cap, p0, 2) &&
+                                            in_range(d, cst[q] - c.slot0 + ccn[q], c.cap + 1, p0, 2)))
+                            ccn[q] = 0;
+#endif
+                        // a cell of the cube itself (not an image of one): its particles' cell
+                        if (sh == 0 && hx >= 1 && hx < HX - 1 && hy >= 1 && hy < HY - 1 && hz >= 1 && hz < HZ - 1)
+                            for (int t = 0; t < ccn[q]; ++t)
+                                if (cst[q] - p0 + t < CB_OWN) C.own[cst[q] - p0 + t] = (unsigned short)h;
+                    }
+                }
+                sum += ccn[q];
+            }
+        }
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) C.wsum[warp] = inc;
+        __syncthreads();
+        int off0 = inc - sum, total = 0;
+        for (int w = 0; w < CB_T / 32; ++w) {
+            if (w < warp) off0 += C.wsum[w];
+            total += C.wsum[w];
+        }
+        {
+            int off = off0;
+#pragma unroll
+            for (int q = 0; q < CHM; ++q) {
+                const int h = tx * CH + q;
+                if (q < CH && h < H) C.off[h] = off;
+                off += ccn[q];
+            }
+            if (tx == 0) C.off[H] = total;
+        }
+        // the cube's particles, CB_T at a time
+        for (int g0 = 0; g0 < n; g0 += CB_T) {
+            const bool mine = g0 + tx < n;
+            const int ps = p0 + g0 + tx;
+            int old = 0, s = 0, nl = 0, h0 = 0;
+            int4 p = make_int4(0, 0, 0, 0);
+            if (mine) {
+                p = d.spos[ps];
+                old = d.perm[ps];
+                s = d.fin[ps];
+            }
+            for (int w0 = 0; w0 < total; w0 += CB_CAP) {
+                const int w1 = min(total, w0 + CB_CAP);
+                if (w0 > 0 || g0 > 0) __syncthreads();   // the previous window is done with
+                if (g0 == 0 || total > CB_CAP) {
+                    // where each position of the window comes from, then the positions, coalesced
+                    int o = off0;
+#pragma unroll
+                    for (int q = 0; q < CHM; ++q) {
+                        for (int t = max(0, w0 - o); t < min(ccn[q], w1 - o); ++t) {
+                            C.m[o + t - w0] = cst[q] + t;
+                            C.shift[o + t - w0] = (unsigned char)csh[q];
+                        }
+                        o += ccn[q];
+                    }
+                    __syncthreads();
+                    for (int t = tx; t < w1 - w0; t += CB_T) {
+                        int4 q = __ldg(d.spos + C.m[t]);
+                        const int sh = C.shift[t];
+                        if (sh & 3) q.x += (sh & 1) ? -c.ext[0] : c.ext[0];
+                        if (sh & 12) q.y += (sh & 4) ? -c.ext[1] : c.ext[1];
+                        C.pos[t] = q;
+                    }
+                }
+                __syncthreads();
+                if (!mine) continue;
+                if (w0 == 0) {
+                    // the run of cells that starts one below the particle's on every axis
+                    if (ps - p0 < CB_OWN)
+                        h0 = (int)C.own[ps - p0] - (HY + 1) * HX - 1;
+                    else
+                        h0 = ((axis_cell(c, 2, p.z) - bz) * HY + axis_cell(c, 1, p.y) - by) * HX + axis_cell(c, 0, p.x) - bx;
+                }
+                const int cut0 = p.w + c.skin;
+                const int before = nl;
+#pragma unroll 1
+                for (int r = 0; r < 9; ++r) {
+                    const int h = h0 + (r / 3 * HY + r % 3) * HX;
+                    const int t1 = min(C.off[h + 3], w1) - w0;
+                    // four at a time, without branches: the loop waits for its loads and products
+                    for (int t = max(C.off[h], w0) - w0; t < t1; t += 4) {
+                        int4 q[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) q[u] = C.pos[min(t + u, t1 - 1)];
+                        bool hit[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int dx = p.x - q[u].x, dy = p.y - q[u].y, dz = p.z - q[u].z;
+                            const int cut = cut0 + q[u].w;
+                            const unsigned long long d2 = (unsigned long long)((long long)dx * dx) +
+                                                          (unsigned long long)((long long)dy * dy) +
+                                                          (unsigned long long)((long long)dz * dz);
+                            hit[u] = t + u < t1 && d2 < (unsigned long long)((long long)cut * cut);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (hit[u]) {
+                                if (nl <= Lmax) row[nl * CB_T] = t + u;
+                                ++nl;
+                            }
+                    }
+                }
+                if (total > CB_CAP)          // the next window takes this one's place
+                    for (int e = before; e < min(nl, Lmax + 1); ++e) row[e * CB_T] = C.m[row[e * CB_T]];
+            }
+            const int most = __reduce_max_sync(0xffffffffu, nl);
+            if (!mine) continue;
+            const bool overflow = nl > Lmax + 1;
+            nl = min(nl, Lmax + 1);
+            auto get = [&](int e, float& key, int& m) {
+                const int t = row[e * CB_T];
+                int4 q;
+                long long dx, dy;
+                if (total > CB_CAP) {
+                    m = t;
+                    q = __ldg(d.spos + m);
+                    dx = min_image(p.x - q.x, c.per[0], c.ext[0], c.half[0]);
+                    dy = min_image(p.y - q.y, c.per[1], c.ext[1], c.half[1]);
+                } else {
+                    m = C.m[t];
+                    q = C.pos[t];
+                    dx = p.x - q.x;
+                    dy = p.y - q.y;
+                }
+                const long long dz = (long long)p.z - q.z, S = (long long)p.w + q.w;
+                key = (float)(dx * dx + dy * dy + dz * dz - S * S);
+            };
+            if (most <= 9) row_out<9>(d, s, old, ps, D, c, nl, overflow, get);
+            else if (most <= 13) row_out<13>(d, s, old, ps, D, c, nl, overflow, get);
+            else if (most <= 17) row_out<17>(d, s, old, ps, D, c, nl, overflow, get);
+            else row_out<MAXL + 1>(d, s, old, ps, D, c, nl, overflow, get);
+        }
+    }
+}
+
+// The other list build (dem_set_list_build): one block per 64 cell-order positions, with RB_W on
+// either side (the cells around the block's particles, in Morton order) staged in shared memory;
+// each thread looks up and scans its 27 cells, candidates inside the window are read from there,
+// the others from L2.
+constexpr int RB_T = 64;                     // threads per block
 constexpr int RB_W = 128;
 constexpr int RB_WIN = RB_T + 2 * RB_W;
 struct Window {
     int4 pos[RB_WIN];
     int lo, n;                               // first cell-order position and length
 };
+struct RowScratch {
+    float key[MAXL][RB_T];
+    int pos[MAXL][RB_T];
+};
 
-template <bool STAGED>
 __device__ __forceinline__ void build_row(const Dev& d, int ps, const InstD& D, const InstC& c, RowScratch& R,
-                                          const Window* W)
+                                          const Window& W)
 {
     const int tx = threadIdx.x;
-    const int cur = D.cur, nxt = cur ^ 1, lp = D.lp, nlp = lp ^ 1;
-    const int ncap = d.ncap;
-    const int s = d.fin[ps];                // this particle's new slot
     const int old = d.perm[ps];
-    const int4 p = d.pos[cur][old];
-    float4 v = d.vel[cur][old];
-    const float4 w = d.omg[cur][old];
-    const unsigned myid = __float_as_uint(v.w) & ID_MASK;
-    if (D.flag == 2) v.w = __uint_as_float(myid);   // fresh start: no floor history
-    d.pos[nxt][s] = p;
-    d.vel[nxt][s] = v;
-    d.omg[nxt][s] = w;
-    d.slot_of_id[c.slot0 + (int)myid] = s;
+    const int s = d.fin[ps];
+    const int4 p = d.spos[ps];
 
     // candidates ordered by (d^2 - (r_i + r_j)^2, ID): deepest overlaps first, so
     // that within a warp the contacts sit in the leading entries of every row
@@ -492,13 +861,8 @@ __device__ __forceinline__ void build_row(const Dev& d, int ps, const InstD& D, 
 #endif
         for (int t = 0; t < cnt; ++t) {
             const int m = start + t;
-            int4 q;
-            if (STAGED) {
-                const unsigned wi = (unsigned)(m - W->lo);
-                q = wi < (unsigned)W->n ? W->pos[wi] : __ldg(d.spos + m);
-            } else {
-                q = __ldg(d.spos + m);
-            }
+            const unsigned wi = (unsigned)(m - W.lo);
+            const int4 q = wi < (unsigned)W.n ? W.pos[wi] : __ldg(d.spos + m);
             const int ddx = min_image(p.x - q.x, per0, ext0, hf0);
             const int ddy = min_image(p.y - q.y, per1, ext1, hf1);
             const long long ddz = (long long)p.z - q.z;
@@ -517,79 +881,24 @@ __device__ __forceinline__ void build_row(const Dev& d, int ps, const InstD& D, 
             ++nc;
         }
     }
-    // order the row by (key, ID): equal keys (rare) by ID, so that the row does not
-    // depend on the scan order
-    for (int i = 1; i < nc; ++i) {
-        const float key = R.key[i][tx];
-        const int m = R.pos[i][tx];
-        int j = i - 1;
-        while (j >= 0 && (R.key[j][tx] > key || (R.key[j][tx] == key && d.sid[R.pos[j][tx]] > d.sid[m]))) {
-            R.key[j + 1][tx] = R.key[j][tx];
-            R.pos[j + 1][tx] = R.pos[j][tx];
-            --j;
-        }
-        R.key[j + 1][tx] = key;
-        R.pos[j + 1][tx] = m;
-    }
-    if (overflow) {
-        atomicOr(&d.g->status, ST_CAPACITY);
-        d.g->err_slot = s;
-    }
-    int* nrow = d.nbr[nlp] + s;
-    float* hn = d.hist[nlp] + s;
-    const size_t plane = (size_t)Lmax * ncap;
-    const int* orow = d.nbr[lp] + old;
-    const float* ho = d.hist[lp] + old;
-    // the new row (partner slots); the keys give way to the partner IDs.  Stored overlaps are
-    // written only where carried: every reader of an entry's overlap first checks its bit in the
-    // history mask, so the other entries' storage is never read
-    for (int e = 0; e < nc; ++e) {
-        const int m = R.pos[e][tx];
-        nrow[(size_t)e * ncap] = d.fin[m];
-        R.key[e][tx] = __int_as_float(d.sid[m]);
-    }
-    // carry every non-zero stored overlap of the old row to the pair's new entry
-    const int ocnt = D.flag == 2 ? 0 : d.cnt[lp][old];
-    unsigned ohm = D.flag == 2 ? 0u : d.hmask[lp][old];
-    if (ocnt < 32) ohm &= (1u << ocnt) - 1u;
-    unsigned nhm = 0u;
-    while (ohm) {
-        const int eo = __ffs(ohm) - 1;
-        ohm &= ohm - 1u;
-        const float hx = ho[(size_t)eo * ncap], hy = ho[plane + (size_t)eo * ncap], hz = ho[2 * plane + (size_t)eo * ncap];
-        if (hx == 0.f && hy == 0.f && hz == 0.f) continue;
-        const int oid = (int)(__float_as_uint(d.vel[cur][orow[(size_t)eo * ncap]].w) & ID_MASK);
-        for (int e = 0; e < nc; ++e) {
-            if (__float_as_int(R.key[e][tx]) == oid) {
-                hn[(size_t)e * ncap] = hx;
-                hn[plane + (size_t)e * ncap] = hy;
-                hn[2 * plane + (size_t)e * ncap] = hz;
-                nhm |= 1u << e;
-                break;
-            }
-        }
-    }
-    d.cnt[nlp][s] = nc;
-    d.hmask[nlp][s] = nhm;
-    if (D.fext) d.fext[nlp][s] = d.fext[lp][old];      // held until overwritten, even across state writes
-    d.whist[nlp][s] = D.flag == 2 ? make_float4(0.f, 0.f, 0.f, 0.f) : d.whist[lp][old];
-    if (c.nwp >= 2) {
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        d.wseg[nlp][s] = D.flag == 2 ? z : d.wseg[lp][old];
-        d.wseg[nlp][ncap + s] = D.flag == 2 ? z : d.wseg[lp][ncap + old];
-    }
+    auto get = [&](int e, float& key, int& m) {
+        key = R.key[e][tx];
+        m = R.pos[e][tx];
+    };
+    const int most = __reduce_max_sync(__activemask(), nc);
+    if (most <= 9) row_out<9>(d, s, old, ps, D, c, nc, overflow, get);
+    else if (most <= 17) row_out<17>(d, s, old, ps, D, c, nc, overflow, get);
+    else row_out<MAXL>(d, s, old, ps, D, c, nc, overflow, get);
 }
 
-template <bool STAGED>
-__global__ void __launch_bounds__(RB_T, 16) k_rb_build(Dev d)
+__global__ void __launch_bounds__(RB_T, 10) k_rb_build(Dev d)
 {
     if (!d.g->any) return;
     __shared__ RowScratch R;
+    __shared__ Window W;
     constexpr int H = TILE / RB_T;           // blocks of RB_T threads per tile
     // over the cell-order positions: the threads of a warp hold neighbouring particles and
-    // scan overlapping cells (the rows go to the particles' new slots in the same tile).  The
-    // direct scan (the default) finds the neighbouring cells' positions in L1: staging them in
-    // shared memory (STAGED) was measured slower (0.83 against 0.70 ms per build of the 1M bed)
+    // scan overlapping cells (the rows go to the particles' new slots in the same tile)
     for (int u = blockIdx.x; u < d.ntiles * H; u += gridDim.x) {
         const int t = u / H;
         const int k = d.tile_inst[t];
@@ -598,34 +907,15 @@ __global__ void __launch_bounds__(RB_T, 16) k_rb_build(Dev d)
         const InstC& c = d.ic[k];
         const int p0 = t * TILE + (u % H) * RB_T;
         const int p = p0 + threadIdx.x;
-        if (STAGED) {
-            __shared__ Window W;
-            const int lo = max(c.slot0, p0 - RB_W), hi = min(c.slot0 + D.n_new, p0 + RB_T + RB_W);
-            __syncthreads();                 // the previous window is no longer read
-            if (threadIdx.x == 0) {
-                W.lo = lo;
-                W.n = max(0, hi - lo);
-            }
-            for (int i = lo + (int)threadIdx.x; i < hi; i += RB_T) W.pos[i - lo] = __ldg(d.spos + i);
-            __syncthreads();
-            if (p - c.slot0 < D.n_new) build_row<true>(d, p, D, c, R, &W);
-        } else {
-            if (p - c.slot0 >= D.n_new) continue;
-            build_row<false>(d, p, D, c, R, nullptr);
+        const int lo = max(c.slot0, p0 - RB_W), hi = min(c.slot0 + D.n_new, p0 + RB_T + RB_W);
+        __syncthreads();                     // the previous window is no longer read
+        if (threadIdx.x == 0) {
+            W.lo = lo;
+            W.n = max(0, hi - lo);
         }
-    }
-}
-
-// live particles after the rebuild: the binned ones (removed particles dropped)
-__global__ void k_rb_count(Dev d)
-{
-    if (!d.g->any) return;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < d.B; k += gridDim.x * blockDim.x) {
-        InstD& D = d.id[k];
-        if (!D.flag) continue;
-        const InstC& c = d.ic[k];
-        const unsigned last = (unsigned)(c.code0 + c.ncode - 1);
-        D.n_new = (int)(d.crange[last].x + d.crange[last].y - d.crange[c.code0].x);
+        for (int i = lo + (int)threadIdx.x; i < hi; i += RB_T) W.pos[i - lo] = __ldg(d.spos + i);
+        __syncthreads();
+        if (p - c.slot0 < D.n_new) build_row(d, p, D, c, R, W);
     }
 }
 
@@ -669,6 +959,7 @@ __global__ void k_rb_finish(Dev d)
     if (threadIdx.x == 0) {
         d.g->nlive = (int)base;
         d.g->any = 0u;
+        d.g->ncubes = 0;
     }
 }
 
@@ -2348,6 +2639,7 @@ struct Layout {
 
 struct Plan {
     std::vector<InstC> ic;
+    std::vector<int> cube_lg;
     std::vector<HostInstLo> hl;
     std::vector<unsigned> spread;
     std::vector<int> tile_inst;
@@ -2357,7 +2649,7 @@ struct Plan {
     unsigned ncodes = 0, nparts = 0;
     // offsets
     size_t o_pos[2], o_vel[2], o_omg[2], o_nbr[2], o_hist[2], o_cnt[2], o_hmask[2], o_fext[2], o_whist[2], o_wseg[2], o_wrem;
-    size_t o_cellcode, o_cslot, o_perm, o_fin, o_spos, o_sid, o_ccount, o_crange, o_part, o_pinst, o_soi, o_tile, o_live, o_bar, o_ic, o_id, o_spread, o_g,
+    size_t o_cellcode, o_cslot, o_perm, o_fin, o_spos, o_sid, o_ccount, o_crange, o_cubes, o_part, o_pinst, o_soi, o_tile, o_live, o_bar, o_ic, o_id, o_spread, o_g,
         o_goff, o_outF, o_outT, o_outV, o_outW, o_outWX, o_xi, o_cmask, o_stage, o_hl, o_small, o_wgeo;
     size_t bytes = 0;
 };
@@ -2440,6 +2732,14 @@ dem_status make_plan(const dem_config* cfg, Plan& p, std::string& err)
         code = (code + SCAN_TILE - 1) / SCAN_TILE * SCAN_TILE;   // scan chunks never straddle instances
         c.code0 = (int)code;
         c.ncode = 1 << tb;
+        {
+            // a cube of CUBE codes: the low 6 bits of the code, by axis
+            int lg[3] = {0, 0, 0}, pos = 0;
+            for (int b = 0; b < 32 && pos < 6; ++b)
+                for (int a = 0; a < 3; ++a)
+                    if (b < bits[a] && pos < 6) { ++lg[a]; ++pos; }
+            p.cube_lg.push_back(lg[0] | (lg[1] << 4) | (lg[2] << 8));
+        }
         code += (unsigned)c.ncode;
         c.floor_on = s.floor_on ? 1 : 0;
         c.zrem = INT_MIN;   // no removal height until dem_set_walls gives one
@@ -2508,6 +2808,7 @@ dem_status make_plan(const dem_config* cfg, Plan& p, std::string& err)
     p.o_sid = L.take(N * 4);
     p.o_ccount = L.take((size_t)p.ncodes * 4);
     p.o_crange = L.take((size_t)p.ncodes * 8);
+    p.o_cubes = L.take(((size_t)p.ncodes / CUBE + 1) * 4);
     p.o_part = L.take((size_t)std::max(1u, p.nparts) * 4);
     p.o_pinst = L.take((size_t)std::max(1u, p.nparts) * 4);
     p.o_soi = L.take(N * 4);
@@ -2602,22 +2903,20 @@ dem_status launch_rebuild(dem_ctx* ctx, cudaStream_t st)
 {
     const Dev& d = ctx->dev;
     const unsigned gt = (unsigned)ctx->grid_rb;
-    k_rb_clear<<<std::min(std::max(1u, ctx->nparts), 152u * 8u), 256, 0, st>>>(d);
     k_rb_bin<<<gt, TILE, 0, st>>>(d);
     k_scan_reduce<<<std::max(1u, ctx->nparts), SCAN_T, 0, st>>>(d);
     k_scan_top<<<1, 1024, 0, st>>>(d);
     k_scan_down<<<std::max(1u, ctx->nparts), SCAN_T, 0, st>>>(d);
     k_rb_scatter<<<gt, TILE, 0, st>>>(d);
     k_rb_cellsort<<<gt, TILE, 0, st>>>(d);
-    k_rb_count<<<1, 256, 0, st>>>(d);
     if (step_block(ctx) == SMW_BS)
         k_rb_winsort<SMW_SORT_W><<<gt, WS_T, 0, st>>>(d, ctx->grid_smw);
     else
         k_rb_tilesort<<<gt, TILE, 0, st>>>(d);
     if (ctx->list_staged)
-        k_rb_build<true><<<ctx->grid_build_staged, RB_T, 0, st>>>(d);
+        k_rb_build<<<ctx->grid_build_staged, RB_T, 0, st>>>(d);
     else
-        k_rb_build<false><<<ctx->grid_build, RB_T, 0, st>>>(d);
+        k_rb_cubes<<<ctx->grid_build, CB_T, cube_smem(ctx->Lmax), st>>>(d);
     k_rb_finish<<<1, 256, 0, st>>>(d);          // 256 threads: its shared arrays
     CU(cudaGetLastError());
     return DEM_OK;
@@ -3102,6 +3401,7 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
     d.sid = (int*)(base + p.o_sid);
     d.ccount = (unsigned*)(base + p.o_ccount);
     d.crange = (uint2*)(base + p.o_crange);
+    d.cubes = (int*)(base + p.o_cubes);
     d.part = (unsigned*)(base + p.o_part);
     d.part_inst = (int*)(base + p.o_pinst);
     d.slot_of_id = (int*)(base + p.o_soi);
@@ -3136,6 +3436,7 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
         idv[k].n = (int)p.count[k];
         idv[k].nid = (int)p.count[k];
         idv[k].flag = 2;
+        idv[k].cube_lg = p.cube_lg[k];
     }
     Glob gl{};
     gl.any = 1u;
@@ -3161,6 +3462,7 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
     CUC(cudaMemcpyAsync(ctx->d_hl, p.hl.data(), sizeof(HostInstLo) * p.B, cudaMemcpyHostToDevice, s));
     CUC(cudaMemsetAsync(d.hist[0], 0, (size_t)p.ncap * p.Lmax * 12, s));
     CUC(cudaMemsetAsync(d.hist[1], 0, (size_t)p.ncap * p.Lmax * 12, s));
+    CUC(cudaMemsetAsync(d.ccount, 0, (size_t)p.ncodes * 4, s));   // every build leaves the counts zero
     CUC(cudaMemsetAsync(d.bar, 0, sizeof(unsigned long long) * 3 * BAR_LINE, s));
     CUC(cudaMemsetAsync(d.wrem, 0, sizeof(double) * 2 * p.B, s));
     k_init_ids<<<nblk(p.ncap, 256), 256, 0, s>>>(d);
@@ -3209,9 +3511,10 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
         ctx->grid1 = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * std::max(1, b1)));
         ctx->grid_rb = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * 8));
         int bb = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_build<false>, RB_T, 0);
-        ctx->grid_build = std::max(1, std::min(ctx->ntiles * (TILE / RB_T), std::max(1, nsm) * std::max(1, bb)));
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_build<true>, RB_T, 0);
+        cudaFuncSetAttribute(k_rb_cubes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cube_smem(MAXL));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_cubes, CB_T, cube_smem(ctx->Lmax));
+        ctx->grid_build = std::max(1, std::min((int)(ctx->ncodes / CUBE) + 1, std::max(1, nsm) * std::max(1, bb)));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_build, RB_T, 0);
         ctx->grid_build_staged = std::max(1, std::min(ctx->ntiles * (TILE / RB_T), std::max(1, nsm) * std::max(1, bb)));
         cudaGetLastError();
     }

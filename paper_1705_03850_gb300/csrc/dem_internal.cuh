@@ -126,7 +126,9 @@ struct InstD {
     int n_new;           // live particles after the pending rebuild (removed ones dropped)
     int fext;            // 1: add the per-particle external force fext to the contact forces
     int nbin;            // slots below slot0 + nbin are in the cell lists of the last build
-    int pad[2];
+    int cube_lg;         // constant: log2 of the cells per axis of a list-build cube (4 bits each; here, as the
+                         // step kernel stages InstC)
+    int pad;
 };
 
 struct Glob {
@@ -149,6 +151,7 @@ struct Glob {
     long long todo;            // steps of the next graph launch (0: as many as the graph was built for)
     int nlive;                 // entries of live_tiles
     unsigned test_stall;       // 1: the next fused launch's first block skips its first barrier
+    int ncubes;                // list build: entries of cubes
     unsigned pool;             // SM-wide step blocks: slices claimed from the shared pool this launch
 };
 
@@ -175,6 +178,7 @@ struct Dev {
     int* sid;                  // particle IDs in cell order (list build)
     unsigned* ccount;
     uint2* crange;             // per cell code: {first cell-order position (exclusive scan), count}
+    int* cubes;                // list build: first cell codes of the cubes (64 codes) that hold particles
     unsigned* part;
     int* part_inst;            // instance owning each scan chunk of cell codes (-1: padding)
     int* slot_of_id;

@@ -328,7 +328,7 @@ class DEM:
         return self
 
     def set_list_build(self, staged):
-        """Neighbour-list build: 0 direct scan of the 27 cells (default), 1 staged in shared memory."""
+        """Neighbour-list build: 0 by cubes of cells (default), 1 by windows of cell-ordered positions."""
         self._check(self.L.dem_set_list_build(self.h, int(staged)), "set list build")
         return self
 
