@@ -976,7 +976,7 @@ __device__ __forceinline__ Coef<float> coef_of(const InstC& c)
 // ================================================================== step
 // MODE 0: one velocity-Verlet step (force at x^n with v^{n-1/2}, merged kick,
 // drift to x^{n+1}, displacement bound, rebuild decision by the last block).
-// MODE 1: forces at the current state only, written to the output arrays.
+// MODE 1: forces at the current state only, the outputs named in `want` (WANT_*) written.
 // MODE 2: one step from a saved state to another (rollouts): Dev's buffers 0 hold the state before
 // the step and receive nothing, buffers 1 receive the state after it, with its overlaps and their
 // mask; lists come from the instance's parity.  No displacement bound, no end of step.
@@ -1177,9 +1177,10 @@ __device__ __forceinline__ void cp_async4(unsigned dst, const void* src)
 // the end of the previous step (-1: none), kept so that a block of one instance stages it once
 // per launch and then only flips its state buffer (all else in them is constant between list
 // builds).
+constexpr int WANT_F = 1, WANT_T = 2, WANT_V = 4, WANT_W = 8, WANT_WX = 16, WANT_CONTACTS = 32, WANT_XI = 64;
 template <int MODE, bool WALLS, int BS, int LPP, bool FUSED = false>
 __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, InstD& sd, float* smax, int& kstaged,
-                                          const int* rows = nullptr, const int* rcnt = nullptr)
+                                          const int* rows = nullptr, const int* rcnt = nullptr, int want = 0)
 {
     const int nthr = FUSED ? (int)blockDim.x : BS;   // fused steps choose their block size by the system's
     const int WPB = nthr / 32;               // warps per block
@@ -1378,9 +1379,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         // for every lane of a group)
 #pragma unroll
         for (int o = 1; o < LPP; o <<= 1) tm |= __shfl_xor_sync(gmask, tm, o);
-        // entries that left contact (or, for the read-out, every non-contact) get no history
-        const unsigned rowmask = ncnt >= 32 ? 0xffffffffu : ((1u << ncnt) - 1u);
-        unsigned clr = MODE == 2 ? 0u : (MODE == 1 ? rowmask : hm) & ~tm & submask;
+        // entries that left contact get no history (the read-out's contacts are in cmask)
+        unsigned clr = MODE != 0 ? 0u : hm & ~tm & submask;
         while (clr) {
             const int e = __ffs(clr) - 1;
             clr &= clr - 1u;
@@ -1463,9 +1463,11 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
                 F = F + fa;
                 Tq = Tq - r * cross(n, ft);
             }
-            ho[(size_t)e * ncap] = xi.x;
-            ho[plane + (size_t)e * ncap] = xi.y;
-            ho[2 * plane + (size_t)e * ncap] = xi.z;
+            if (MODE != 1 || (want & WANT_XI)) {
+                ho[(size_t)e * ncap] = xi.x;
+                ho[plane + (size_t)e * ncap] = xi.y;
+                ho[2 * plane + (size_t)e * ncap] = xi.z;
+            }
             sl ^= 1;
         }
         // the group's partial sums, combined in a fixed order (every lane ends with the same bits)
@@ -1517,12 +1519,14 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         }
         if (MODE == 1) {
             const float hk = prime ? 0.f : 0.5f * c.dt;
-            d.outF[s] = make_float4(F.x, F.y, F.z, 0.f);
-            d.outT[s] = make_float4(Tq.x, Tq.y, Tq.z, 0.f);
-            d.outV[s] = make_float4(Vv.x + hk * F.x * inv_m, Vv.y + hk * F.y * inv_m, Vv.z + hk * F.z * inv_m, 0.f);
-            d.outW[s] = make_float4(Wv.x + hk * Tq.x * inv_I, Wv.y + hk * Tq.y * inv_I, Wv.z + hk * Tq.z * inv_I, 0.f);
-            d.outWX[s] = make_float4(wxi.x, wxi.y, wxi.z, (float)((wall_now ? 1 : 0) + nseg));
-            d.cmask[s] = cm;
+            if (want & WANT_F) d.outF[s] = make_float4(F.x, F.y, F.z, 0.f);
+            if (want & WANT_T) d.outT[s] = make_float4(Tq.x, Tq.y, Tq.z, 0.f);
+            if (want & WANT_V)
+                d.outV[s] = make_float4(Vv.x + hk * F.x * inv_m, Vv.y + hk * F.y * inv_m, Vv.z + hk * F.z * inv_m, 0.f);
+            if (want & WANT_W)
+                d.outW[s] = make_float4(Wv.x + hk * Tq.x * inv_I, Wv.y + hk * Tq.y * inv_I, Wv.z + hk * Tq.z * inv_I, 0.f);
+            if (want & WANT_WX) d.outWX[s] = make_float4(wxi.x, wxi.y, wxi.z, (float)((wall_now ? 1 : 0) + nseg));
+            if (want & WANT_CONTACTS) d.cmask[s] = cm;
         } else {
             const float kick = prime ? 0.5f * c.dt : c.dt;
             Vv.x += kick * F.x * inv_m;
@@ -1652,7 +1656,7 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
 // or no step left to do, does nothing (the graph's loop at the end makes up for the steps left
 // out), so that no step runs on lists that are out of date.
 struct StepCtl {
-    int counted;                           // 0: a launch of its own (no graph): always steps
+    int counted;                           // 0: a launch of its own (no graph): always steps (MODE 1: WANT_*)
     int set_rb, set_loop;                  // set the condition h_rb (a list build is due) / h_loop (steps remain)
     cudaGraphConditionalHandle h_rb, h_loop;
 };
@@ -1677,7 +1681,7 @@ __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int 
             return;
         }
     }
-    step_pass<MODE, WALLS, BS, LPP>(d, prime, sc, sd, smax, kstaged);
+    step_pass<MODE, WALLS, BS, LPP>(d, prime, sc, sd, smax, kstaged, nullptr, nullptr, MODE == 1 ? ctl.counted : 0);
     if (MODE == 0) {
         // the last block to finish accumulates the bound per instance and decides on rebuilds
         if (threadIdx.x == 0) am_last = add_acq_rel(&d.g->counter) == gridDim.x - 1;
@@ -1966,14 +1970,16 @@ __global__ void k_write_field(Dev d, int field, const double* __restrict__ src, 
     const int s = d.slot_of_id[c.slot0 + id];
     if (s < 0) return;                       // removed particle
     const int cur = d.id[k].cur;
-    const double q = hl[k].q;
+    const double iq = 1.0 / hl[k].q;
     if (field == DEM_F_POS) {
         int4 p = d.pos[cur][s];
         int xi[3];
         for (int a = 0; a < 3; ++a) {
-            double u = rint((src[3 * g + a] - hl[k].lo[a]) / q);
-            if (c.per[a]) {
-                double L = (double)c.ext[a];
+            // (the quantum is a power of two: its reciprocal is exact; the period's division is only
+            // for positions outside the box)
+            double u = rint((src[3 * g + a] - hl[k].lo[a]) * iq);
+            const double L = (double)c.ext[a];
+            if (c.per[a] && !(u >= 0.0 && u < L)) {
                 u = u - L * floor(u / L);
                 if (u >= L) u -= L;
             }
@@ -1996,7 +2002,7 @@ __global__ void k_write_field(Dev d, int field, const double* __restrict__ src, 
     } else if (field == DEM_F_RADIUS) {
         int4 p = d.pos[cur][s];
         const double r = src[g];
-        p.w = (int)rint(r / q);
+        p.w = (int)rint(r * iq);
         d.pos[cur][s] = p;
         float4 w = d.omg[cur][s];
         w.w = (float)(hl[k].rho * (4.0 / 3.0) * 3.14159265358979323846 * r * r * r);
@@ -2955,11 +2961,13 @@ dem_status order_slots(dem_ctx* ctx)
     return launch_rebuild(ctx, ctx->stream);
 }
 
-dem_status launch_eval(dem_ctx* ctx)
+// the forces at the current state, with the outputs in `want` (WANT_*): the others' stores cost a
+// read of one field a fifth of its time
+dem_status launch_eval(dem_ctx* ctx, int want)
 {
     dem_status st = ensure_lists(ctx);
     if (st) return st;
-    k_step<1, true><<<ctx->grid1, TILE, 0, ctx->stream>>>(ctx->dev, ctx->fresh ? 1 : 0, StepCtl{});
+    k_step<1, true><<<ctx->grid1, TILE, 0, ctx->stream>>>(ctx->dev, ctx->fresh ? 1 : 0, StepCtl{want, 0, 0, 0, 0});
     CU(cudaGetLastError());
     return DEM_OK;
 }
@@ -3599,9 +3607,10 @@ dem_status dem_read(dem_ctx* ctx, int32_t field, void* dst, int64_t n)
     if (n != total_count(ctx)) return fail(ctx, DEM_ERR_ARG, "n must equal the total particle count");
     if (n == 0) return DEM_OK;
     if (!dst) return fail(ctx, DEM_ERR_ARG, "null destination");
-    if (field == DEM_F_VEL || field == DEM_F_OMEGA || field == DEM_F_FORCE || field == DEM_F_TORQUE ||
-        field == DEM_F_WALL_XI || field == DEM_F_NBR_COUNT) {
-        dem_status st = launch_eval(ctx);
+    const int want = field == DEM_F_VEL ? WANT_V : field == DEM_F_OMEGA ? WANT_W : field == DEM_F_FORCE ? WANT_F
+                   : field == DEM_F_TORQUE ? WANT_T : field == DEM_F_WALL_XI ? WANT_WX : 0;
+    if (want || field == DEM_F_NBR_COUNT) {
+        dem_status st = want ? launch_eval(ctx, want) : ensure_lists(ctx);
         if (st) return st;
     }
     const bool dev = is_device_ptr(dst);
@@ -3623,7 +3632,7 @@ dem_status dem_read_contacts(dem_ctx* ctx, int32_t* partner, double* xi, int32_t
     if (dem_status st = refresh_count(ctx)) return st;
     if (n != total_count(ctx) || width < 1 || !partner || !xi) return fail(ctx, DEM_ERR_ARG, "bad contacts arguments");
     if (!is_device_ptr(partner) || !is_device_ptr(xi)) return fail(ctx, DEM_ERR_ARG, "contacts buffers must be device memory");
-    dem_status st = launch_eval(ctx);
+    dem_status st = launch_eval(ctx, WANT_CONTACTS | WANT_XI);
     if (st) return st;
     k_read_contacts<<<nblk(ctx->ncap, 256), 256, 0, ctx->stream>>>(ctx->dev, partner, xi, width);
     CU(cudaGetLastError());
@@ -3735,7 +3744,7 @@ dem_status dem_stats(dem_ctx* ctx, dem_stats_t* out)
     if (dem_status st = refresh_count(ctx)) return st;
     out->particles = total_count(ctx);
     if (!ctx->have_state) return DEM_OK;
-    dem_status st = launch_eval(ctx);
+    dem_status st = launch_eval(ctx, WANT_CONTACTS | WANT_WX);
     if (st) return st;
     CU(cudaMemsetAsync(&ctx->dev.g->sum_list, 0, 24, ctx->stream));
     k_stats<<<nblk(ctx->ncap, 256), 256, 0, ctx->stream>>>(ctx->dev);
@@ -3881,7 +3890,7 @@ dem_status dem_grid_fields(dem_ctx* ctx, int32_t k, const double lo[3], double h
     if (out_len != 5 * ncell) return fail(ctx, DEM_ERR_ARG, "out must hold 5 values per cell");
     if (!is_device_ptr(out)) return fail(ctx, DEM_ERR_ARG, "out must be device memory");
     if (!ctx->have_state) return fail(ctx, DEM_ERR_STATE, "write the state first");
-    dem_status st = launch_eval(ctx);
+    dem_status st = launch_eval(ctx, WANT_V);
     if (st) return st;
     CU(cudaMemsetAsync(out, 0, sizeof(double) * 5 * ncell, ctx->stream));
     k_grid_sums<<<ctx->grid_rb, 256, 0, ctx->stream>>>(ctx->dev, k, ctx->d_hl, lo[0], lo[1], lo[2], h, n[0], n[1],
@@ -4155,7 +4164,7 @@ dem_status dem_observables(dem_ctx* ctx, const double* axis, double* out)
     if (!ctx || !axis || !out) return DEM_ERR_ARG;
     if (ctx->status) return check_status(ctx);
     if (!ctx->have_state) return fail(ctx, DEM_ERR_STATE, "write the state first");
-    dem_status st = launch_eval(ctx);
+    dem_status st = launch_eval(ctx, WANT_V | WANT_W);
     if (st) return st;
     std::vector<double> sm(16 * ctx->B, 0.0);
     for (int k = 0; k < ctx->B; ++k) { sm[16 * k] = axis[2 * k]; sm[16 * k + 1] = axis[2 * k + 1]; }
@@ -4177,7 +4186,7 @@ dem_status dem_rollout_adjoint(dem_ctx* ctx, const double* weights, const double
     if (!ro.ready) return fail(ctx, DEM_ERR_STATE, "run dem_rollout_forward first");
     cudaStream_t s = ctx->stream;
     // observables and their seeds at the final step N
-    dem_status st = launch_eval(ctx);
+    dem_status st = launch_eval(ctx, WANT_V | WANT_W);
     if (st) return st;
     std::vector<double> sm(16 * ctx->B, 0.0);
     for (int k = 0; k < ctx->B; ++k) {

@@ -84,7 +84,6 @@ dem_status check_status(dem_ctx* ctx);
 dem_status refresh_count(dem_ctx* ctx);
 dem_status launch_rebuild(dem_ctx* ctx, cudaStream_t st);
 dem_status ensure_lists(dem_ctx* ctx);
-dem_status launch_eval(dem_ctx* ctx);
 long long total_count(const dem_ctx* ctx);
 void set_thread_error(const std::string& msg);
 }  // namespace cgdem
