@@ -261,7 +261,7 @@ class DEM:
         shape = (self.n, 3) if _WIDTH[field] == 3 else (self.n,)
         if out is None:
             out = (torch.empty(shape, dtype=torch.float64, device=self.device) if not host
-                   else torch.empty(shape, dtype=torch.float64).pin_memory())
+                   else torch.empty(shape, dtype=torch.float64, pin_memory=True))
         self._check(self.L.dem_read(self.h, field, ctypes.c_void_p(out.data_ptr()), self.n), "read")
         return out.numpy() if host and out.device.type == "cpu" else out
 
