@@ -87,6 +87,10 @@ struct Acc {
     // build, [2] particles appended at this call
     unsigned long long* pairs;   // [PAIRS_MAX]
     int* npairs;                 // [4]
+    // particles in transition cells found by the passes over the levels: {slot, cell}, and their
+    // number, per level (0 coarse, 1 fine)
+    int2* layl[2];
+    int* nlay;                   // [2]
 };
 constexpr int PAIRS_MAX = 4096;
 
@@ -179,6 +183,17 @@ __device__ __forceinline__ int layer_cell(const Geo& g, const double* x, int* fi
     return -1;
 }
 
+// notes a particle in a transition cell (one atomic per warp)
+__device__ __forceinline__ void layer_list(const Acc& a, int L, int s, int cell)
+{
+    const unsigned act = __activemask();
+    const int lane = (int)threadIdx.x & 31, lead = __ffs(act) - 1;
+    int at = 0;
+    if (lane == lead) at = atomicAdd(a.nlay + L, __popc(act));
+    at = __shfl_sync(act, at, lead) + __popc(act & ((1u << lane) - 1u));
+    a.layl[L][at] = make_int2(s, cell);
+}
+
 // add (m, m v, V) of a particle to its correction cell.  With the whole warp active, the lanes
 // form runs of equal cells (consecutive slots: Morton order keeps a cell's particles together);
 // a segmented scan over the warp sums each run in float (at most 32 terms) and the run's last
@@ -219,13 +234,30 @@ __device__ __forceinline__ void atomic_max_f(unsigned* a, float v)
     if (v > 0.f) atomicMax(a, __float_as_uint(v));
 }
 
+// components of a symmetric tensor: xx, yy, zz, xy, xz, yz
+__device__ __forceinline__ constexpr int ij(int k, int i)
+{
+    return i == 0 ? (k < 3 ? k : k == 5 ? 1 : 0) : (k < 3 ? k : k == 3 ? 1 : 2);
+}
+
+// st += r f on the diagonal, r_a f_b + r_b f_a beside it: nine multiply-adds (an instruction of the
+// FP64 pipe takes 16 cycles of an SM here, and these are most of the layer pass's)
+__device__ __forceinline__ void add_dyad(double* st, double x, double y, double z, Vec3<float> f)
+{
+    const double fx = f.x, fy = f.y, fz = f.z;
+    st[0] = fma(x, fx, st[0]);
+    st[1] = fma(y, fy, st[1]);
+    st[2] = fma(z, fz, st[2]);
+    st[3] = fma(x, fy, fma(y, fx, st[3]));
+    st[4] = fma(x, fz, fma(z, fx, st[4]));
+    st[5] = fma(y, fz, fma(z, fy, st[5]));
+}
+
 // Eq. 7 accumulation of one particle into a transition cell: mass, momentum,
 // m v v, volume, and the contact part 1/2 r_ij (x) f_ij over its contacts
 // (floor contact: branch vector to the contact point, no 1/2), symmetrised.
-// (not inlined: few particles lie in a transition cell, and inlining the contact law would
-// give every thread of the per-particle passes its registers)
-__device__ __noinline__ void layer_add(const Dev& d, const InstC& c, const InstD& D, int s, double* acc, unsigned* vmax,
-                                       int fresh)
+__device__ __forceinline__ void layer_add(const Dev& d, const InstC& c, const InstD& D, int s, double* acc, unsigned* vmax,
+                                          int fresh)
 {
     const int cur = D.cur, lp = D.lp, ncap = d.ncap;
     const size_t plane = (size_t)d.Lmax * ncap;
@@ -234,10 +266,10 @@ __device__ __noinline__ void layer_add(const Dev& d, const InstC& c, const InstD
     const double m = Wv.w, q = c.q;
     const double r = (double)P.w * q;
     const double v[3] = {Vv.x, Vv.y, Vv.z};
+    const double mv[3] = {m * v[0], m * v[1], m * v[2]};
     atomicAdd(acc + 0, m);
-    for (int a = 0; a < 3; ++a) atomicAdd(acc + 1 + a, m * v[a]);
-    const int ij[6][2] = {{0, 0}, {1, 1}, {2, 2}, {0, 1}, {0, 2}, {1, 2}};
-    for (int k = 0; k < 6; ++k) atomicAdd(acc + 4 + k, m * v[ij[k][0]] * v[ij[k][1]]);
+    for (int a = 0; a < 3; ++a) atomicAdd(acc + 1 + a, mv[a]);
+    for (int k = 0; k < 6; ++k) atomicAdd(acc + 4 + k, mv[ij(k, 0)] * v[ij(k, 1)]);
     atomicAdd(acc + 10, 4.0 / 3.0 * 3.14159265358979323846 * r * r * r);
     atomic_max_f(vmax, sqrtf(Vv.x * Vv.x + Vv.y * Vv.y + Vv.z * Vv.z));
     const Coef<float> cf{c.c_kn, c.c_kt, c.nbeta, c.gt_ratio, c.mu, c.mu_w, c.clamp_fn};
@@ -289,12 +321,11 @@ __device__ __noinline__ void layer_add(const Dev& d, const InstC& c, const InstD
                                                          Wj.w, mk3(Vv.x, Vv.y, Vv.z), mk3(Vj.x, Vj.y, Vj.z),
                                                          mk3(Wv.x, Wv.y, Wv.z), mk3(Wj.x, Wj.y, Wj.z), xi, dt_hist,
                                                          ft, slip);
-        const double rv[3] = {dx * q, dy * q, dz * q}, f[3] = {fa.x, fa.y, fa.z};
-        for (int k = 0; k < 6; ++k) {
-            const int a = ij[k][0], b = ij[k][1];
-            st[k] += 0.25 * (rv[a] * f[b] + rv[b] * f[a]);
-        }
+        // 1/2 (r_a f_b + r_b f_a) with the separation still in units: its quantum, and the other 1/2
+        // of Eq. 7, once at the end
+        add_dyad(st, (double)dx, (double)dy, (double)dz, fa);
     }
+    for (int k = 0; k < 6; ++k) st[k] *= (k < 3 ? 0.5 : 0.25) * q;
     if (c.floor_on && P.w - P.z > 0) {
         const float4 hw = d.whist[lp][s];
         const bool wall_prev = (__float_as_uint(Vv.w) & WALL_BIT) != 0u;
@@ -305,22 +336,41 @@ __device__ __noinline__ void layer_add(const Dev& d, const InstC& c, const InstD
                                                         (float)m, 0.f, mk3(Vv.x, Vv.y, Vv.z),
                                                         mk3(c.floor_v[0], c.floor_v[1], c.floor_v[2]),
                                                         mk3(Wv.x, Wv.y, Wv.z), mk3(0.f, 0.f, 0.f), xi, dt_hist, ft, slip);
-        const double rv[3] = {0.0, 0.0, (double)P.z * q}, f[3] = {fa.x, fa.y, fa.z};
-        for (int k = 0; k < 6; ++k) {
-            const int a = ij[k][0], b = ij[k][1];
-            st[k] += 0.5 * (rv[a] * f[b] + rv[b] * f[a]);
-        }
+        const double rz = (double)P.z * q;
+        st[2] += rz * fa.z;
+        st[4] += 0.5 * rz * fa.x;
+        st[5] += 0.5 * rz * fa.y;
     }
     if (c.nwp >= 2) {   // axisymmetric walls: branch vector from the contact point to the centre
-        const double ex = (double)P.x - c.wax, ey = (double)P.y - c.way, z = (double)P.z;
-        const double rho = sqrt(ex * ex + ey * ey);
-        float erx = 1.f, ery = 0.f;
-        if (rho > 0.0) {
-            erx = (float)(ex / rho);
-            ery = (float)(ey / rho);
-        }
-        const float4 h0 = d.wseg[lp][s], h1 = d.wseg[lp][(size_t)ncap + s];
+        // the segments a float pre-test leaves (as the step kernel's: its margin is far above its
+        // error); the roots and divisions in double are for those alone
+        const float exf = (float)(P.x - c.waxi) - c.waxf, eyf = (float)(P.y - c.wayi) - c.wayf, zf = (float)P.z;
+        const float rhof = sqrtf(exf * exf + eyf * eyf);
+        const float lim = (float)P.w * (1.f + 1.f / 64.f) + 1e-6f * (rhof + fabsf(zf) + c.wmag) + 4.f;
+        const WallGeo& G = d.wgeo[0];
+        unsigned nearm = 0u;
         for (int k = 0; k + 1 < c.nwp; ++k) {
+            const float r0 = c.wpf[2 * k], z0 = c.wpf[2 * k + 1];
+            const float dr = c.wpf[2 * k + 2] - r0, dz = c.wpf[2 * k + 3] - z0;
+            const float t = fminf(fmaxf(((rhof - r0) * dr + (zf - z0) * dz) * G.inv2[k], 0.f), 1.f);
+            const float a = rhof - (r0 + t * dr), b = zf - (z0 + t * dz);
+            if (a * a + b * b < lim * lim) nearm |= 1u << k;
+        }
+        const double ex = (double)P.x - c.wax, ey = (double)P.y - c.way, z = (double)P.z;
+        double rho = 0.0;
+        float erx = 1.f, ery = 0.f;
+        float4 h0, h1;
+        if (nearm) {
+            rho = sqrt(ex * ex + ey * ey);
+            if (rho > 0.0) {
+                erx = (float)(ex / rho);
+                ery = (float)(ey / rho);
+            }
+            h0 = d.wseg[lp][s];
+            h1 = d.wseg[lp][(size_t)ncap + s];
+        }
+        for (; nearm; nearm &= nearm - 1u) {
+            const int k = __ffs(nearm) - 1;
             double a, b;
             wall_seg_offset(c, k, rho, z, a, b);
             const double dist = sqrt(a * a + b * b);
@@ -338,38 +388,27 @@ __device__ __noinline__ void layer_add(const Dev& d, const InstC& c, const InstD
                                                             mk3(Vv.x, Vv.y, Vv.z), mk3(0.f, 0.f, 0.f),
                                                             mk3(Wv.x, Wv.y, Wv.z), mk3(0.f, 0.f, 0.f), xi, dt_hist,
                                                             ft, slip);
-            const double rv[3] = {dist * q * n.x, dist * q * n.y, dist * q * n.z}, f[3] = {fa.x, fa.y, fa.z};
-            for (int kk = 0; kk < 6; ++kk) {
-                const int ia = ij[kk][0], ib = ij[kk][1];
-                st[kk] += 0.5 * (rv[ia] * f[ib] + rv[ib] * f[ia]);
-            }
+            double sw[6] = {0, 0, 0, 0, 0, 0};
+            add_dyad(sw, dist * q * n.x, dist * q * n.y, dist * q * n.z, fa);
+            for (int kk = 0; kk < 6; ++kk) st[kk] += kk < 3 ? sw[kk] : 0.5 * sw[kk];
         }
     }
     for (int k = 0; k < 6; ++k) atomicAdd(acc + 11 + k, st[k]);
 }
 
-// the live slots of a single-instance context (coupling contexts have one instance), two per
-// thread and iteration, with both slots' position and velocity loaded before either is used;
-// removed particles (below a wall's removal height) are skipped
+// the live slots of a single-instance context (coupling contexts have one instance), one per
+// thread of blocks of TILE over all its tiles; removed particles (below a wall's removal height)
+// are skipped
 template <typename Fn>
 __device__ __forceinline__ void for_live(const Dev& d, Fn fn)
 {
     const InstD D = d.id[0];
     const InstC& c = d.ic[0];
-    const int4* __restrict__ pos = d.pos[D.cur];
-    const float4* __restrict__ vel = d.vel[D.cur];
-    const int end = c.slot0 + D.n;
-    const int stride = (int)(gridDim.x * blockDim.x);
-    for (int s0 = c.slot0 + (int)(blockIdx.x * blockDim.x + threadIdx.x); s0 < end; s0 += 2 * stride) {
-        const int s1 = s0 + stride;
-        const bool has1 = s1 < end;
-        const int4 P0 = pos[s0];
-        const float4 V0 = vel[s0];
-        const int4 P1 = has1 ? pos[s1] : P0;
-        const float4 V1 = has1 ? vel[s1] : V0;
-        if (!(__float_as_uint(V0.w) & GONE_BIT)) fn(s0, c, D, P0, V0);
-        if (has1 && !(__float_as_uint(V1.w) & GONE_BIT)) fn(s1, c, D, P1, V1);
-    }
+    const int s = c.slot0 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (s >= c.slot0 + D.n) return;
+    const int4 P = d.pos[D.cur][s];
+    const float4 V = d.vel[D.cur][s];
+    if (!(__float_as_uint(V.w) & GONE_BIT)) fn(s, c, D, P, V);
 }
 
 // one element of the per-call accumulators per thread (a thread per cell with a loop over its
@@ -387,6 +426,7 @@ __global__ void k_cp_clear(Geo g, Acc a)
         a.nins[i] = 0;
     }
     if (i == 0) a.removed[0] = 0;
+    if (i < 2) a.nlay[i] = 0;
 }
 inline int clear_threads(int S, int C) { return std::max(std::max(S * MAXBINS, 2 * S * 20), 2 * C * 5); }
 
@@ -451,7 +491,7 @@ __global__ void __launch_bounds__(TILE, 8) k_cp_coarse(Dev d, Geo g, Acc a, int 
             }
             int fk;
             const int lc = maybe_layer(g, 0, P) ? layer_cell(g, x, &fk) : -1;
-            if (lc >= 0) layer_add(d, c, D, s, a.lay + (size_t)lc * 20, a.vmax + lc, g.fresh_c);
+            if (lc >= 0) layer_list(a, 0, s, lc);
             const float rf = (float)r;
             corr_add(a.cor, corr_cell_u(g, a.thr, 0, P), mf, V, 4.18879020f * rf * rf * rf);
         }
@@ -466,36 +506,38 @@ __global__ void __launch_bounds__(TILE, 8) k_cp_coarse(Dev d, Geo g, Acc a, int 
     });
 }
 
-// fine level: transition and correction cells, removal through drain faces
+// fine level: transition and correction cells
 __global__ void __launch_bounds__(TILE, 8) k_cp_fine(Dev d, Geo g, Acc a)
 {
-    for_live(d, [&](int s, const InstC& c, const InstD& D, const int4 P, float4 V) {
-        const float mf = d.omg[D.cur][s].w;     // loaded before the layer call (which may write memory)
+    for_live(d, [&](int s, const InstC& c, const InstD& D, const int4 P, const float4 V) {
+        const float mf = d.omg[D.cur][s].w;
         if (maybe_layer(g, 1, P)) {
             const double x[3] = {posm(g.lof, g.qf, P.x, 0), posm(g.lof, g.qf, P.y, 1), posm(g.lof, g.qf, P.z, 2)};
             int fk;
             const int lc = layer_cell(g, x, &fk);
-            if (lc >= 0) layer_add(d, c, D, s, a.lay + ((size_t)g.S + lc) * 20, a.vmax + g.S + lc, g.fresh_f);
+            if (lc >= 0) layer_list(a, 1, s, lc);
         }
         const float rf = (float)((double)P.w * g.qf);
         corr_add(a.cor + (size_t)g.C * 5, corr_cell_u(g, a.thr, 1, P), mf, V, 4.18879020f * rf * rf * rf);
-        // drain faces: x < lo or x >= hi on their axes (the region bounds as integer thresholds)
-        bool gone = false;
-        for (int ax = 0; ax < 3; ++ax) {
-            const long long* T = a.thr + ((size_t)3 + ax) * (MAXCR + 1);
-            const long long u = ax == 0 ? P.x : ax == 1 ? P.y : P.z;
-            if ((g.drain >> (2 * ax)) & 1) gone |= u < __ldg(T);
-            if ((g.drain >> (2 * ax + 1)) & 1) gone |= u >= __ldg(T + g.ncr[ax]);
-        }
-        if (gone) {
-            // marked and left in place with no radius until the next list build drops it (its
-            // neighbours, further than a radius from its centre, can no longer touch it)
-            V.w = __uint_as_float(__float_as_uint(V.w) | GONE_BIT);
-            d.vel[D.cur][s] = V;
-            d.pos[D.cur][s] = make_int4(P.x, P.y, P.z, 0);
-            atomicAdd(a.removed, 1);
-        }
     });
+}
+
+// Eq. 7 of the listed particles of both levels (the few in transition cells, a particle a thread):
+// walking a row and its contacts takes some 10 us of latency and the contact law's registers, which
+// the passes over all particles, in which whole warps waited for a few lanes, are spared.  Two-level
+// silo: 32 us here and 13 and 12 us in the passes over the levels, against 36 and 45 us with the law
+// called from those; three-level chute 31, 15 and 22 us against 29 and 62 us.  With four lanes a
+// particle the pass takes 29 us, but the periods no less.
+__global__ void __launch_bounds__(64) k_cp_layer(const __grid_constant__ Dev dc, const __grid_constant__ Dev df, Geo g, Acc a)
+{
+    const int n0 = a.nlay[0], n1 = a.nlay[1];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n0 + n1; i += gridDim.x * blockDim.x) {
+        const int L = i < n0 ? 0 : 1;
+        const int2 sl = a.layl[L][L ? i - n0 : i];
+        const Dev& d = L ? df : dc;
+        const size_t cell = (size_t)L * g.S + sl.y;
+        layer_add(d, d.ic[0], d.id[0], sl.x, a.lay + cell * 20, a.vmax + cell, L ? g.fresh_f : g.fresh_c);
+    }
 }
 
 // per cell: finish the averages, update the controllers.  Threads 2i and 2i + 1 take surface
@@ -558,11 +600,30 @@ __global__ void k_cp_cells(Geo g, Acc a)
         }
     }
 }
+constexpr int LAYER_BLOCKS = 152 * 8;
 inline int cells_threads(int S, int C) { return ((2 * S + 31) & ~31) + C; }
 
+// the stress controllers' force on the fine level's particles, and removal through drain faces
 __global__ void __launch_bounds__(TILE) k_cp_force_fine(Dev d, Geo g, Acc a)
 {
-    for_live(d, [&](int s, const InstC& c, const InstD& D, const int4 P, const float4 V) {
+    for_live(d, [&](int s, const InstC& c, const InstD& D, const int4 P, float4 V) {
+        // drain faces: x < lo or x >= hi on their axes (the region bounds as integer thresholds)
+        bool gone = false;
+        for (int ax = 0; ax < 3; ++ax) {
+            const long long* T = a.thr + ((size_t)3 + ax) * (MAXCR + 1);
+            const long long u = ax == 0 ? P.x : ax == 1 ? P.y : P.z;
+            if ((g.drain >> (2 * ax)) & 1) gone |= u < __ldg(T);
+            if ((g.drain >> (2 * ax + 1)) & 1) gone |= u >= __ldg(T + g.ncr[ax]);
+        }
+        if (gone) {
+            // marked and left in place with no radius until the next list build drops it (its
+            // neighbours, further than a radius from its centre, can no longer touch it)
+            V.w = __uint_as_float(__float_as_uint(V.w) | GONE_BIT);
+            d.vel[D.cur][s] = V;
+            d.pos[D.cur][s] = make_int4(P.x, P.y, P.z, 0);
+            atomicAdd(a.removed, 1);
+            return;
+        }
         // the held force first: a load with no dependence on the layer test below
         const float4 o = g.add ? d.fext[D.lp][s] : make_float4(0.f, 0.f, 0.f, 0.f);
         float4 F = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -577,6 +638,8 @@ __global__ void __launch_bounds__(TILE) k_cp_force_fine(Dev d, Geo g, Acc a)
             const Face& f = g.face[fk];
             const double r = (double)P.w * g.qf, m = d.omg[D.cur][s].w;
             const double sdist = f.side == 0 ? x[f.axis] - f.plane : f.plane - x[f.axis];
+            // deeper than the fade (most of the layer): no force, and none of the divisions below
+            if (!(sdist >= 3.0 * r && isfinite(a.ctrl[3 * (size_t)lc + 2]))) {
             const double w = fmax(0.0, 1.0 - sdist / (1.5 * 2.0 * r));
             const double u = a.ctrl[3 * (size_t)lc + 2];
             double Fv[3] = {0, 0, 0};
@@ -598,6 +661,7 @@ __global__ void __launch_bounds__(TILE) k_cp_force_fine(Dev d, Geo g, Acc a)
                 else lam = fmin(1.0, (-VA + sqrt(VA * VA - A2 * (V2 - vmax * vmax))) / A2);
             }
             F = make_float4((float)(lam * Fv[0]), (float)(lam * Fv[1]), (float)(lam * Fv[2]), 0.f);
+            }
         }
         if (g.add) F = make_float4(o.x + F.x, o.y + F.y, o.z + F.z, 0.f);
         d.fext[D.lp][s] = F;
@@ -1135,7 +1199,7 @@ size_t coupler_layout(dem_coupler* cp, char* base)
            o_vmax = L.take(2 * S * 4), o_ctrl = L.take(S * 24), o_out = L.take(2 * S * 88), o_cor = L.take(2 * C * 40),
            o_dv = L.take(C * 24), o_prev = L.take(ncap * 16), o_pok = L.take(ncap * 4), o_rem = L.take(16),
            o_ovf = L.take(16), o_thr = L.take(2 * 3 * (MAXCR + 1) * 8), o_pairs = L.take(PAIRS_MAX * 8),
-           o_np = L.take(16);
+           o_np = L.take(16), o_lc = L.take(ncap * 8), o_lf = L.take((size_t)cp->f->ncap * 8), o_nl = L.take(16);
     if (base) {
         Acc& a = cp->a;
         a.cross = (unsigned long long*)(base + o_cross);
@@ -1157,6 +1221,9 @@ size_t coupler_layout(dem_coupler* cp, char* base)
         a.removed = (int*)(base + o_rem);
         a.pairs = (unsigned long long*)(base + o_pairs);
         a.npairs = (int*)(base + o_np);
+        a.layl[0] = (int2*)(base + o_lc);
+        a.layl[1] = (int2*)(base + o_lf);
+        a.nlay = (int*)(base + o_nl);
         cp->overflow = (int*)(base + o_ovf);
     }
     return L.t;
@@ -1389,7 +1456,7 @@ dem_status dem_coupler_create(dem_ctx* coarse, dem_ctx* fine, const dem_coupling
     // first sample of the coarse positions
     cp->g.call = 0;
     cudaStreamSynchronize(coarse->stream);
-    k_cp_coarse<<<coarse->grid_rb, TILE, 0, s>>>(coarse->dev, cp->g, cp->a, 1);
+    k_cp_coarse<<<coarse->ntiles, TILE, 0, s>>>(coarse->dev, cp->g, cp->a, 1);
     CU(cudaGetLastError());
     CU(cudaStreamSynchronize(s));
     *out = cp;
@@ -1419,11 +1486,12 @@ dem_status dem_couple(dem_coupler* cp)
     g.fresh_c = coarse->fresh ? 1 : 0;
     g.fresh_f = ctx->fresh ? 1 : 0;
     k_cp_clear<<<(clear_threads(g.S, g.C) + 255) / 256, 256, 0, s>>>(g, cp->a);
-    k_cp_coarse<<<coarse->grid_rb, TILE, 0, s>>>(coarse->dev, g, cp->a, 0);
-    k_cp_fine<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, g, cp->a);
+    k_cp_coarse<<<coarse->ntiles, TILE, 0, s>>>(coarse->dev, g, cp->a, 0);
+    k_cp_fine<<<ctx->ntiles, TILE, 0, s>>>(ctx->dev, g, cp->a);
+    k_cp_layer<<<LAYER_BLOCKS, 64, 0, s>>>(coarse->dev, ctx->dev, g, cp->a);
     k_cp_cells<<<(cells_threads(g.S, g.C) + 255) / 256, 256, 0, s>>>(g, cp->a);
-    k_cp_force_fine<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, g, cp->a);
-    k_cp_force_coarse<<<coarse->grid_rb, TILE, 0, s>>>(coarse->dev, g, cp->a);
+    k_cp_force_fine<<<ctx->ntiles, TILE, 0, s>>>(ctx->dev, g, cp->a);
+    k_cp_force_coarse<<<coarse->ntiles, TILE, 0, s>>>(coarse->dev, g, cp->a);
     for (int fk = 0; fk < g.nface; ++fk)
         k_cp_insert<<<g.face[fk].nb * g.face[fk].nc, 32 * INS_WARPS, 0, s>>>(ctx->dev, g, cp->a, fk, cp->rho_f);
     CU(cudaMemsetAsync(cp->overflow, 0, sizeof(int), s));
