@@ -1025,14 +1025,13 @@ __device__ __forceinline__ double root_refined(double s2)
 // The tangential overlaps of up to two segment contacts are kept per particle, tagged with the
 // segment; MODE 0 stores them.
 template <int MODE>
-__device__ __forceinline__ int wall_contacts(const Dev& d, const InstC& c, int kinst, int s, int lp, int4 P, float r,
+__device__ __forceinline__ int wall_contacts(const Dev& d, const InstC& c, const WallGeo& G, int s, int lp, int4 P, float r,
                                              float m, V3 vme, V3 wme, float dt_hist, V3& F, V3& Tq)
 {
     const float exf = (float)(P.x - c.waxi) - c.waxf, eyf = (float)(P.y - c.wayi) - c.wayf, zf = (float)P.z;
     const float rhof = sqrtf(exf * exf + eyf * eyf);
     const float tol = 1e-6f * (rhof + fabsf(zf) + c.wmag) + 4.f;
     const float lim = (float)P.w * (1.f + 1.f / 64.f) + tol;
-    const WallGeo& G = d.wgeo[kinst];
     unsigned nearm = 0u;
     for (int k = 0; k + 1 < c.nwp; ++k) {
         const float r0 = c.wpf[2 * k], z0 = c.wpf[2 * k + 1];
@@ -1216,6 +1215,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
                          : (int)((long long)(blockIdx.x + 1) * NU / gridDim.x);
     const int ncap = d.ncap;
     const size_t plane = (size_t)d.Lmax * ncap;
+    // the walls' constants too in fused steps, whose barriers empty the L1 (trips to L2 in every step)
+    __shared__ WallGeo swg;
     int kprev = FUSED ? kstaged : -1;
     if (FUSED && kprev >= 0) {
         __syncthreads();
@@ -1293,6 +1294,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
             if (threadIdx.x < (int)(sizeof(InstD) / 4))
                 ((int*)&sd)[threadIdx.x] = FUSED ? __ldcg((const int*)(d.id + k) + threadIdx.x)
                                                  : ((const int*)(d.id + k))[threadIdx.x];
+            if (FUSED && WALLS)
+                for (int i = threadIdx.x; i < (int)(sizeof(WallGeo) / 4); i += nthr) ((int*)&swg)[i] = ((const int*)(d.wgeo + k))[i];
             __syncthreads();
             kprev = k;
         }
@@ -1517,7 +1520,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
             }
         }
         int nseg = 0;
-        if (WALLS && c.nwp >= 2) nseg = wall_contacts<MODE>(d, c, kprev, s, lp, P, r, m, vme, wme, dt_hist, F, Tq);
+        if (WALLS && c.nwp >= 2) nseg = wall_contacts<MODE>(d, c, FUSED ? swg : d.wgeo[kprev], s, lp, P, r, m, vme, wme, dt_hist, F, Tq);
         const float inv_m = 1.0f / m;
         const float inv_I = 2.5f / (m * r * r);
         if (!(isfinite(F.x) && isfinite(F.y) && isfinite(F.z) && isfinite(Tq.x) && isfinite(Tq.y) &&
