@@ -266,6 +266,10 @@ __global__ void __launch_bounds__(TILE) k_rb_tilesort(Dev d)
             if (D.flag != 2)
                 kk = (order_contacts(d, D, old) << 8) | (unsigned)min(d.cnt[D.lp][old], 255);
         }
+        if (D.flag == 2) {                  // a written state: no contacts to order by (the whole block's tile)
+            if (valid) d.fin[p] = p;
+            continue;
+        }
         __syncthreads();                    // the previous tile's keys are no longer read
         key[threadIdx.x] = kk;
         __syncthreads();

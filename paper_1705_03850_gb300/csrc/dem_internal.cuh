@@ -253,9 +253,16 @@ struct AdjBufs {
 
 __device__ __forceinline__ int axis_cell(const InstC& c, int a, int x)
 {
+    // floor(x nc / ext) from a float estimate, made exact by 64-bit products (the estimate is off by
+    // one at most; a 64-bit division is some hundred instructions)
+    const int nc = c.nc[a], ext = c.ext[a];
     if (x <= 0) return 0;
-    long long t = (long long)x * c.nc[a] / c.ext[a];
-    return t >= c.nc[a] ? c.nc[a] - 1 : (int)t;
+    if (x >= ext) return nc - 1;
+    const long long p = (long long)x * nc;
+    int t = (int)(__fdividef((float)x, (float)ext) * (float)nc);
+    while ((long long)t * ext > p) --t;
+    while ((long long)(t + 1) * ext <= p) ++t;
+    return t;
 }
 
 __device__ __forceinline__ unsigned cell_code(const Dev& d, const InstC& c, int cx, int cy, int cz)
