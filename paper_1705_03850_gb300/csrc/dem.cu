@@ -2356,16 +2356,18 @@ __global__ void __launch_bounds__(TILE) k_adj_prep(Dev d, AdjBufs a, float kick)
 // Pulls the force adjoints (buffers par) back to x^n, v^{n-1/2}, w^{n-1/2}, xi^{n-1} and (E, e, mu),
 // then takes this particle one step further back (kick_next, its step's kick in dt): the drift and
 // the force adjoints of step n - 1 go to the other pair of buffers, so that the reverse step is one
-// kernel.  tmask: the contacts of x^n, which the forward step left in the mask of x^{n+1}
-// (nullptr: found from the positions, at the last step).
+// kernel.  tmask: the contacts of x^n, which the forward step left in the mask of x^{n+1}.
 // Bound by the latency of the gathers of a contact's five neighbour records: 154 registers leave 12
 // warps an SM.  So the next contact's records are copied asynchronously into shared memory while
 // one is evaluated, blocks are single warps (a 32-slot slice each, in the order of contact counts:
 // persistent blocks left the last of eight rounds nearly empty), and a rollout orders the slots by
 // contact count first (14 of 32 lanes were active without).  64 columns of 10,000 spheres, 100
-// steps forward and back: 31.3 ms against 37.4 ms without these (148 against about 180 us a reverse
-// step); 37.0 ms with the ordering alone, 32.1 ms at 128 registers (16 warps, 48 bytes spilled).
-__global__ void __launch_bounds__(32, 12) k_adj_force(Dev d, AdjBufs a, Snap S, const unsigned* __restrict__ tmask, int prime,
+// steps forward and back: 31.3 ms against 37.4 ms without these, 37.0 ms with the ordering alone.
+// LAST: the evaluation at the last step, with the search for contacts.  WARPS: 16 a SM (127 registers)
+// where the slices are more than 12 a SM hold at once, 30.5 against 31.2 ms; below that 12, as a
+// slice alone takes longer with fewer registers (4 columns of 1,003 spheres 2.36 against 2.46 ms).
+template <bool LAST, int WARPS>
+__global__ void __launch_bounds__(32, WARPS) k_adj_force(Dev d, AdjBufs a, Snap S, const unsigned* __restrict__ tmask, int prime,
                                                     int par, float kick_next)
 {
     const size_t plane = (size_t)d.Lmax * d.ncap;
@@ -2400,8 +2402,8 @@ __global__ void __launch_bounds__(32, 12) k_adj_force(Dev d, AdjBufs a, Snap S, 
         const int per0 = c.per[0], per1 = c.per[1], ext0 = c.ext[0], ext1 = c.ext[1], hf0 = c.half[0],
                   hf1 = c.half[1];
         // pass 1 (the last step only): which entries touch (independent loads, four at a time)
-        unsigned tm = tmask ? tmask[s] : 0u;
-        for (int e0 = tmask ? ncnt : 0; e0 < ncnt; e0 += 4) {
+        unsigned tm = LAST ? 0u : tmask[s];
+        for (int e0 = 0; LAST && e0 < ncnt; e0 += 4) {
             int jb[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) jb[k] = e0 + k < ncnt ? __ldg(nb + (size_t)(e0 + k) * ncap) : s;
@@ -4222,8 +4224,11 @@ dem_status dem_rollout_adjoint(dem_ctx* ctx, const double* weights, const double
     auto prime_at = [&](long long t) { return t == 0 && ro.prime0; };
     auto kick_at = [&](long long t) { return prime_at(t) ? 0.5f : 1.0f; };
     int par = 0;
+    int nsm = 0;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device);
+    auto adj = 4 * ctx->ntiles > 12 * nsm ? k_adj_force<false, 16> : k_adj_force<false, 12>;
     k_adj_prep<<<ctx->grid_rb, TILE, 0, s>>>(ctx->dev, ro.a, 0.5f);
-    k_adj_force<<<4 * ctx->ntiles, 32, 0, s>>>(ctx->dev, ro.a, ro.ck[ro.ncp - 1], nullptr, 0, par, kick_at(N - 1));
+    k_adj_force<true, 12><<<4 * ctx->ntiles, 32, 0, s>>>(ctx->dev, ro.a, ro.ck[ro.ncp - 1], nullptr, 0, par, kick_at(N - 1));
     CU(cudaGetLastError());
     for (int c = ro.ncp - 2; c >= 0; --c) {
         const long long s0 = (long long)c * K, s1 = std::min(s0 + K, N);
@@ -4234,8 +4239,8 @@ dem_status dem_rollout_adjoint(dem_ctx* ctx, const double* weights, const double
             if ((st = step_between(ctx, at(t), at(t + 1), prime_at(t) ? 1 : 0))) return st;
         for (long long t = s1 - 1; t >= s0; --t) {
             par ^= 1;
-            k_adj_force<<<4 * ctx->ntiles, 32, 0, s>>>(ctx->dev, ro.a, at(t), at(t + 1).hmask, prime_at(t) ? 1 : 0, par,
-                                                       t > 0 ? kick_at(t - 1) : 0.0f);
+            adj<<<4 * ctx->ntiles, 32, 0, s>>>(ctx->dev, ro.a, at(t), at(t + 1).hmask, prime_at(t) ? 1 : 0, par,
+                                               t > 0 ? kick_at(t - 1) : 0.0f);
             CU(cudaGetLastError());
         }
     }
