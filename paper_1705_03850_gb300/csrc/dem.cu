@@ -419,7 +419,7 @@ __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, co
                                         Get get)
 {
     const int cur = D.cur, nxt = cur ^ 1, lp = D.lp, nlp = lp ^ 1;
-    const int ncap = d.ncap;
+    const int ncap = d.ncap, Lmax = d.Lmax;
     const bool fresh = D.flag == 2;          // a written state: no histories
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     const int ocnt = fresh ? 0 : d.cnt[lp][old];
@@ -477,7 +477,7 @@ __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, co
     }
 #pragma unroll
     for (int i = 0; i < N; ++i)
-        if (m[i] != ps) nrow[(size_t)r[i] * ncap] = d.fin[m[i]];
+        if (m[i] != ps && r[i] < Lmax) nrow[(size_t)r[i] * ncap] = d.fin[m[i]];
     if (overflow) {
         atomicOr(&d.g->status, ST_CAPACITY);
         d.g->err_slot = s;
@@ -488,7 +488,7 @@ __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, co
     const int* orow = d.nbr[lp] + old;
     const float* ho = d.hist[lp] + old;
     float* hn = d.hist[nlp] + s;
-    const size_t plane = (size_t)d.Lmax * ncap;
+    const size_t plane = (size_t)Lmax * ncap;
     if (ocnt < 32) ohm &= (1u << ocnt) - 1u;
     unsigned nhm = 0u;
     while (ohm) {
@@ -517,7 +517,7 @@ __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, co
 #pragma unroll
             for (int i = 0; i < N; ++i)
                 if (id[i] == oid[k]) re = r[i];
-            if (re >= 0) {
+            if (re >= 0 && re < Lmax) {
                 float* x = hn + (size_t)re * ncap;
                 x[0] = h[k][0];
                 x[plane] = h[k][1];
@@ -536,7 +536,7 @@ __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, co
     d.vel[nxt][s] = v;
     d.omg[nxt][s] = w;
     d.slot_of_id[c.slot0 + (int)myid] = s;
-    d.cnt[nlp][s] = nc;
+    d.cnt[nlp][s] = min(nc, Lmax);           // (one more can be listed where the row overflows)
     d.hmask[nlp][s] = nhm;
     if (D.fext) d.fext[nlp][s] = d.fext[lp][old];      // held until overwritten, even across state writes
     d.whist[nlp][s] = wh;
@@ -2947,20 +2947,35 @@ dem_status launch_rebuild(dem_ctx* ctx, cudaStream_t st)
     return DEM_OK;
 }
 
+// whether the caller is capturing the context's stream (noted: its replays then change the state
+// without a call, so nothing the host knows of the lists can be relied on any more)
+bool capturing(dem_ctx* ctx)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess) {
+        cudaGetLastError();              // the legacy stream, while another captures
+        return false;
+    }
+    if (st != cudaStreamCaptureStatusNone) ctx->captured = true;
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // Lists valid for the current state, on the context's stream: nothing to do when nothing ran since
-// the last build that could ask for one; the chain when a state was written; otherwise the chain
-// behind one condition, where a graph holds it (one launch instead of eleven kernels that find
-// nothing to do), else the chain.
+// the last build that could ask for one; the chain when a state was written, or into a capture of the
+// caller's; otherwise the chain behind one condition, where a graph holds it (one launch instead of
+// nine kernels that find nothing to do), else the chain.
 dem_status ensure_lists(dem_ctx* ctx)
 {
-    if (ctx->lists_ok) return DEM_OK;
-    if (ctx->rb_if && !ctx->must_build) {
+    const bool cap = capturing(ctx);
+    if (ctx->lists_ok && !ctx->captured) return DEM_OK;
+    if (ctx->rb_if && !ctx->must_build && !cap) {
         CU(cudaGraphLaunch(ctx->rb_if, ctx->stream));
     } else {
         dem_status st = launch_rebuild(ctx, ctx->stream);
         if (st) return st;
-        if (ctx->must_build) ctx->written = true;
+        if (ctx->must_build) ctx->written = !ctx->captured;
     }
+    if (cap) return DEM_OK;
     ctx->lists_ok = true;
     ctx->must_build = false;
     return DEM_OK;
@@ -2972,7 +2987,7 @@ dem_status ensure_lists(dem_ctx* ctx)
 // same rows, for callers with enough steps ahead; results do not depend on the slots' order.
 dem_status order_slots(dem_ctx* ctx)
 {
-    if (!ctx->written) return DEM_OK;
+    if (!ctx->written || ctx->captured) return DEM_OK;
     ctx->written = false;
     k_touch<<<ctx->grid_rb, TILE, 0, ctx->stream>>>(ctx->dev);
     k_mark_order<<<1, 256, 0, ctx->stream>>>(ctx->dev);
@@ -3695,13 +3710,16 @@ dem_status dem_step(dem_ctx* ctx, int64_t nsteps)
     if (ctx->status) return check_status(ctx);
     if (!ctx->have_state) return fail(ctx, DEM_ERR_STATE, "write the state before stepping");
     int64_t done = 0;
+    const bool cap = capturing(ctx);
     while (done < nsteps) {
         // the graph, also for a remainder of at least 1/GRAPH_PART of its steps (the step kernels
         // beyond it find none left and end at once, about 4 us each with their share of the graph's
         // other nodes, where a step launched alone comes with the eleven kernels of the rebuild
         // chain, 25 us); fused steps run any number
         const int64_t left = nsteps - done;
-        if (!ctx->fresh && ctx->gexec && (ctx->graph_fused || left * GRAPH_PART >= ctx->graph_steps)) {
+        // (a remainder inside a capture of the caller's is launched step by step)
+        if (!ctx->fresh && ctx->gexec &&
+            (left >= ctx->graph_steps || (!cap && (ctx->graph_fused || left * GRAPH_PART >= ctx->graph_steps)))) {
             const int64_t now = std::min<int64_t>(left, ctx->graph_steps);
             if (now < ctx->graph_steps) k_set_todo<<<1, 1, 0, ctx->stream>>>(ctx->dev, (long long)now);
             CU(cudaGraphLaunch(ctx->gexec, ctx->stream));
@@ -3712,7 +3730,7 @@ dem_status dem_step(dem_ctx* ctx, int64_t nsteps)
         }
         dem_status st = ensure_lists(ctx);
         if (st) return st;
-        if (left >= ORDER_STEPS && !ctx->graph_fused && (st = order_slots(ctx))) return st;
+        if (left >= ORDER_STEPS && !ctx->graph_fused && !cap && (st = order_slots(ctx))) return st;
         st = launch_step(ctx, ctx->fresh ? 1 : 0);
         if (st) return st;
         ctx->written = false;

@@ -49,6 +49,7 @@ struct dem_ctx {
     bool lists_ok = false;
     bool must_build = true;
     bool written = false;             // lists built for a written state, nothing but reads since
+    bool captured = false;            // the caller captured calls: its replays change the state unseen
     long long steps = 0;
     unsigned status = 0;
     std::string err;
@@ -60,7 +61,7 @@ struct dem_ctx {
     int fused_threads = 0, fused_blocks = 0;   // its launch in the current graph
     cudaGraph_t rb_graph = nullptr;
     cudaGraph_t rb_if_graph = nullptr;   // the rebuild chain behind one condition, for calls that need valid
-    cudaGraphExec_t rb_if = nullptr;     // lists (reads, coupling): a launch instead of the chain's eleven
+    cudaGraphExec_t rb_if = nullptr;     // lists (reads, coupling): a launch instead of the chain's nine
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     std::vector<cudaEvent_t> ev0, ev1;   // around every EV_EVERY-th step kernel of the graph
