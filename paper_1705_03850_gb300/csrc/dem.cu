@@ -3714,8 +3714,8 @@ dem_status dem_step(dem_ctx* ctx, int64_t nsteps)
     while (done < nsteps) {
         // the graph, also for a remainder of at least 1/GRAPH_PART of its steps (the step kernels
         // beyond it find none left and end at once, about 4 us each with their share of the graph's
-        // other nodes, where a step launched alone comes with the eleven kernels of the rebuild
-        // chain, 25 us); fused steps run any number
+        // other nodes, where a step launched alone comes with the nine kernels of the rebuild
+        // chain, 20 us or more); fused steps run any number
         const int64_t left = nsteps - done;
         // (a remainder inside a capture of the caller's is launched step by step)
         if (!ctx->fresh && ctx->gexec &&
