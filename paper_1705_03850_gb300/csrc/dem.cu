@@ -2242,69 +2242,16 @@ __device__ __forceinline__ void for_live_slots(const Dev& d, Fn fn)
 }
 
 // the same by slices of 32 slots, for blocks of one warp
-template <typename Slot, typename Fn>
-__device__ __forceinline__ void for_live_slices(const Dev& d, Slot slot, Fn fn)
+template <typename Fn>
+__device__ __forceinline__ void for_live_slices(const Dev& d, Fn fn)
 {
     for (int u = blockIdx.x; u < 4 * d.ntiles; u += gridDim.x) {
         const int k = d.tile_inst[u >> 2];
         const InstD D = d.id[k];
-        const int s = slot(u, d.ic[k].slot0 + D.n);
+        const int s = u * 32 + threadIdx.x;
         if (s - d.ic[k].slot0 >= D.n) continue;
         fn(s, k, D);
     }
-}
-
-// The slot of this lane when the 128 slots of slice u's tile are dealt to its four slices by the
-// number of bits of mask, most first, equal ones in slot order; slots from `end` on come last, their
-// masks unread.  Each of the four slices ranks the whole tile by itself (a warp, four slots a lane:
-// per group of 32 the lanes of equal count, then a scan over the counts), so they need not meet.
-// tmp: 160 ints of shared memory, free for other use on return.
-__device__ __forceinline__ int ranked_slot(const unsigned* __restrict__ mask, int u, int end, int* tmp)
-{
-    const unsigned full = 0xffffffffu;
-    const int lane = (int)threadIdx.x, base = (u & ~3) * 32;
-    int key[4], rank[4];
-    __syncwarp();                        // a slice before this one is done with tmp
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const int i = base + 32 * v + lane;
-        key[v] = i < end ? min(__popc(mask[i]), 30) + 1 : 0;     // 0..31
-        tmp[32 * v + lane] = 0;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const unsigned same = __match_any_sync(full, key[v]);
-        rank[v] = __popc(same & ((1u << lane) - 1u));
-        if (rank[v] == 0) tmp[32 * v + key[v]] = __popc(same);
-    }
-    __syncwarp();
-    // lane L: the places of count L, after those of all larger counts
-    int n[4], at = 0;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) at += n[v] = tmp[32 * v + lane];
-    const int own = at;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int up = __shfl_down_sync(full, at, o);
-        if (lane + o < 32) at += up;
-    }
-    at -= own;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        tmp[32 * v + lane] = at;
-        at += n[v];
-    }
-    __syncwarp();
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const int place = tmp[32 * v + key[v]] + rank[v];
-        if ((place >> 5) == (u & 3)) tmp[128 + (place & 31)] = base + 32 * v + lane;
-    }
-    __syncwarp();
-    const int s = tmp[128 + lane];
-    __syncwarp();                        // read before the caller writes there
-    return s;
 }
 
 template <bool SAVE>
@@ -2419,29 +2366,19 @@ __global__ void __launch_bounds__(TILE) k_adj_prep(Dev d, AdjBufs a, float kick)
 // LAST: the evaluation at the last step, with the search for contacts.  WARPS: 16 a SM (127 registers)
 // where the slices are more than 12 a SM hold at once, 30.5 against 31.2 ms; below that 12, as a
 // slice alone takes longer with fewer registers (4 columns of 1,003 spheres 2.36 against 2.46 ms).
-// There the slots of a tile are also dealt to its slices by this step's contacts (ranked_slot): those
-// of jostling spheres change from step to step, and with the order of the rollout's start 18 of 32
-// lanes were active (slices of 3.5 contacts a slot, but 6.1 in their longest), with this one 24.  The
-// first two arguments stay in constant memory (__grid_constant__): the lists' buffers, chosen by
-// parity, were copied to each thread's stack otherwise.  Both together 30.4 -> 29.1 ms (the ranking
-// alone 30.1, the arguments alone 29.9).  Small contexts keep the order: no slice waits for a place.
 template <bool LAST, int WARPS>
-__global__ void __launch_bounds__(32, WARPS) k_adj_force(const __grid_constant__ Dev d, const __grid_constant__ AdjBufs a,
-                                                    Snap S, const unsigned* __restrict__ tmask, int prime,
+__global__ void __launch_bounds__(32, WARPS) k_adj_force(Dev d, AdjBufs a, Snap S, const unsigned* __restrict__ tmask, int prime,
                                                     int par, float kick_next)
 {
     const size_t plane = (size_t)d.Lmax * d.ncap;
     const int ncap = d.ncap;
     // a block of one warp per 32-slot slice: the slices' contact counts differ, and what is resident
     // is limited by registers, so blocks of one warp that come and go by themselves fill the SMs
-    __shared__ float4 stg[2][5][32];           // the next contact's position, velocity, spin, force adjoints,
-    __shared__ float stx[2][6][32];            // overlap and overlap adjoint
-    auto slot = [&](int u, int end) {
-        return WARPS == 16 && !LAST ? ranked_slot(tmask, u, end, (int*)&stx[0][0][0]) : u * 32 + (int)threadIdx.x;
-    };
-    for_live_slices(d, slot, [&](int s, int k, const InstD& D) {
+    for_live_slices(d, [&](int s, int k, const InstD& D) {
         const InstC& c = d.ic[k];
         const int lane = (int)threadIdx.x;
+        __shared__ float4 stg[2][5][32];       // the next contact's position, velocity, spin, force adjoints,
+        __shared__ float stx[2][6][32];        // overlap and overlap adjoint
         const Coef<float> cf = coef_of(c);
         const int lp = D.lp;
         const float q = c.q;

@@ -20,18 +20,3 @@ def test_gradients_do_not_depend_on_the_variant(every):
     assert np.isfinite(out[0]).all() and (out[0] != 0).all()
     # the same float arithmetic; the sums over particles are in double, in the order of the slots
     np.testing.assert_allclose(out[1], out[0], rtol=1e-12)
-
-
-@pytest.mark.parametrize("shape", [(5, 4, 4), (5, 5, 5), (8, 4, 4), (13, 9, 11)])
-def test_slots_ranked_by_contacts_cover_ragged_tiles(shape):
-    """The variant for large contexts deals a tile's slots to its four slices by their contacts:
-    tiles with dead slots (80, 125 and 1287 particles) and a full one (128)."""
-    wl = workloads.dense_block(*shape, seed=96, squeeze=2e-4, vel=0.05)
-    out = []
-    for capacity in (wl.n, 80_000):
-        sim = dem.from_workload(wl, max_neighbors=16, capacity=capacity)
-        sim.rollout_forward(7, 3)
-        out.append(sim.rollout_adjoint(np.ones((1, 2)), np.array([[0.0, 0.0]])))
-    assert np.isfinite(out[0]).all() and (out[0] != 0).all()
-    # the same float arithmetic; the sums over particles are in double, in the order of the slots
-    np.testing.assert_allclose(out[1], out[0], rtol=1e-12)
