@@ -2366,8 +2366,14 @@ __global__ void __launch_bounds__(TILE) k_adj_prep(Dev d, AdjBufs a, float kick)
 // LAST: the evaluation at the last step, with the search for contacts.  WARPS: 16 a SM (127 registers)
 // where the slices are more than 12 a SM hold at once, 30.5 against 31.2 ms; below that 12, as a
 // slice alone takes longer with fewer registers (4 columns of 1,003 spheres 2.36 against 2.46 ms).
+// The structures stay in constant memory (__grid_constant__): the buffers chosen by parity were
+// copied to every thread's stack otherwise (88 bytes), 30.4 -> 30.0 ms.  18 of 32 lanes are active,
+// as contacts change from step to step; ranking a tile's slots anew by each step's contacts made
+// 24 of it, 29.1 ms, but cost 8 % where spheres have few contacts.
 template <bool LAST, int WARPS>
-__global__ void __launch_bounds__(32, WARPS) k_adj_force(Dev d, AdjBufs a, Snap S, const unsigned* __restrict__ tmask, int prime,
+__global__ void __launch_bounds__(32, WARPS) k_adj_force(const __grid_constant__ Dev d, const __grid_constant__ AdjBufs a,
+                                                    const __grid_constant__ Snap S,
+                                                    const unsigned* __restrict__ tmask, int prime,
                                                     int par, float kick_next)
 {
     const size_t plane = (size_t)d.Lmax * d.ncap;
