@@ -1193,7 +1193,7 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
     constexpr bool SMW = BS == SMW_BS;       // single instance, slices claimed from a shared counter
     static_assert(!SMW || (LPP == 1 && !FUSED), "SM-wide blocks: one lane per particle, per-step launches");
     static_assert(LPP == 1 || LPP == 2 || LPP == 4 || LPP == 8, "1, 2, 4 or 8 lanes per particle");
-    static_assert(LPP == 1 || MODE == 0, "several lanes per particle only for the step");
+    static_assert(LPP == 1 || MODE != 1, "several lanes per particle only for steps");
     static_assert(MODE != 2 || (!WALLS && !FUSED), "rollouts have no walls and are not fused");
     static_assert((WPT & (WPT - 1)) == 0, "warps per tile must be a power of two");
     // entries of a lane's share of a row: bits e with e mod LPP == sub
@@ -4027,7 +4027,9 @@ dem_status step_once(dem_ctx* ctx, int prime)
     return DEM_OK;
 }
 
-// one step from the saved state A to B's buffers (lists frozen)
+// one step from the saved state A to B's buffers (lists frozen), with the lanes per particle that the
+// forward steps had: they decide the order of a particle's sums, and the recomputed states have to be
+// the forward ones bit for bit (the reverse step takes its contacts from the forward steps' masks)
 dem_status step_between(dem_ctx* ctx, const Snap& A, const Snap& B, int prime)
 {
     Dev d = ctx->dev;
@@ -4040,7 +4042,13 @@ dem_status step_between(dem_ctx* ctx, const Snap& A, const Snap& B, int prime)
         d.hmask[i] = S[i]->hmask;
         d.whist[i] = S[i]->whist;
     }
-    k_step<2, false><<<ctx->grid_bs[1], TILE, 0, ctx->stream>>>(d, prime, StepCtl{});
+    const StepCtl ctl{};
+    switch (ctx->ro.lanes) {
+    case 2: k_step<2, false, TILE, 2><<<ctx->grid_lanes[0], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+    case 4: k_step<2, false, TILE, 4><<<ctx->grid_lanes[1], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+    case 8: k_step<2, false, TILE, 8><<<ctx->grid_lanes[2], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+    default: k_step<2, false><<<ctx->grid_bs[1], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+    }
     CU(cudaGetLastError());
     return DEM_OK;
 }
@@ -4184,6 +4192,7 @@ dem_status dem_rollout_forward(dem_ctx* ctx, int64_t nsteps, int64_t checkpoint_
     ro.K = checkpoint_every;
     ro.ncp = (int)ro.ck.size();
     ro.prime0 = ctx->fresh;
+    ro.lanes = ctx->step_lanes;
     dem_status st = ensure_lists(ctx);                      // the lists the whole rollout uses
     if (st) return st;
     if (nsteps >= ORDER_ROLLOUT && (st = order_slots(ctx))) return st;

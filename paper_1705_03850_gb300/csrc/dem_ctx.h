@@ -73,6 +73,7 @@ struct dem_ctx {
         long long nsteps = 0, K = 0;
         int ncp = 0;
         bool prime0 = false;
+        int lanes = 1;                   // lanes per particle of the forward steps
         std::vector<Snap> ck, seg;       // checkpoints (every K steps and the end), segment steps
         AdjBufs a{};
     } ro;
