@@ -1356,12 +1356,16 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         jn3 = sub + 3 * LPP < ncnt ? jn3 : s;
         // removed below the removal height: parked until the next list build drops it (tested
         // here, after the row's first loads are in flight, so that live rows do not wait on it)
-        if (MODE != 2 && (idw & GONE_BIT)) {
-            if (MODE == 0 && sub == 0) {
+        if (idw & GONE_BIT) {
+            if (MODE != 1 && sub == 0) {
                 d.pos[cur ^ 1][s] = P;
                 d.vel[cur ^ 1][s] = Vv;
                 d.omg[cur ^ 1][s] = Wv;
-            } else {
+                if (MODE == 2) {
+                    d.hmask[hout][s] = 0u;
+                    d.whist[hout][s] = d.whist[hin][s];
+                }
+            } else if (MODE != 2) {
                 d.outWX[s] = make_float4(0.f, 0.f, 0.f, 0.f);
                 d.cmask[s] = 0ull;
             }
@@ -2265,10 +2269,13 @@ __global__ void __launch_bounds__(TILE) k_snap(Dev d, Snap S)
         float* h = d.hist[lp] + s;
         float* hs = S.hist + s;
         if (SAVE) {
+            const float4 v = d.vel[cur][s];
             S.pos[s] = d.pos[cur][s];
-            S.vel[s] = d.vel[cur][s];
+            S.vel[s] = v;
             S.omg[s] = d.omg[cur][s];
-            unsigned hm = d.hmask[lp][s];
+            // (a removed particle, parked until the next list build, keeps the mask of its last step: it has
+            // no contacts, and the reverse step takes those of the step before from this mask)
+            unsigned hm = (__float_as_uint(v.w) & GONE_BIT) ? 0u : d.hmask[lp][s];
             S.hmask[s] = hm;
             S.whist[s] = d.whist[lp][s];
             while (hm) {
