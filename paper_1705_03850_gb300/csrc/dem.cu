@@ -727,11 +727,14 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
                         bool hit[4];
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            const int dx = p.x - q[u].x, dy = p.y - q[u].y, dz = p.z - q[u].z;
+                            const int dx = p.x - q[u].x, dy = p.y - q[u].y;
+                            // z reaches +-2e9 units, outside the box too: |dz| in 32 bits without sign, cut off
+                            // where it is beyond any cut
+                            const unsigned dz = min(__sad(p.z, q[u].z, 0u), 0x7fffffffu);
                             const int cut = cut0 + q[u].w;
                             const unsigned long long d2 = (unsigned long long)((long long)dx * dx) +
                                                           (unsigned long long)((long long)dy * dy) +
-                                                          (unsigned long long)((long long)dz * dz);
+                                                          (unsigned long long)dz * dz;
                             hit[u] = t + u < t1 && d2 < (unsigned long long)((long long)cut * cut);
                         }
 #pragma unroll
