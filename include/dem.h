@@ -256,6 +256,10 @@ dem_status dem_set_list_build(dem_ctx *ctx, int32_t staged);
  * fused steps.  Not in the paper. */
 dem_status dem_test_stall_barrier(dem_ctx *ctx);
 
+/* For tests of the fused steps' barrier in long runs: its step tag becomes `tag`, as after that many
+ * fused steps of a single-instance context.  Results do not depend on it. */
+dem_status dem_test_barrier_tag(dem_ctx *ctx, uint32_t tag);
+
 /* CUDA-event time of step kernels of the most recent graph launch: every fifth
  * step kernel of the graph (the first, the sixth, ... that its steps reach) is bracketed by event
  * nodes; total_ms = the sum over those, count = their number (total_ms / count is

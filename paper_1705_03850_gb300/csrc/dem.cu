@@ -1737,7 +1737,8 @@ __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int 
 // What bounds it is the chain of dependent round trips to L2 of one step, so:
 // - single instance: each block folds {step tag, its largest displacement} into one word and adds
 //   itself to a count; once the count is full every block reads the word, advances the
-//   displacement bound and decides on the list build alike.  (Tags grow, so nothing is reset; the
+//   displacement bound and decides on the list build alike.  (Tags grow within a graph launch, whose
+//   start resets them: a tag that wrapped would leave the maxima of before in the words.  The
 //   words alternate by the tag's parity, as a block can be one step ahead, never two.)  With
 //   several instances the last block to arrive ends the step for each and releases the others.
 // - the barrier's cost is its fences and the arrivals at one word: one release and one acquire per
@@ -1936,6 +1937,9 @@ __global__ void k_steps_init(Dev d, long long S, cudaGraphConditionalHandle h_rb
     const long long t = d.g->todo > 0 ? d.g->todo : S;
     d.g->todo = 0;
     d.g->remain = t;
+    // the fused steps' barrier starts anew: its tag counts the steps of one graph launch
+    d.g->bar_gen = d.g->bar_count = 0u;
+    for (int i = 0; i < 3; ++i) d.bar[i * BAR_LINE] = 0ull;
     cudaGraphSetConditional(h_rb, d.g->any ? 1u : 0u);
     if (set_loop) cudaGraphSetConditional(h_loop, t > 0 ? 1u : 0u);
 }
@@ -3521,7 +3525,6 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
     CUC(cudaMemsetAsync(d.hist[0], 0, (size_t)p.ncap * p.Lmax * 12, s));
     CUC(cudaMemsetAsync(d.hist[1], 0, (size_t)p.ncap * p.Lmax * 12, s));
     CUC(cudaMemsetAsync(d.ccount, 0, (size_t)p.ncodes * 4, s));   // every build leaves the counts zero
-    CUC(cudaMemsetAsync(d.bar, 0, sizeof(unsigned long long) * 3 * BAR_LINE, s));
     CUC(cudaMemsetAsync(d.wrem, 0, sizeof(double) * 2 * p.B, s));
     k_init_ids<<<nblk(p.ncap, 256), 256, 0, s>>>(d);
     CUC(cudaGetLastError());
@@ -3845,6 +3848,17 @@ dem_status dem_test_stall_barrier(dem_ctx* ctx)
     if (!ctx) return DEM_ERR_ARG;
     static const unsigned one = 1u;
     CU(cudaMemcpyAsync(&ctx->dev.g->test_stall, &one, sizeof(unsigned), cudaMemcpyHostToDevice, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    return DEM_OK;
+}
+
+dem_status dem_test_barrier_tag(dem_ctx* ctx, uint32_t tag)
+{
+    if (!ctx) return DEM_ERR_ARG;
+    const unsigned long long word = (unsigned long long)tag << 32;
+    CU(cudaMemcpyAsync(&ctx->dev.g->bar_gen, &tag, sizeof tag, cudaMemcpyHostToDevice, ctx->stream));
+    for (int i = 0; i < 2; ++i)
+        CU(cudaMemcpyAsync(ctx->dev.bar + i * BAR_LINE, &word, sizeof word, cudaMemcpyHostToDevice, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
     return DEM_OK;
 }

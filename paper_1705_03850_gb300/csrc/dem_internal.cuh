@@ -145,8 +145,8 @@ struct Glob {
     int err_site;              // (1 cell code, 2 cell range of the list build; 3 touch pass,
     int err_pad;               //  4 contact pass of the step kernel)
     unsigned bar_gen;          // fused steps: grid-barrier generation (bumped by each release); with a single
-                               // instance the tag of the last step's maximum
-    unsigned bar_count;        // fused steps of a single instance: the barrier's arrivals so far
+                               // instance the tag of the last step's maximum; 0 at the start of a graph launch
+    unsigned bar_count;        // fused steps of a single instance: the barrier's arrivals in this graph launch
     long long remain;          // steps still to do in the current graph launch
     long long todo;            // steps of the next graph launch (0: as many as the graph was built for)
     int nlive;                 // entries of live_tiles

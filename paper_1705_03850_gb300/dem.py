@@ -110,6 +110,7 @@ def lib():
         "dem_set_step_lanes": [vp, i32],
         "dem_set_graph_mode": [vp, i32],
         "dem_test_stall_barrier": [vp],
+        "dem_test_barrier_tag": [vp, ctypes.c_uint32],
         "dem_set_list_build": [vp, i32],
         "dem_graph_step_kernel_ms": [vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(i32)],
         "dem_rollout_workspace": [vp, i64, i64, ctypes.POINTER(i64)],
@@ -144,7 +145,7 @@ def lib():
 def exported_symbols():
     return ["dem_query_workspace", "dem_create", "dem_destroy", "dem_write", "dem_read", "dem_read_contacts", "dem_read_neighbors",
             "dem_write_contacts", "dem_step", "dem_sync_status", "dem_instance_info_get", "dem_stats",
-            "dem_set_graph", "dem_set_step_block", "dem_set_step_lanes", "dem_set_graph_mode", "dem_test_stall_barrier", "dem_set_list_build", "dem_graph_step_kernel_ms", "dem_neighbor_counts_noalloc", "dem_rollout_workspace",
+            "dem_set_graph", "dem_set_step_block", "dem_set_step_lanes", "dem_set_graph_mode", "dem_test_stall_barrier", "dem_test_barrier_tag", "dem_set_list_build", "dem_graph_step_kernel_ms", "dem_neighbor_counts_noalloc", "dem_rollout_workspace",
             "dem_rollout_forward", "dem_rollout_adjoint", "dem_observables", "dem_set_material",
             "dem_coupler_workspace", "dem_coupler_create", "dem_couple", "dem_coupler_read", "dem_coupler_destroy",
             "dem_counts", "dem_clear_external_force", "dem_grid_fields", "dem_set_walls", "dem_wall_removed",
@@ -335,6 +336,11 @@ class DEM:
     def test_stall_barrier(self):
         """Make the next fused launch's barrier wait run out (tests of DEM_ERR_TIMEOUT)."""
         self._check(self.L.dem_test_stall_barrier(self.h), "test stall barrier")
+        return self
+
+    def test_barrier_tag(self, tag):
+        """Set the fused steps' barrier tag, as after `tag` fused steps (tests of long runs)."""
+        self._check(self.L.dem_test_barrier_tag(self.h, int(tag)), "test barrier tag")
         return self
 
     def graph_step_kernel_ms(self):
