@@ -3052,6 +3052,7 @@ void destroy_graph(dem_ctx* ctx)
     ctx->rb_if = nullptr;
     ctx->rb_if_graph = nullptr;
     ctx->last_graph_steps = 0;
+    ctx->graph_fused = false;
     ctx->graph = nullptr;
     ctx->rb_graph = nullptr;
 }
@@ -3187,7 +3188,10 @@ dem_status build_fused_graph(dem_ctx* ctx, cudaGraph_t g, int S)
 dem_status build_graph(dem_ctx* ctx, int S)
 {
     destroy_graph(ctx);
-    if (S <= 0) return DEM_OK;
+    if (S <= 0) {
+        ctx->graph_steps = 0;            // a setting changed later does not bring the graph back
+        return DEM_OK;
+    }
     // the rebuild chain, captured once
     cudaStream_t cs;
     CU(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
