@@ -128,7 +128,8 @@ typedef struct {
     int64_t contacts;        /* contacts (particle pairs counted from both sides + floor) at that call */
     int64_t particles;       /* live particles */
     int64_t wall_contacts;   /* floor contacts among `contacts` */
-    int32_t step_threads;    /* threads per block of the step kernel in use (dem_set_step_block) */
+    int32_t step_threads;    /* the step block in effect (dem_set_step_block): threads per block of the step
+                                kernel; 128 with fused steps, whose launches size their own blocks */
     int32_t step_lanes;      /* lanes per particle of the step kernel (dem_set_step_lanes) */
     int32_t graph_fused;     /* 1: the captured graph runs fused steps (dem_set_graph_mode) */
     int32_t reserved;
@@ -226,15 +227,19 @@ dem_status dem_set_step_lanes(dem_ctx *ctx, int32_t lanes);
 /* How a captured graph (dem_set_graph) runs its steps.  1: one step-kernel launch per step,
  * with a conditional list-build node before every fifth (a kernel that finds a list build
  * due leaves its step to the loop at the graph's end).  2: fused steps: one cooperative launch
- * (one block per 128-slot tile, or as many blocks as are resident at once, each walking a
- * range of tiles) runs every step up to the next list build, with a grid barrier
- * between steps (the last block to arrive ends the step for every instance); the graph loops
- * (a conditional while node) over list build + fused launch until its steps are done.  Each
- * step computes exactly what the per-step kernel computes (the same bits); fused steps save
- * the per-step launch and node latency of systems too small to fill the GPU.  Needs one lane
- * per particle and 128-thread blocks (DEM_ERR_STATE otherwise; the previous graph is kept).
- * 0 (the default): fused when those hold and a block for every 128-slot tile holding live
- * particles is resident at once, else one launch per step.  A barrier wait that does not end within about a second reports
+ * runs every step up to the next list build, with a grid barrier between steps; the graph loops
+ * (a conditional while node) over list build + fused launch until its steps are done.  A single
+ * instance runs one block per SM, of the 64 to 640 threads that spread its rows over the SMs,
+ * which deal the 32-row slices out in turn; at the barrier every block reads the step's largest
+ * displacement and decides on the list build alike.  Several instances run 128-thread blocks,
+ * as many as are resident at once or as their slices fill, each walking a range of tiles; the
+ * last block to arrive ends the step for every instance.  Each step computes exactly what the
+ * per-step kernel computes with the same lanes per particle (the same bits); fused steps save
+ * the per-step launch and node latency of systems too small to fill the GPU.  Any number of
+ * lanes per particle; a step block other than 0 or 128 threads is DEM_ERR_STATE (the previous
+ * graph is kept).  0 (the default): fused when the block allows it and a 128-thread block for
+ * every 128 / lanes slots of the tiles holding live particles is resident at once, else one
+ * launch per step.  A barrier wait that does not end within about a second reports
  * DEM_ERR_TIMEOUT.  With fused steps dem_graph_step_kernel_ms times the whole graph launch
  * (list builds included) and counts its steps.  Not in the paper: a scheduling choice of this
  * implementation. */

@@ -3798,7 +3798,7 @@ dem_status dem_stats(dem_ctx* ctx, dem_stats_t* out)
     if (ctx->status) return check_status(ctx);
     memset(out, 0, sizeof(*out));
     out->steps = ctx->steps;
-    out->step_threads = ctx->graph_fused ? TILE : step_block(ctx);
+    out->step_threads = ctx->graph_fused ? TILE : step_block(ctx);   // (the setting that fused steps need)
     out->step_lanes = ctx->step_lanes;
     out->graph_fused = ctx->graph_fused ? 1 : 0;
     if (dem_status st = refresh_count(ctx)) return st;
@@ -3842,7 +3842,7 @@ dem_status dem_set_step_block(dem_ctx* ctx, int32_t threads)
 dem_status dem_set_list_build(dem_ctx* ctx, int32_t staged)
 {
     if (!ctx) return DEM_ERR_ARG;
-    if (staged != 0 && staged != 1) return fail(ctx, DEM_ERR_ARG, "list build must be 0 (direct scan) or 1 (staged)");
+    if (staged != 0 && staged != 1) return fail(ctx, DEM_ERR_ARG, "list build must be 0 (by cubes of cells) or 1 (staged)");
     ctx->list_staged = staged != 0;
     return ctx->graph_steps > 0 ? build_graph(ctx, ctx->graph_steps) : DEM_OK;   // the graph holds the chain
 }
