@@ -248,9 +248,10 @@ dem_status dem_set_graph_mode(dem_ctx *ctx, int32_t mode);
 /* How the neighbour lists are built (the cell-range and list-build step of the rebuild; the
  * list is the same either way, bit for bit): 0 (the default), each block copies the positions of a
  * cube of 64 cells and of the cells around it to shared memory, where its particles find their
- * neighbours; 1, each block first stages the cell-ordered positions around its 64 particles in
- * shared memory, and each particle looks up the 27 cells around it and reads the candidates that
- * fall there from it.  DEM_ERR_ARG for other values.  A captured graph is rebuilt with it.
+ * neighbours (those of crowded cubes, and of sparse ones where there are many, look up the 27 cells
+ * around them instead); 1, each block first stages the cell-ordered positions around its 128
+ * particles in shared memory, and each particle looks up the 27 cells around it and reads the
+ * candidates that fall there from it.  DEM_ERR_ARG for other values.  A captured graph is rebuilt with it.
  * Not in the paper: an implementation choice (the second measured slower on the 1M bed). */
 dem_status dem_set_list_build(dem_ctx *ctx, int32_t staged);
 

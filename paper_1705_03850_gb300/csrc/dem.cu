@@ -114,20 +114,23 @@ __global__ void __launch_bounds__(1024) k_scan_top(Dev d)
     }
 }
 
-// Also lists the cubes of CUBE codes that hold particles (the list build's units of work) and leaves
-// the counts zero for the next build.
+// Also lists the cubes of CUBE codes that hold particles (the list build's units of work), by what they
+// hold: ordinary ones from the front of the list, sparse ones (fewer than CUBE_MIN particles) from its
+// back, crowded ones (more than CUBE_MAX) not at all; noted in cube_dir and counted with their particles,
+// which decides who builds their rows (cube_route).  Leaves the counts zero for the next build.
 constexpr int CUBE = 64;       // 4 x 4 x 4 cells where each axis has at least four
+constexpr unsigned CUBE_MIN = 44, CUBE_MAX = 224;
 __global__ void __launch_bounds__(SCAN_T) k_scan_down(Dev d)
 {
     if (!d.g->any || !chunk_active(d, blockIdx.x)) return;
     constexpr int TPC = CUBE / SCAN_V, NC = SCAN_TILE / CUBE;   // threads per cube, cubes per chunk
     static_assert(32 % TPC == 0 && NC <= 32, "a cube within a warp, a chunk's cubes in one mask");
-    __shared__ unsigned held;
-    __shared__ int first;
+    __shared__ unsigned mask[3], parts[3];       // by DIR_*: the chunk's cubes and their particles
+    __shared__ int first, last;
     const unsigned base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
     unsigned v[SCAN_V];
     unsigned s = 0;
-    if (threadIdx.x == 0) held = 0u;
+    if (threadIdx.x < 3) mask[threadIdx.x] = parts[threadIdx.x] = 0u;
 #pragma unroll
     for (int k = 0; k < SCAN_V; ++k) {
         unsigned i = base + k;
@@ -136,7 +139,15 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_down(Dev d)
     }
     unsigned tot;
     unsigned ex = block_exclusive_scan(s, &tot) + d.part[blockIdx.x];
-    if (s) atomicOr(&held, 1u << (threadIdx.x / TPC));
+    unsigned n = s;                              // the cube's particles
+#pragma unroll
+    for (int o = 1; o < TPC; o <<= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+    if (threadIdx.x % TPC == 0 && n) {
+        const int dir = n < CUBE_MIN ? DIR_SPARSE : n > CUBE_MAX ? DIR_CROWDED : DIR_CUBE;
+        atomicOr(&mask[dir], 1u << (threadIdx.x / TPC));
+        atomicAdd(&parts[dir], n);
+        d.cube_dir[base / CUBE] = (unsigned char)dir;
+    }
 #pragma unroll
     for (int k = 0; k < SCAN_V; ++k) {
         unsigned i = base + k;
@@ -147,21 +158,86 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_down(Dev d)
         ex += v[k];
     }
     __syncthreads();
-    if (threadIdx.x == 0) first = atomicAdd(&d.g->ncubes, __popc(held));
+    if (threadIdx.x % 32 == 0 && threadIdx.x < 96) {
+        const int dir = threadIdx.x / 32;
+        if (mask[dir]) {
+            const unsigned long long c = ((unsigned long long)__popc(mask[dir]) << 32) | parts[dir];
+            const int at = (int)(atomicAdd(&d.g->cubes[dir], c) >> 32);
+            if (dir == DIR_CUBE) first = at;
+            if (dir == DIR_SPARSE) last = (int)(d.ncodes / CUBE) - at;
+        }
+    }
     __syncthreads();
-    if (threadIdx.x < NC && ((held >> threadIdx.x) & 1u))
-        d.cubes[first + __popc(held & ((1u << threadIdx.x) - 1u))] = (int)(blockIdx.x * SCAN_TILE + threadIdx.x * CUBE);
+    if (threadIdx.x < NC) {
+        const unsigned bit = 1u << threadIdx.x;
+        const int code = (int)(blockIdx.x * SCAN_TILE + threadIdx.x * CUBE);
+        if (mask[DIR_CUBE] & bit) d.cubes[first + __popc(mask[DIR_CUBE] & (bit - 1u))] = code;
+        if (mask[DIR_SPARSE] & bit) d.cubes[last - __popc(mask[DIR_SPARSE] & (bit - 1u))] = code;
+    }
+}
+
+// Which kinds of cubes are left out of the build by cubes (a block per cube), for their particles to look
+// their 27 cells up one by one (a thread per particle): bit DIR_*.  Crowded ones always: a thread scans
+// their long runs as fast from L2 (300,000 spheres, cells of 3.8: 288 and 290 us), and a block takes several
+// passes over such a cube, in few blocks (a call with a build of 10,000 spheres in 18 cubes: 298 against 185 us).
+// All cubes where a quarter of the particles are in crowded ones: half the work each way
+// takes longer (a call of 532 against 475 us, cells of 3.4), and the few cubes at a bed's rim a round alone.
+// Sparse ones by the time of either way, as a block looks up 216 cells whatever the cube holds: with n
+// particles a cube 5.4 + 0.25 n ns a cube there, on the whole chip, and 0.159 + 0.0048 n ns a particle
+// here, with 20 us for doing both (calls with a build of 300,000 spheres, by cubes and by threads: n = 98
+// 193 and 289 us, 49 202 and 219, 38 204 and 166, 25 238 and 160, 10 401 and 153, 0.6 3230 and 904); from
+// 2,000 cubes, as one or two rounds of blocks are over before (10,000 spheres, n = 25: 73 and 82 us; n = 3: 95
+// and 79).
+__device__ __forceinline__ unsigned cube_route(const Dev& d)
+{
+    float N[3], P[3];
+    for (int i = 0; i < 3; ++i) {
+        const unsigned long long c = d.g->cubes[i];
+        N[i] = (float)(unsigned)(c >> 32);
+        P[i] = (float)(unsigned)c;
+    }
+    const float pc = P[DIR_CROWDED];
+    if (4.f * pc > P[DIR_CUBE] + P[DIR_SPARSE] + pc) return DIR_ALL;
+    unsigned left = 1u << DIR_CROWDED;
+    if (N[DIR_CUBE] + N[DIR_SPARSE] < 2000.f) return left;
+    auto cube = [&](int i) { return 5.4f * N[i] + 0.25f * P[i]; };
+    auto direct = [&](int i) { return 0.159f * P[i] + 0.0048f * P[i] * P[i] / fmaxf(N[i], 1.f); };
+    const float all = cube(DIR_CUBE) + cube(DIR_SPARSE);
+    const float both = cube(DIR_CUBE) + direct(DIR_SPARSE) + (pc > 0.f ? 0.f : 20000.f);
+    const float none = direct(DIR_CUBE) + direct(DIR_SPARSE);
+    if (none < all && none < both) left = DIR_ALL;
+    else if (both < all) left |= 1u << DIR_SPARSE;
+    return left;
 }
 
 // ==================================================================== cells
 // (axis_cell, cell_code, min_image in dem_internal.cuh)
+
+// counters of the blocks that are done: a release of the block's earlier writes and an acquire of
+// the other blocks' (lighter than __threadfence, which is a sequentially consistent fence)
+__device__ __forceinline__ unsigned add_acq_rel(unsigned* p)
+{
+    unsigned v;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void add_release(unsigned* p)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 
 // ================================================================ rebuild
 // Triggered per instance by the displacement bound (flag != 0).  Sequence:
 // bin (atomic slot in cell) -> scan -> scatter -> order each
 // cell by particle ID -> order the slots of each tile by contact count
 // (and copy positions and IDs in cell order) -> build lists, permute state,
-// carry histories -> finish.
+// carry histories, finish.
 
 // Per-slot rebuild work runs on a persistent grid of TILE-thread blocks that
 // strides over the tiles and skips tiles of instances that are not rebuilding.
@@ -182,6 +258,7 @@ __device__ __forceinline__ void for_rebuilding_slots(const Dev& d, Fn fn)
 __global__ void __launch_bounds__(TILE) k_rb_bin(Dev d)
 {
     if (!d.g->any) return;
+    if (blockIdx.x == 0 && threadIdx.x < 3) d.g->cubes[threadIdx.x] = 0ull;
     for_rebuilding_slots(d, [&](int s, const InstD& D, const InstC& c) {
         const unsigned idw = __float_as_uint(d.vel[D.cur][s].w);
         if (idw & GONE_BIT) {               // removed particle: not binned, its ID unmapped
@@ -199,6 +276,7 @@ __global__ void __launch_bounds__(TILE) k_rb_bin(Dev d)
 __global__ void __launch_bounds__(TILE) k_rb_scatter(Dev d)
 {
     if (!d.g->any) return;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) d.g->left = cube_route(d);   // (a block with little else)
     for_rebuilding_slots(d, [&](int s, const InstD& D, const InstC& c) {
         if (d.cslot[s] == 0xffffffffu) return;   // removed
         const unsigned code = d.cellcode[s];
@@ -408,6 +486,30 @@ __global__ void __launch_bounds__(WS_T) k_rb_winsort(Dev d, int G)
 // other state buffer, and carry the tangential overlaps of pairs that were already
 // listed (found by ID in the particle's previous row).
 
+// the particle's state from its slot `old` to its new slot s
+__device__ __forceinline__ void move_state(const Dev& d, int s, int old, const InstD& D, const InstC& c)
+{
+    const int cur = D.cur, nxt = cur ^ 1, lp = D.lp, nlp = lp ^ 1;
+    const bool fresh = D.flag == 2;          // a written state: no histories
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 v = d.vel[cur][old];
+    const int4 p = d.pos[cur][old];
+    const float4 w = d.omg[cur][old];
+    const float4 wh = fresh ? z4 : d.whist[lp][old];
+    const unsigned myid = __float_as_uint(v.w) & ID_MASK;
+    if (fresh) v.w = __uint_as_float(myid);  // no floor history
+    d.pos[nxt][s] = p;
+    d.vel[nxt][s] = v;
+    d.omg[nxt][s] = w;
+    d.slot_of_id[c.slot0 + (int)myid] = s;
+    if (D.fext) d.fext[nlp][s] = d.fext[lp][old];      // held until overwritten, even across state writes
+    d.whist[nlp][s] = wh;
+    if (c.nwp >= 2) {
+        d.wseg[nlp][s] = fresh ? z4 : d.wseg[lp][old];
+        d.wseg[nlp][d.ncap + s] = fresh ? z4 : d.wseg[lp][d.ncap + old];
+    }
+}
+
 // The particle `old` (cell-order position ps) with its list of nl <= N candidates, get(i, key, m):
 // key d^2 - (r_i + r_j)^2 (rounded to float: monotone) and cell-order position, the particle itself
 // among them or not.  The row goes out ordered by (key, ID) to the particle's new slot s, with the
@@ -418,10 +520,9 @@ template <int N, typename Get>
 __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, const InstD& D, const InstC& c, int nl, bool overflow,
                                         Get get)
 {
-    const int cur = D.cur, nxt = cur ^ 1, lp = D.lp, nlp = lp ^ 1;
+    const int cur = D.cur, lp = D.lp, nlp = lp ^ 1;
     const int ncap = d.ncap, Lmax = d.Lmax;
     const bool fresh = D.flag == 2;          // a written state: no histories
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     const int ocnt = fresh ? 0 : d.cnt[lp][old];
     unsigned ohm = fresh ? 0u : d.hmask[lp][old];
     float key[N];
@@ -526,281 +627,109 @@ __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, co
             }
         }
     }
-    float4 v = d.vel[cur][old];
-    const int4 p = d.pos[cur][old];
-    const float4 w = d.omg[cur][old];
-    const float4 wh = fresh ? z4 : d.whist[lp][old];
-    const unsigned myid = __float_as_uint(v.w) & ID_MASK;
-    if (fresh) v.w = __uint_as_float(myid);  // no floor history
-    d.pos[nxt][s] = p;
-    d.vel[nxt][s] = v;
-    d.omg[nxt][s] = w;
-    d.slot_of_id[c.slot0 + (int)myid] = s;
     d.cnt[nlp][s] = min(nc, Lmax);           // (one more can be listed where the row overflows)
     d.hmask[nlp][s] = nhm;
-    if (D.fext) d.fext[nlp][s] = d.fext[lp][old];      // held until overwritten, even across state writes
-    d.whist[nlp][s] = wh;
-    if (c.nwp >= 2) {
-        d.wseg[nlp][s] = fresh ? z4 : d.wseg[lp][old];
-        d.wseg[nlp][ncap + s] = fresh ? z4 : d.wseg[lp][ncap + old];
-    }
+    move_state(d, s, old, D, c);
 }
 
-// The default list build: one block per cube of CUBE consecutive Morton codes (4 x 4 x 4 cells)
-// that holds particles.  The block copies the positions of the cube's cells and of the layer of
-// cells around them (6 x 6 x 6) into shared memory, x fastest, shifted to the image next to the
-// cube, so that the three cells of a row along x are one run: a particle scans nine runs there,
-// without image arithmetic, cell lookups or trips to L2.  The copy goes by windows of CB_CAP
-// positions, so that any occupancy fits; at ordinary densities (370 to 530 positions for 110 to
-// 155 particles) one window holds them all.  The distance test needs no check of the axes first:
-// in unsigned 64 bits three squares of 32-bit differences cannot overflow.
-// Bound by latency: of the 40,000 cycles a block spends on a cube of the 1M bed, half go to the
-// scan (16-byte shared loads at random, four candidates at a time) and a third to the row's way out.
-// One list build of a 1M bed adds 390 us to a step, of a 100,000-sphere bed 55 us, against 575 and
-// 78 us with a thread looking up and scanning its 27 cells in global memory; blocks of 192 threads
-// and 4 to 7 resident blocks of 128 came within 5 % of this.
-constexpr int CB_T = 128;                    // threads per block
-constexpr int CB_CAP = 640;                  // positions per window
-constexpr int CB_H = 600;                    // cells of a cube and around it: 216, at most 66 x 3 x 3
-constexpr int CB_OWN = 384;                  // particles of the cube whose cell is noted (the others' is computed)
-struct CubeScratch {
-    int4 pos[CB_CAP];
-    int m[CB_CAP];                           // their cell-order positions
-    unsigned char shift[CB_CAP];             // images: bits 0-1 x, 2-3 y (0 none, 1 from below, 2 from above)
-    unsigned short own[CB_OWN];              // the cell (as h) of the cube's particles
-    int off[CB_H + 1];                       // cell h's first position in the copied order
-    int wsum[CB_T / 32];
-};
-__host__ __device__ constexpr size_t cube_smem(int lmax) { return (size_t)(lmax + 1) * CB_T * 4; }
-
-__global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
+// As row_out for a row of any length, ordered in place in shared memory, without the state: key(e) and
+// pos(e) are references to entry e, cell(x) the cell-order position that pos(e) = x stands for.  Of nc
+// entries the first d.Lmax go out.  By key first, then the entries of equal keys by ID, so that the row does not
+// depend on the scan order; the keys give way to the IDs, whose loads are in flight together.
+template <typename Key, typename Pos, typename Cell>
+__device__ __forceinline__ void row_sorted(const Dev& d, int s, int old, const InstD& D, int nc, bool overflow, Key key, Pos pos,
+                                           Cell cell)
 {
-    if (!d.g->any) return;
-    __shared__ CubeScratch C;
-    extern __shared__ int cube_rows[];       // candidates [Lmax + 1][CB_T]: the particle itself is among them
-    const int tx = threadIdx.x, lane = tx & 31, warp = tx >> 5;
-    const int Lmax = d.Lmax;
-    int* row = cube_rows + tx;
-    const int ncubes = d.g->ncubes;
-    for (int i = blockIdx.x; i < ncubes; i += gridDim.x) {
-        const int code = d.cubes[i];
-        const int k = d.B == 1 ? 0 : d.part_inst[code / SCAN_TILE];
-        const InstD D = d.id[k];
-        const InstC& c = d.ic[k];
-        const unsigned cbase = d.crange[c.code0].x;
-        const int last = min(code + CUBE, c.code0 + c.ncode) - 1;
-        const uint2 rl = d.crange[last];
-        const int first = (int)d.crange[code].x;
-        const int p0 = c.slot0 + first - (int)cbase, n = (int)(rl.x + rl.y) - first;
-        // the cube's first cell, from any of its particles
-        const int4 pf = d.spos[p0];
-        const int lgx = D.cube_lg & 15, lgy = (D.cube_lg >> 4) & 15, lgz = (D.cube_lg >> 8) & 15;
-        const int bx = axis_cell(c, 0, pf.x) >> lgx << lgx, by = axis_cell(c, 1, pf.y) >> lgy << lgy,
-                  bz = axis_cell(c, 2, pf.z) >> lgz << lgz;
-        const int HX = (1 << lgx) + 2, HY = (1 << lgy) + 2, HZ = (1 << lgz) + 2;
-        const int H = HX * HY * HZ;
-        __syncthreads();                     // the previous cube is done with the shared arrays
-        // the cells, each thread a run of them: starts, counts and images, then their offsets
-        constexpr int CHM = (CB_H + CB_T - 1) / CB_T;
-        const int CH = (H + CB_T - 1) / CB_T;
-        int cst[CHM], ccn[CHM], csh[CHM];
-        int sum = 0;
-#pragma unroll
-        for (int q = 0; q < CHM; ++q) {
-            const int h = tx * CH + q;
-            cst[q] = ccn[q] = csh[q] = 0;
-            if (q < CH && h < H) {
-                const int hx = h % HX, hy = (h / HX) % HY, hz = h / (HX * HY);
-                int cx = bx - 1 + hx, cy = by - 1 + hy;
-                const int cz = bz - 1 + hz;
-                int sh = 0;
-                if (c.per[0]) {
-                    if (cx < 0) { cx += c.nc[0]; sh |= 1; }
-                    else if (cx == c.nc[0]) { cx = 0; sh |= 2; }
-                }
-                if (c.per[1]) {
-                    if (cy < 0) { cy += c.nc[1]; sh |= 4; }
-                    else if (cy == c.nc[1]) { cy = 0; sh |= 8; }
-                }
-                if (cx >= 0 && cx < c.nc[0] && cy >= 0 && cy < c.nc[1] && cz >= 0 && cz < c.nc[2]) {
-                    const unsigned cd = cell_code(d, c, cx, cy, cz);
-                    bool ok = true;
-#if DEM_CHECKS
-                    ok = in_range(d, (long long)cd - c.code0, c.ncode, p0, 1);
-#endif
-                    if (ok) {
-                        const uint2 r = d.crange[cd];
-                        cst[q] = c.slot0 + (int)(r.x - cbase);
-                        ccn[q] = (int)r.y;
-                        csh[q] = sh;
-#if DEM_CHECKS
-                        if (ccn[q] > 0 && !(in_range(d, cst[q] - c.slot0, c.cap, p0, 2) &&
-                                            in_range(d, cst[q] - c.slot0 + ccn[q], c.cap + 1, p0, 2)))
-                            ccn[q] = 0;
-#endif
-                        // a cell of the cube itself (not an image of one): its particles' cell
-                        if (sh == 0 && hx >= 1 && hx < HX - 1 && hy >= 1 && hy < HY - 1 && hz >= 1 && hz < HZ - 1)
-                            for (int t = 0; t < ccn[q]; ++t)
-                                if (cst[q] - p0 + t < CB_OWN) C.own[cst[q] - p0 + t] = (unsigned short)h;
-                    }
-                }
-                sum += ccn[q];
-            }
+    const int cur = D.cur, lp = D.lp, nlp = lp ^ 1;
+    const int ncap = d.ncap;
+    for (int i = 1; i < nc; ++i) {
+        const float k = key(i);
+        const auto m = pos(i);
+        int j = i - 1;
+        for (; j >= 0 && key(j) > k; --j) {
+            key(j + 1) = key(j);
+            pos(j + 1) = pos(j);
         }
-        int inc = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
+        key(j + 1) = k;
+        pos(j + 1) = m;
+    }
+    unsigned long long tie = 0ull;           // bit e: entry e has the key of the one before it
+    for (int e = 1; e < nc; ++e) tie |= (unsigned long long)(key(e) == key(e - 1)) << e;
+#pragma unroll 4
+    for (int e = 0; e < nc; ++e) key(e) = __int_as_float(d.sid[cell(pos(e))]);
+    for (unsigned long long t = tie; t; t &= t - 1ull) {
+        const int i = __ffsll(t) - 1;
+        const float k = key(i);
+        const auto m = pos(i);
+        int j = i - 1;
+        for (; ((tie >> (j + 1)) & 1ull) && __float_as_int(key(j)) > __float_as_int(k); --j) {
+            key(j + 1) = key(j);
+            pos(j + 1) = pos(j);
         }
-        if (lane == 31) C.wsum[warp] = inc;
-        __syncthreads();
-        int off0 = inc - sum, total = 0;
-        for (int w = 0; w < CB_T / 32; ++w) {
-            if (w < warp) off0 += C.wsum[w];
-            total += C.wsum[w];
-        }
-        {
-            int off = off0;
-#pragma unroll
-            for (int q = 0; q < CHM; ++q) {
-                const int h = tx * CH + q;
-                if (q < CH && h < H) C.off[h] = off;
-                off += ccn[q];
+        key(j + 1) = k;
+        pos(j + 1) = m;
+    }
+    nc = min(nc, d.Lmax);
+    if (overflow) {
+        atomicOr(&d.g->status, ST_CAPACITY);
+        d.g->err_slot = s;
+    }
+    int* nrow = d.nbr[nlp] + s;
+#pragma unroll 4
+    for (int e = 0; e < nc; ++e) nrow[(size_t)e * ncap] = d.fin[cell(pos(e))];
+    const size_t plane = (size_t)d.Lmax * ncap;
+    const int* orow = d.nbr[lp] + old;
+    const float* ho = d.hist[lp] + old;
+    float* hn = d.hist[nlp] + s;
+    const int ocnt = D.flag == 2 ? 0 : d.cnt[lp][old];
+    unsigned ohm = D.flag == 2 ? 0u : d.hmask[lp][old];
+    if (ocnt < 32) ohm &= (1u << ocnt) - 1u;
+    unsigned nhm = 0u;
+    while (ohm) {
+        const int eo = __ffs(ohm) - 1;
+        ohm &= ohm - 1u;
+        const float hx = ho[(size_t)eo * ncap], hy = ho[plane + (size_t)eo * ncap], hz = ho[2 * plane + (size_t)eo * ncap];
+        if (hx == 0.f && hy == 0.f && hz == 0.f) continue;
+        const int oid = (int)(__float_as_uint(d.vel[cur][orow[(size_t)eo * ncap]].w) & ID_MASK);
+        for (int e = 0; e < nc; ++e) {
+            if (__float_as_int(key(e)) == oid) {
+                hn[(size_t)e * ncap] = hx;
+                hn[plane + (size_t)e * ncap] = hy;
+                hn[2 * plane + (size_t)e * ncap] = hz;
+                nhm |= 1u << e;
+                break;
             }
-            if (tx == 0) C.off[H] = total;
-        }
-        // the cube's particles, CB_T at a time
-        for (int g0 = 0; g0 < n; g0 += CB_T) {
-            const bool mine = g0 + tx < n;
-            const int ps = p0 + g0 + tx;
-            int old = 0, s = 0, nl = 0, h0 = 0;
-            int4 p = make_int4(0, 0, 0, 0);
-            if (mine) {
-                p = d.spos[ps];
-                old = d.perm[ps];
-                s = d.fin[ps];
-            }
-            for (int w0 = 0; w0 < total; w0 += CB_CAP) {
-                const int w1 = min(total, w0 + CB_CAP);
-                if (w0 > 0 || g0 > 0) __syncthreads();   // the previous window is done with
-                if (g0 == 0 || total > CB_CAP) {
-                    // where each position of the window comes from, then the positions, coalesced
-                    int o = off0;
-#pragma unroll
-                    for (int q = 0; q < CHM; ++q) {
-                        for (int t = max(0, w0 - o); t < min(ccn[q], w1 - o); ++t) {
-                            C.m[o + t - w0] = cst[q] + t;
-                            C.shift[o + t - w0] = (unsigned char)csh[q];
-                        }
-                        o += ccn[q];
-                    }
-                    __syncthreads();
-                    for (int t = tx; t < w1 - w0; t += CB_T) {
-                        int4 q = __ldg(d.spos + C.m[t]);
-                        const int sh = C.shift[t];
-                        if (sh & 3) q.x += (sh & 1) ? -c.ext[0] : c.ext[0];
-                        if (sh & 12) q.y += (sh & 4) ? -c.ext[1] : c.ext[1];
-                        C.pos[t] = q;
-                    }
-                }
-                __syncthreads();
-                if (!mine) continue;
-                if (w0 == 0) {
-                    // the run of cells that starts one below the particle's on every axis
-                    if (ps - p0 < CB_OWN)
-                        h0 = (int)C.own[ps - p0] - (HY + 1) * HX - 1;
-                    else
-                        h0 = ((axis_cell(c, 2, p.z) - bz) * HY + axis_cell(c, 1, p.y) - by) * HX + axis_cell(c, 0, p.x) - bx;
-                }
-                const int cut0 = p.w + c.skin;
-                const int before = nl;
-#pragma unroll 1
-                for (int r = 0; r < 9; ++r) {
-                    const int h = h0 + (r / 3 * HY + r % 3) * HX;
-                    const int t1 = min(C.off[h + 3], w1) - w0;
-                    // four at a time, without branches: the loop waits for its loads and products
-                    for (int t = max(C.off[h], w0) - w0; t < t1; t += 4) {
-                        int4 q[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) q[u] = C.pos[min(t + u, t1 - 1)];
-                        bool hit[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int dx = p.x - q[u].x, dy = p.y - q[u].y;
-                            // z reaches +-2e9 units, outside the box too: |dz| in 32 bits without sign, cut off
-                            // where it is beyond any cut
-                            const unsigned dz = min(__sad(p.z, q[u].z, 0u), 0x7fffffffu);
-                            const int cut = cut0 + q[u].w;
-                            const unsigned long long d2 = (unsigned long long)((long long)dx * dx) +
-                                                          (unsigned long long)((long long)dy * dy) +
-                                                          (unsigned long long)dz * dz;
-                            hit[u] = t + u < t1 && d2 < (unsigned long long)((long long)cut * cut);
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (hit[u]) {
-                                if (nl <= Lmax) row[nl * CB_T] = t + u;
-                                ++nl;
-                            }
-                    }
-                }
-                if (total > CB_CAP)          // the next window takes this one's place
-                    for (int e = before; e < min(nl, Lmax + 1); ++e) row[e * CB_T] = C.m[row[e * CB_T]];
-            }
-            const int most = __reduce_max_sync(0xffffffffu, nl);
-            if (!mine) continue;
-            const bool overflow = nl > Lmax + 1;
-            nl = min(nl, Lmax + 1);
-            auto get = [&](int e, float& key, int& m) {
-                const int t = row[e * CB_T];
-                int4 q;
-                long long dx, dy;
-                if (total > CB_CAP) {
-                    m = t;
-                    q = __ldg(d.spos + m);
-                    dx = min_image(p.x - q.x, c.per[0], c.ext[0], c.half[0]);
-                    dy = min_image(p.y - q.y, c.per[1], c.ext[1], c.half[1]);
-                } else {
-                    m = C.m[t];
-                    q = C.pos[t];
-                    dx = p.x - q.x;
-                    dy = p.y - q.y;
-                }
-                const long long dz = (long long)p.z - q.z, S = (long long)p.w + q.w;
-                key = (float)(dx * dx + dy * dy + dz * dz - S * S);
-            };
-            if (most <= 9) row_out<9>(d, s, old, ps, D, c, nl, overflow, get);
-            else if (most <= 13) row_out<13>(d, s, old, ps, D, c, nl, overflow, get);
-            else if (most <= 17) row_out<17>(d, s, old, ps, D, c, nl, overflow, get);
-            else row_out<MAXL + 1>(d, s, old, ps, D, c, nl, overflow, get);
         }
     }
+    d.cnt[nlp][s] = nc;
+    d.hmask[nlp][s] = nhm;
 }
 
-// The other list build (dem_set_list_build): one block per 64 cell-order positions, with RB_W on
-// either side (the cells around the block's particles, in Morton order) staged in shared memory;
-// each thread looks up and scans its 27 cells, candidates inside the window are read from there,
-// the others from L2.
-constexpr int RB_T = 64;                     // threads per block
+constexpr int RB_T = 128;                    // threads per block of the list build
+
+// The list build of one particle by a thread that looks up and scans the 27 cells around it in the
+// cell-ordered positions: from L2 (cube_route), or, where dem_set_list_build asks for it (STAGED), with
+// the positions of the block's particles and RB_W on either side (the cells around them, in Morton
+// order) staged in shared memory.  The row is kept in shared memory meanwhile, entry-major.
 constexpr int RB_W = 128;
 constexpr int RB_WIN = RB_T + 2 * RB_W;
 struct Window {
     int4 pos[RB_WIN];
     int lo, n;                               // first cell-order position and length
 };
-struct RowScratch {
-    float key[MAXL][RB_T];
-    int pos[MAXL][RB_T];
+struct RowScratch {                          // [Lmax][RB_T] each, from the thread's own on
+    float* key;
+    int* pos;
 };
+__host__ __device__ constexpr size_t row_smem(int lmax) { return (size_t)lmax * RB_T * 8; }
 
-__device__ __forceinline__ void build_row(const Dev& d, int ps, const InstD& D, const InstC& c, RowScratch& R,
-                                          const Window& W)
+template <bool STAGED>
+__device__ __forceinline__ void build_row(const Dev& d, int ps, int old, const InstD& D, const InstC& c, const RowScratch& R,
+                                          const Window* W)
 {
-    const int tx = threadIdx.x;
-    const int old = d.perm[ps];
     const int s = d.fin[ps];
     const int4 p = d.spos[ps];
+    move_state(d, s, old, D, c);
 
     // candidates ordered by (d^2 - (r_i + r_j)^2, ID): deepest overlaps first, so
     // that within a warp the contacts sit in the leading entries of every row
@@ -868,8 +797,13 @@ __device__ __forceinline__ void build_row(const Dev& d, int ps, const InstD& D, 
 #endif
         for (int t = 0; t < cnt; ++t) {
             const int m = start + t;
-            const unsigned wi = (unsigned)(m - W.lo);
-            const int4 q = wi < (unsigned)W.n ? W.pos[wi] : __ldg(d.spos + m);
+            int4 q;
+            if (STAGED) {
+                const unsigned wi = (unsigned)(m - W->lo);
+                q = wi < (unsigned)W->n ? W->pos[wi] : __ldg(d.spos + m);
+            } else {
+                q = __ldg(d.spos + m);
+            }
             const int ddx = min_image(p.x - q.x, per0, ext0, hf0);
             const int ddy = min_image(p.y - q.y, per1, ext1, hf1);
             const long long ddz = (long long)p.z - q.z;
@@ -883,37 +817,322 @@ __device__ __forceinline__ void build_row(const Dev& d, int ps, const InstD& D, 
                 overflow = true;
                 continue;
             }
-            R.key[nc][tx] = (float)(d2 - S * S);
-            R.pos[nc][tx] = m;
+            R.key[nc * RB_T] = (float)(d2 - S * S);
+            R.pos[nc * RB_T] = m;
             ++nc;
         }
     }
-    auto get = [&](int e, float& key, int& m) {
-        key = R.key[e][tx];
-        m = R.pos[e][tx];
-    };
-    const int most = __reduce_max_sync(__activemask(), nc);
-    if (most <= 9) row_out<9>(d, s, old, ps, D, c, nc, overflow, get);
-    else if (most <= 17) row_out<17>(d, s, old, ps, D, c, nc, overflow, get);
-    else row_out<MAXL>(d, s, old, ps, D, c, nc, overflow, get);
+    row_sorted(
+        d, s, old, D, nc, overflow, [&](int e) -> float& { return R.key[e * RB_T]; }, [&](int e) -> int& { return R.pos[e * RB_T]; },
+        [](int m) { return m; });
 }
 
-__global__ void __launch_bounds__(RB_T, 10) k_rb_build(Dev d)
+// The end of the rebuild, by the block that is the last to have written its rows.
+__device__ __forceinline__ void rb_finish(const Dev& d)
+{
+    __shared__ bool am_last;
+    __syncthreads();
+    if (threadIdx.x == 0) am_last = add_acq_rel(&d.g->rb_done) == gridDim.x - 1;
+    __syncthreads();
+    if (!am_last) return;
+    // the instances that were built, and the tiles fused steps walk: per instance the pairs of tiles that
+    // hold its live slots (offsets by a scan over a chunk of instances, then the chunk's ranges written by
+    // the block)
+    __shared__ unsigned s_off[RB_T], s_lt[RB_T];
+    __shared__ int s_t0[RB_T];
+    unsigned base = 0u;
+    for (int k0 = 0; k0 < d.B; k0 += blockDim.x) {
+        const int k = k0 + (int)threadIdx.x;
+        unsigned lt = 0u;
+        int t0 = 0;
+        if (k < d.B) {
+            InstD& D = d.id[k];
+            t0 = d.ic[k].slot0 / TILE;
+            const int flag = D.flag, n = flag ? D.n_new : D.n;
+            lt = 2u * (unsigned)((n + 2 * TILE - 1) / (2 * TILE));
+            if (flag) {
+                D.cur ^= 1;
+                D.lp ^= 1;
+                if (flag != 3) atomicAdd(&d.g->rebuilds, 1ull);
+                D.flag = 0;
+                D.n = n;
+                D.nbin = n;
+                D.disp = 0.f;
+            }
+        }
+        unsigned tot;
+        const unsigned off = base + block_exclusive_scan(lt, &tot);
+        s_off[threadIdx.x] = off;
+        s_lt[threadIdx.x] = lt;
+        s_t0[threadIdx.x] = t0;
+        __syncthreads();
+        const int nk = min((int)blockDim.x, d.B - k0);
+        const bool few = nk < RB_T / 32;         // a block or a warp per instance
+        for (int j = few ? 0 : (int)threadIdx.x / 32; j < nk; j += few ? 1 : RB_T / 32)
+            for (unsigned i = few ? threadIdx.x : threadIdx.x % 32; i < s_lt[j]; i += few ? RB_T : 32)
+                d.live_tiles[s_off[j] + i] = s_t0[j] + (int)i;
+        __syncthreads();
+        base += tot;
+    }
+    if (threadIdx.x == 0) {
+        d.g->nlive = (int)base;
+        d.g->any = 0u;
+        d.g->rb_done = 0u;
+    }
+}
+
+// The default list build: one block per cube of CUBE consecutive Morton codes (4 x 4 x 4 cells)
+// that holds particles.  The block copies the positions of the cube's cells and of the layer of
+// cells around them (6 x 6 x 6) into shared memory, x fastest, shifted to the image next to the
+// cube, so that the three cells of a row along x are one run: a particle scans nine runs there,
+// without image arithmetic, cell lookups or trips to L2.  At ordinary densities these are 370 to 530
+// positions for 110 to 155 particles.  The distance test needs no check of the axes first: in
+// unsigned 64 bits three squares of 32-bit differences cannot overflow.  The particles of sparse and
+// crowded cubes (cube_route) look their cells up one by one, by tiles, after the cubes, and so do at
+// once those of a cube with more than CB_CAP positions around it: a kernel of its own for them made
+// every call that launches the chain without a graph 2 to 4 us longer.
+// Bound by latency: of the 40,000 cycles a block spends on a cube of the 1M bed, half go to the
+// scan (16-byte shared loads at random, four candidates at a time) and a third to the row's way out.
+// One list build of a 1M bed adds 390 us to a step, of a 100,000-sphere bed 55 us, against 575 and
+// 78 us with a thread looking up and scanning its 27 cells in global memory; blocks of 192 threads
+// and 4 to 7 resident blocks of 128 came within 5 % of this.
+constexpr int CB_T = RB_T;
+static_assert(CB_T == TILE, "a tile a block where cubes are left");
+constexpr int CB_CAP = 800;                  // positions of a cube and around it (5 blocks an SM with lists of 32)
+constexpr int CB_H = 600;                    // cells of a cube and around it: 216, at most 66 x 3 x 3
+struct CubeScratch {
+    int4 pos[CB_CAP];
+    int m[CB_CAP];                           // their cell-order positions
+    unsigned char shift[CB_CAP];             // images: bits 0-1 x, 2-3 y (0 none, 1 from below, 2 from above)
+    unsigned short own[CUBE_MAX];            // the cell (as h) of the cube's particles
+    int off[CB_H + 1];                       // cell h's first position in the copied order
+    int wsum[CB_T / 32];
+};
+__host__ __device__ constexpr size_t cube_smem(int lmax)
+{
+    const size_t rows = (size_t)(lmax + 1) * CB_T * 2;   // the candidates of a thread's row as positions of the copy
+    return sizeof(CubeScratch) + rows > row_smem(lmax) ? sizeof(CubeScratch) + rows : row_smem(lmax);
+}
+
+__global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
 {
     if (!d.g->any) return;
-    __shared__ RowScratch R;
+    extern __shared__ int4 cube_mem[];       // the cube and the rows of its particles, or rows alone
+    CubeScratch& C = *reinterpret_cast<CubeScratch*>(cube_mem);
+    const int tx = threadIdx.x, lane = tx & 31, warp = tx >> 5;
+    const int Lmax = d.Lmax;
+    unsigned short* row = (unsigned short*)(&C + 1) + tx;   // [Lmax + 1][CB_T]: the particle itself is among them
+    const unsigned left = d.g->left;
+    const int nfront = (left >> DIR_CUBE) & 1u ? 0 : (int)(d.g->cubes[DIR_CUBE] >> 32);
+    const int ncubes = nfront + ((left >> DIR_SPARSE) & 1u ? 0 : (int)(d.g->cubes[DIR_SPARSE] >> 32));
+    const bool some = left != 1u << DIR_CROWDED || d.g->cubes[DIR_CROWDED] != 0ull;
+    const RowScratch R{(float*)cube_mem + tx, (int*)cube_mem + Lmax * RB_T + tx};
+    for (int i = blockIdx.x; i < ncubes + (some ? d.ntiles : 0); i += gridDim.x) {
+        if (i >= ncubes) {                   // a tile of cell-order positions: those of the cubes that were left
+            const int t = i - ncubes, k = d.tile_inst[t], ps = t * TILE + tx;
+            const InstD D = d.id[k];
+            const InstC& c = d.ic[k];
+            if (!D.flag) continue;           // the same for the whole block
+            if (ncubes > 0) __syncthreads(); // a cube's arrays were here
+            if (ps - c.slot0 >= D.n_new) continue;
+            const int old = d.perm[ps];
+            if (left == DIR_ALL || ((left >> d.cube_dir[d.cellcode[old] / CUBE]) & 1u)) build_row<false>(d, ps, old, D, c, R, nullptr);
+            continue;
+        }
+        const int code = d.cubes[i < nfront ? i : (int)(d.ncodes / CUBE) - (i - nfront)];
+        const int k = d.B == 1 ? 0 : d.part_inst[code / SCAN_TILE];
+        const InstD D = d.id[k];
+        const InstC& c = d.ic[k];
+        const unsigned cbase = d.crange[c.code0].x;
+        const int last = min(code + CUBE, c.code0 + c.ncode) - 1;
+        const uint2 rl = d.crange[last];
+        const int first = (int)d.crange[code].x;
+        const int p0 = c.slot0 + first - (int)cbase, n = (int)(rl.x + rl.y) - first;
+        // the cube's first cell, from any of its particles
+        const int4 pf = d.spos[p0];
+        const int lgx = D.cube_lg & 15, lgy = (D.cube_lg >> 4) & 15, lgz = (D.cube_lg >> 8) & 15;
+        const int bx = axis_cell(c, 0, pf.x) >> lgx << lgx, by = axis_cell(c, 1, pf.y) >> lgy << lgy,
+                  bz = axis_cell(c, 2, pf.z) >> lgz << lgz;
+        const int HX = (1 << lgx) + 2, HY = (1 << lgy) + 2, HZ = (1 << lgz) + 2;
+        const int H = HX * HY * HZ;
+        __syncthreads();                     // the previous cube is done with the shared arrays
+        // the cells, each thread a run of them: starts, counts and images, then their offsets
+        constexpr int CHM = (CB_H + CB_T - 1) / CB_T;
+        const int CH = (H + CB_T - 1) / CB_T;
+        int cst[CHM], ccn[CHM], csh[CHM];
+        int sum = 0;
+#pragma unroll
+        for (int q = 0; q < CHM; ++q) {
+            const int h = tx * CH + q;
+            cst[q] = ccn[q] = csh[q] = 0;
+            if (q < CH && h < H) {
+                const int hx = h % HX, hy = (h / HX) % HY, hz = h / (HX * HY);
+                int cx = bx - 1 + hx, cy = by - 1 + hy;
+                const int cz = bz - 1 + hz;
+                int sh = 0;
+                if (c.per[0]) {
+                    if (cx < 0) { cx += c.nc[0]; sh |= 1; }
+                    else if (cx == c.nc[0]) { cx = 0; sh |= 2; }
+                }
+                if (c.per[1]) {
+                    if (cy < 0) { cy += c.nc[1]; sh |= 4; }
+                    else if (cy == c.nc[1]) { cy = 0; sh |= 8; }
+                }
+                if (cx >= 0 && cx < c.nc[0] && cy >= 0 && cy < c.nc[1] && cz >= 0 && cz < c.nc[2]) {
+                    const unsigned cd = cell_code(d, c, cx, cy, cz);
+                    bool ok = true;
+#if DEM_CHECKS
+                    ok = in_range(d, (long long)cd - c.code0, c.ncode, p0, 1);
+#endif
+                    if (ok) {
+                        const uint2 r = d.crange[cd];
+                        cst[q] = c.slot0 + (int)(r.x - cbase);
+                        ccn[q] = (int)r.y;
+                        csh[q] = sh;
+#if DEM_CHECKS
+                        if (ccn[q] > 0 && !(in_range(d, cst[q] - c.slot0, c.cap, p0, 2) &&
+                                            in_range(d, cst[q] - c.slot0 + ccn[q], c.cap + 1, p0, 2)))
+                            ccn[q] = 0;
+#endif
+                        // a cell of the cube itself (not an image of one): its particles' cell
+                        if (sh == 0 && hx >= 1 && hx < HX - 1 && hy >= 1 && hy < HY - 1 && hz >= 1 && hz < HZ - 1)
+                            for (int t = 0; t < ccn[q]; ++t)
+                                if (cst[q] - p0 + t < (int)CUBE_MAX) C.own[cst[q] - p0 + t] = (unsigned short)h;
+                    }
+                }
+                sum += ccn[q];
+            }
+        }
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) C.wsum[warp] = inc;
+        __syncthreads();
+        int off0 = inc - sum, total = 0;
+        for (int w = 0; w < CB_T / 32; ++w) {
+            if (w < warp) off0 += C.wsum[w];
+            total += C.wsum[w];
+        }
+        {
+            int off = off0;
+#pragma unroll
+            for (int q = 0; q < CHM; ++q) {
+                const int h = tx * CH + q;
+                if (q < CH && h < H) C.off[h] = off;
+                off += ccn[q];
+            }
+            if (tx == 0) C.off[H] = total;
+        }
+        if (total > CB_CAP) {                // too much around it
+            __syncthreads();                 // the rows take the cube's place
+            for (int g = tx; g < n; g += CB_T) build_row<false>(d, p0 + g, d.perm[p0 + g], D, c, R, nullptr);
+            continue;
+        }
+        // where each position comes from, then the positions, coalesced
+        {
+            int o = off0;
+#pragma unroll
+            for (int q = 0; q < CHM; ++q) {
+                for (int t = 0; t < ccn[q]; ++t) {
+                    C.m[o + t] = cst[q] + t;
+                    C.shift[o + t] = (unsigned char)csh[q];
+                }
+                o += ccn[q];
+            }
+        }
+        __syncthreads();
+        for (int t = tx; t < total; t += CB_T) {
+            int4 q = __ldg(d.spos + C.m[t]);
+            const int sh = C.shift[t];
+            if (sh & 3) q.x += (sh & 1) ? -c.ext[0] : c.ext[0];
+            if (sh & 12) q.y += (sh & 4) ? -c.ext[1] : c.ext[1];
+            C.pos[t] = q;
+        }
+        __syncthreads();
+        // the cube's particles, CB_T at a time
+        for (int g0 = 0; g0 < n; g0 += CB_T) {
+            const bool mine = g0 + tx < n;
+            const int ps = p0 + g0 + tx;
+            int old = 0, s = 0, nl = 0;
+            int4 p = make_int4(0, 0, 0, 0);
+            if (mine) {
+                p = d.spos[ps];
+                old = d.perm[ps];
+                s = d.fin[ps];
+                // the run of cells that starts one below the particle's on every axis
+                const int h0 = (int)C.own[ps - p0] - (HY + 1) * HX - 1;
+                const int cut0 = p.w + c.skin;
+#pragma unroll 1
+                for (int r = 0; r < 9; ++r) {
+                    const int h = h0 + (r / 3 * HY + r % 3) * HX;
+                    const int t1 = C.off[h + 3];
+                    // four at a time, without branches: the loop waits for its loads and products
+                    for (int t = C.off[h]; t < t1; t += 4) {
+                        int4 q[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) q[u] = C.pos[min(t + u, t1 - 1)];
+                        bool hit[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int dx = p.x - q[u].x, dy = p.y - q[u].y;
+                            // z reaches +-2e9 units, outside the box too: |dz| in 32 bits without sign, cut off
+                            // where it is beyond any cut
+                            const unsigned dz = min(__sad(p.z, q[u].z, 0u), 0x7fffffffu);
+                            const int cut = cut0 + q[u].w;
+                            const unsigned long long d2 = (unsigned long long)((long long)dx * dx) +
+                                                          (unsigned long long)((long long)dy * dy) +
+                                                          (unsigned long long)dz * dz;
+                            hit[u] = t + u < t1 && d2 < (unsigned long long)((long long)cut * cut);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (hit[u]) {
+                                if (nl <= Lmax) row[nl * CB_T] = (unsigned short)(t + u);
+                                ++nl;
+                            }
+                    }
+                }
+            }
+            const bool overflow = nl > Lmax + 1;
+            nl = min(nl, Lmax + 1);
+            const int most = __reduce_max_sync(0xffffffffu, nl);
+            if (!mine) continue;
+            auto get = [&](int e, float& key, int& m) {
+                const int t = row[e * CB_T];
+                m = C.m[t];
+                const int4 q = C.pos[t];
+                const long long dx = p.x - q.x, dy = p.y - q.y;
+                const long long dz = (long long)p.z - q.z, S = (long long)p.w + q.w;
+                key = (float)(dx * dx + dy * dy + dz * dz - S * S);
+            };
+            if (most <= 9) row_out<9>(d, s, old, ps, D, c, nl, overflow, get);
+            else if (most <= 13) row_out<13>(d, s, old, ps, D, c, nl, overflow, get);
+            else if (most <= 17) row_out<17>(d, s, old, ps, D, c, nl, overflow, get);
+            else row_out<MAXL + 1>(d, s, old, ps, D, c, nl, overflow, get);
+        }
+    }
+    rb_finish(d);
+}
+
+// The list build by windows (dem_set_list_build), over the cell-order positions: the threads of a warp hold
+// neighbouring particles and scan overlapping cells (the rows go to the particles' new slots in the same
+// tile).
+__global__ void __launch_bounds__(RB_T, 8) k_rb_windows(Dev d)
+{
+    if (!d.g->any) return;
+    extern __shared__ float row_mem[];
     __shared__ Window W;
-    constexpr int H = TILE / RB_T;           // blocks of RB_T threads per tile
-    // over the cell-order positions: the threads of a warp hold neighbouring particles and
-    // scan overlapping cells (the rows go to the particles' new slots in the same tile)
-    for (int u = blockIdx.x; u < d.ntiles * H; u += gridDim.x) {
-        const int t = u / H;
+    const RowScratch R{row_mem + threadIdx.x, (int*)row_mem + d.Lmax * RB_T + threadIdx.x};
+    static_assert(RB_T == TILE, "a tile a block");
+    for (int t = blockIdx.x; t < d.ntiles; t += gridDim.x) {
         const int k = d.tile_inst[t];
         const InstD D = d.id[k];
         if (!D.flag) continue;               // the same for the whole block
         const InstC& c = d.ic[k];
-        const int p0 = t * TILE + (u % H) * RB_T;
-        const int p = p0 + threadIdx.x;
+        const int p0 = t * TILE, p = p0 + threadIdx.x;
         const int lo = max(c.slot0, p0 - RB_W), hi = min(c.slot0 + D.n_new, p0 + RB_T + RB_W);
         __syncthreads();                     // the previous window is no longer read
         if (threadIdx.x == 0) {
@@ -922,52 +1141,9 @@ __global__ void __launch_bounds__(RB_T, 10) k_rb_build(Dev d)
         }
         for (int i = lo + (int)threadIdx.x; i < hi; i += RB_T) W.pos[i - lo] = __ldg(d.spos + i);
         __syncthreads();
-        if (p - c.slot0 < D.n_new) build_row(d, p, D, c, R, W);
+        if (p - c.slot0 < D.n_new) build_row<true>(d, p, d.perm[p], D, c, R, &W);
     }
-}
-
-__global__ void k_rb_finish(Dev d)
-{
-    if (!d.g->any) return;
-    for (int k = threadIdx.x; k < d.B; k += blockDim.x) {
-        InstD& D = d.id[k];
-        if (D.flag) {
-            D.cur ^= 1;
-            D.lp ^= 1;
-            if (D.flag != 3) atomicAdd(&d.g->rebuilds, 1ull);
-            D.flag = 0;
-            D.n = D.n_new;
-            D.nbin = D.n_new;
-            D.disp = 0.f;
-        }
-    }
-    __syncthreads();
-    // the tiles fused steps walk: per instance the pairs of tiles that hold its live slots
-    // (offsets by a scan over a chunk of instances, then the chunk's ranges written by the block)
-    __shared__ unsigned s_off[256], s_lt[256];
-    __shared__ int s_t0[256];
-    unsigned base = 0u;
-    for (int k0 = 0; k0 < d.B; k0 += blockDim.x) {
-        const int k = k0 + (int)threadIdx.x;
-        unsigned lt = 0u;
-        if (k < d.B) lt = 2u * (unsigned)((d.id[k].n + 2 * TILE - 1) / (2 * TILE));
-        unsigned tot;
-        const unsigned off = base + block_exclusive_scan(lt, &tot);
-        s_off[threadIdx.x] = off;
-        s_lt[threadIdx.x] = lt;
-        s_t0[threadIdx.x] = k < d.B ? d.ic[k].slot0 / TILE : 0;
-        __syncthreads();
-        const int nk = min((int)blockDim.x, d.B - k0);
-        for (int j = 0; j < nk; ++j)
-            for (unsigned i = threadIdx.x; i < s_lt[j]; i += blockDim.x) d.live_tiles[s_off[j] + i] = s_t0[j] + (int)i;
-        __syncthreads();
-        base += tot;
-    }
-    if (threadIdx.x == 0) {
-        d.g->nlive = (int)base;
-        d.g->any = 0u;
-        d.g->ncubes = 0;
-    }
+    rb_finish(d);
 }
 
 // ============================================================= contact law
@@ -1652,25 +1828,6 @@ __device__ __forceinline__ void step_finish_instances(const Dev& d)
             }
         }
     }
-}
-
-// counters of the blocks that are done: a release of the block's earlier writes and an acquire of
-// the other blocks' (lighter than __threadfence, which is a sequentially consistent fence)
-__device__ __forceinline__ unsigned add_acq_rel(unsigned* p)
-{
-    unsigned v;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void add_release(unsigned* p)
-{
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
-}
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
 }
 
 // What a step kernel inside a graph does besides its step.  Step kernels of a graph are launched
@@ -2694,7 +2851,7 @@ struct Plan {
     unsigned ncodes = 0, nparts = 0;
     // offsets
     size_t o_pos[2], o_vel[2], o_omg[2], o_nbr[2], o_hist[2], o_cnt[2], o_hmask[2], o_fext[2], o_whist[2], o_wseg[2], o_wrem;
-    size_t o_cellcode, o_cslot, o_perm, o_fin, o_spos, o_sid, o_ccount, o_crange, o_cubes, o_part, o_pinst, o_soi, o_tile, o_live, o_bar, o_ic, o_id, o_spread, o_g,
+    size_t o_cellcode, o_cslot, o_perm, o_fin, o_spos, o_sid, o_ccount, o_crange, o_cubes, o_cdir, o_part, o_pinst, o_soi, o_tile, o_live, o_bar, o_ic, o_id, o_spread, o_g,
         o_goff, o_outF, o_outT, o_outV, o_outW, o_outWX, o_xi, o_cmask, o_stage, o_hl, o_small, o_wgeo;
     size_t bytes = 0;
 };
@@ -2854,6 +3011,7 @@ dem_status make_plan(const dem_config* cfg, Plan& p, std::string& err)
     p.o_ccount = L.take((size_t)p.ncodes * 4);
     p.o_crange = L.take((size_t)p.ncodes * 8);
     p.o_cubes = L.take(((size_t)p.ncodes / CUBE + 1) * 4);
+    p.o_cdir = L.take((size_t)p.ncodes / CUBE + 1);
     p.o_part = L.take((size_t)std::max(1u, p.nparts) * 4);
     p.o_pinst = L.take((size_t)std::max(1u, p.nparts) * 4);
     p.o_soi = L.take(N * 4);
@@ -2959,10 +3117,9 @@ dem_status launch_rebuild(dem_ctx* ctx, cudaStream_t st)
     else
         k_rb_tilesort<<<gt, TILE, 0, st>>>(d);
     if (ctx->list_staged)
-        k_rb_build<<<ctx->grid_build_staged, RB_T, 0, st>>>(d);
+        k_rb_windows<<<ctx->grid_build_staged, RB_T, row_smem(ctx->Lmax), st>>>(d);
     else
         k_rb_cubes<<<ctx->grid_build, CB_T, cube_smem(ctx->Lmax), st>>>(d);
-    k_rb_finish<<<1, 256, 0, st>>>(d);          // 256 threads: its shared arrays
     CU(cudaGetLastError());
     return DEM_OK;
 }
@@ -2983,7 +3140,7 @@ bool capturing(dem_ctx* ctx)
 // Lists valid for the current state, on the context's stream: nothing to do when nothing ran since
 // the last build that could ask for one; the chain when a state was written, or into a capture of the
 // caller's; otherwise the chain behind one condition, where a graph holds it (one launch instead of
-// nine kernels that find nothing to do), else the chain.
+// eight kernels that find nothing to do), else the chain.
 dem_status ensure_lists(dem_ctx* ctx)
 {
     const bool cap = capturing(ctx);
@@ -3468,6 +3625,7 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
     d.ccount = (unsigned*)(base + p.o_ccount);
     d.crange = (uint2*)(base + p.o_crange);
     d.cubes = (int*)(base + p.o_cubes);
+    d.cube_dir = (unsigned char*)(base + p.o_cdir);
     d.part = (unsigned*)(base + p.o_part);
     d.part_inst = (int*)(base + p.o_pinst);
     d.slot_of_id = (int*)(base + p.o_soi);
@@ -3578,9 +3736,9 @@ dem_status dem_create(const dem_config* cfg, void* workspace, int64_t workspace_
         int bb = 0;
         cudaFuncSetAttribute(k_rb_cubes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cube_smem(MAXL));
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_cubes, CB_T, cube_smem(ctx->Lmax));
-        ctx->grid_build = std::max(1, std::min((int)(ctx->ncodes / CUBE) + 1, std::max(1, nsm) * std::max(1, bb)));
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_build, RB_T, 0);
-        ctx->grid_build_staged = std::max(1, std::min(ctx->ntiles * (TILE / RB_T), std::max(1, nsm) * std::max(1, bb)));
+        ctx->grid_build = std::max(1, std::min(std::max((int)(ctx->ncodes / CUBE) + 1, ctx->ntiles), std::max(1, nsm) * std::max(1, bb)));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bb, k_rb_windows, RB_T, row_smem(ctx->Lmax));
+        ctx->grid_build_staged = std::max(1, std::min(ctx->ntiles, std::max(1, nsm) * std::max(1, bb)));
         cudaGetLastError();
     }
     *out = ctx;
@@ -3737,7 +3895,7 @@ dem_status dem_step(dem_ctx* ctx, int64_t nsteps)
     while (done < nsteps) {
         // the graph, also for a remainder of at least 1/GRAPH_PART of its steps (the step kernels
         // beyond it find none left and end at once, about 4 us each with their share of the graph's
-        // other nodes, where a step launched alone comes with the nine kernels of the rebuild
+        // other nodes, where a step launched alone comes with the eight kernels of the rebuild
         // chain, 20 us or more); fused steps run any number
         const int64_t left = nsteps - done;
         // (a remainder inside a capture of the caller's is launched step by step)

@@ -61,7 +61,7 @@ struct dem_ctx {
     int fused_threads = 0, fused_blocks = 0;   // its launch in the current graph
     cudaGraph_t rb_graph = nullptr;
     cudaGraph_t rb_if_graph = nullptr;   // the rebuild chain behind one condition, for calls that need valid
-    cudaGraphExec_t rb_if = nullptr;     // lists (reads, coupling): a launch instead of the chain's nine
+    cudaGraphExec_t rb_if = nullptr;     // lists (reads, coupling): a launch instead of the chain's eight
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     std::vector<cudaEvent_t> ev0, ev1;   // around every EV_EVERY-th step kernel of the graph

@@ -35,6 +35,8 @@ constexpr int MAXL = 32;       // largest list width (one bit per entry in a 32-
 constexpr unsigned ID_MASK = 0x3fffffffu;   // particle ID (< 2^30)
 constexpr unsigned GONE_BIT = 0x40000000u;  // removed: dropped at the next list build
 constexpr unsigned WALL_BIT = 0x80000000u;  // in contact with the floor at the last step
+constexpr int DIR_CUBE = 0, DIR_SPARSE = 1, DIR_CROWDED = 2;   // the list build's kinds of cubes of cells
+constexpr unsigned DIR_ALL = 7u;
 constexpr int BAR_LINE = 16;   // 64-bit words per line of the fused steps' barrier
 constexpr int MAX_WP = 8;      // points of an axisymmetric wall polyline
 
@@ -151,7 +153,9 @@ struct Glob {
     long long todo;            // steps of the next graph launch (0: as many as the graph was built for)
     int nlive;                 // entries of live_tiles
     unsigned test_stall;       // 1: the next fused launch's first block skips its first barrier
-    int ncubes;                // list build: entries of cubes
+    unsigned long long cubes[3];   // list build, by DIR_*: {number of cubes, their particles}
+    unsigned left;             // list build: the kinds of cubes left out of the build by cubes (cube_route)
+    unsigned rb_done;          // list build: blocks that are done
     unsigned pool;             // SM-wide step blocks: slices claimed from the shared pool this launch
 };
 
@@ -178,7 +182,8 @@ struct Dev {
     int* sid;                  // particle IDs in cell order (list build)
     unsigned* ccount;
     uint2* crange;             // per cell code: {first cell-order position (exclusive scan), count}
-    int* cubes;                // list build: first cell codes of the cubes (64 codes) that hold particles
+    int* cubes;                // list build: first cell codes of the cubes (64 codes) that hold particles, those
+                               // of few from the back
     unsigned* part;
     int* part_inst;            // instance owning each scan chunk of cell codes (-1: padding)
     int* slot_of_id;
@@ -206,6 +211,7 @@ struct Dev {
     int Lmax;
     unsigned ncodes;
     unsigned nparts;
+    unsigned char* cube_dir;   // list build, per cube that holds particles: DIR_*
 };
 
 // DEM_CHECKS: true if i lies in [0, n); otherwise records ST_BOUNDS, the slot s, the index and
