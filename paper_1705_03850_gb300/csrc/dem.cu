@@ -555,25 +555,16 @@ __device__ __forceinline__ void row_out(const Dev& d, int s, int old, int ps, co
 #pragma unroll
     for (int i = 0; i < N; ++i) id[i] = m[i] != ps ? d.sid[m[i]] : -2;
     if (tie) {
-        // equal keys (rare) by ID, so that the row does not depend on the scan order
-#pragma unroll 1
+        // equal keys by ID, so that the row does not depend on the scan order (those were counted as
+        // they came); unrolled, as lattices are full of them: 12 neighbours at one distance 386 -> 243 us a
+        // call with a build of 300,000 spheres, against pairs picked out of the registers one by one
+#pragma unroll
         for (int i = 1; i < N; ++i)
-#pragma unroll 1
+#pragma unroll
             for (int j = 0; j < i; ++j) {
-                float ki = 0.f, kj = 1.f;
-                int di = 0, dj = 0;
-#pragma unroll
-                for (int q = 0; q < N; ++q) {
-                    if (q == i) { ki = key[q]; di = id[q]; }
-                    if (q == j) { kj = key[q]; dj = id[q]; }
-                }
-                if (ki == kj && ki < INFINITY && dj > di) {   // counted the other way round above
-#pragma unroll
-                    for (int q = 0; q < N; ++q) {
-                        if (q == i) --r[q];
-                        if (q == j) ++r[q];
-                    }
-                }
+                const bool swap = key[j] == key[i] && id[j] > id[i];   // (not a neighbour: ID -2, all at one key)
+                r[i] -= swap ? 1 : 0;
+                r[j] += swap ? 1 : 0;
             }
     }
 #pragma unroll
@@ -908,9 +899,14 @@ struct CubeScratch {
     int off[CB_H + 1];                       // cell h's first position in the copied order
     int wsum[CB_T / 32];
 };
+// The candidates of a thread's row as positions of the copy, and for lists wider than the rows kept in
+// registers (CB_REG) their keys: longer rows are ordered in shared memory.  In registers, 33 candidates
+// spill 600 bytes a thread and take 528 comparisons for all 32 rows of a warp (calls with a build of
+// 300,000 spheres, rows of 20: 561 us, and 445 us in shared memory).
+constexpr int CB_REG = 17;
 __host__ __device__ constexpr size_t cube_smem(int lmax)
 {
-    const size_t rows = (size_t)(lmax + 1) * CB_T * 2;   // the candidates of a thread's row as positions of the copy
+    const size_t rows = (size_t)(lmax + 1) * CB_T * (lmax + 1 > CB_REG ? 6 : 2);
     return sizeof(CubeScratch) + rows > row_smem(lmax) ? sizeof(CubeScratch) + rows : row_smem(lmax);
 }
 
@@ -919,9 +915,12 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
     if (!d.g->any) return;
     extern __shared__ int4 cube_mem[];       // the cube and the rows of its particles, or rows alone
     CubeScratch& C = *reinterpret_cast<CubeScratch*>(cube_mem);
+    // [Lmax + 1][CB_T]: keys (wide lists), then candidates: the particle itself is among them
+    float* cube_rows = reinterpret_cast<float*>(&C + 1);
     const int tx = threadIdx.x, lane = tx & 31, warp = tx >> 5;
     const int Lmax = d.Lmax;
-    unsigned short* row = (unsigned short*)(&C + 1) + tx;   // [Lmax + 1][CB_T]: the particle itself is among them
+    float* keys = cube_rows + tx;
+    unsigned short* row = (unsigned short*)(cube_rows + (Lmax + 1 > CB_REG ? (Lmax + 1) * CB_T : 0)) + tx;
     const unsigned left = d.g->left;
     const int nfront = (left >> DIR_CUBE) & 1u ? 0 : (int)(d.g->cubes[DIR_CUBE] >> 32);
     const int ncubes = nfront + ((left >> DIR_SPARSE) & 1u ? 0 : (int)(d.g->cubes[DIR_SPARSE] >> 32));
@@ -1098,7 +1097,7 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
             }
             const bool overflow = nl > Lmax + 1;
             nl = min(nl, Lmax + 1);
-            const int most = __reduce_max_sync(0xffffffffu, nl);
+            const int most = __reduce_max_sync(0xffffffffu, nl);   // (at most Lmax + 1: the keys' room)
             if (!mine) continue;
             auto get = [&](int e, float& key, int& m) {
                 const int t = row[e * CB_T];
@@ -1110,8 +1109,24 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
             };
             if (most <= 9) row_out<9>(d, s, old, ps, D, c, nl, overflow, get);
             else if (most <= 13) row_out<13>(d, s, old, ps, D, c, nl, overflow, get);
-            else if (most <= 17) row_out<17>(d, s, old, ps, D, c, nl, overflow, get);
-            else row_out<MAXL + 1>(d, s, old, ps, D, c, nl, overflow, get);
+            else if (most <= CB_REG) row_out<CB_REG>(d, s, old, ps, D, c, nl, overflow, get);
+            else {
+                int nc = 0;                  // without the particle itself
+                for (int e = 0; e < nl; ++e) {
+                    float key;
+                    int m;
+                    const unsigned short t = row[e * CB_T];
+                    get(e, key, m);
+                    if (m == ps) continue;
+                    keys[nc * CB_T] = key;
+                    row[nc * CB_T] = t;
+                    ++nc;
+                }
+                row_sorted(
+                    d, s, old, D, nc, overflow, [&](int e) -> float& { return keys[e * CB_T]; },
+                    [&](int e) -> unsigned short& { return row[e * CB_T]; }, [&](int t) { return C.m[t]; });
+                move_state(d, s, old, D, c);
+            }
         }
     }
     rb_finish(d);
