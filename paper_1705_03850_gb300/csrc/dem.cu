@@ -889,7 +889,7 @@ __device__ __forceinline__ void rb_finish(const Dev& d)
 // and 4 to 7 resident blocks of 128 came within 5 % of this.
 constexpr int CB_T = RB_T;
 static_assert(CB_T == TILE, "a tile a block where cubes are left");
-constexpr int CB_CAP = 800;                  // positions of a cube and around it (5 blocks an SM with lists of 32)
+constexpr int CB_CAP = 800;                  // positions of a cube and around it
 constexpr int CB_H = 600;                    // cells of a cube and around it: 216, at most 66 x 3 x 3
 struct CubeScratch {
     int4 pos[CB_CAP];
@@ -899,14 +899,14 @@ struct CubeScratch {
     int off[CB_H + 1];                       // cell h's first position in the copied order
     int wsum[CB_T / 32];
 };
-// The candidates of a thread's row as positions of the copy, and for lists wider than the rows kept in
-// registers (CB_REG) their keys: longer rows are ordered in shared memory.  In registers, 33 candidates
-// spill 600 bytes a thread and take 528 comparisons for all 32 rows of a warp (calls with a build of
-// 300,000 spheres, rows of 20: 561 us, and 445 us in shared memory).
+// Rows of more candidates than this are ordered in place, with their keys in local memory, not in registers:
+// there, 33 candidates spill 600 bytes a thread and take 528 comparisons for all 32 rows of a warp (calls with
+// a build of 300,000 spheres, rows of 20: 561 us, and 445 us in place).  (Keys in shared memory take the L1
+// that the rows' way out lives on: 90 against 80 us in the build kernel, 300,000 spheres and lists of 32.)
 constexpr int CB_REG = 17;
 __host__ __device__ constexpr size_t cube_smem(int lmax)
 {
-    const size_t rows = (size_t)(lmax + 1) * CB_T * (lmax + 1 > CB_REG ? 6 : 2);
+    const size_t rows = (size_t)(lmax + 1) * CB_T * 2;   // the candidates of a thread's row as positions of the copy
     return sizeof(CubeScratch) + rows > row_smem(lmax) ? sizeof(CubeScratch) + rows : row_smem(lmax);
 }
 
@@ -915,12 +915,9 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
     if (!d.g->any) return;
     extern __shared__ int4 cube_mem[];       // the cube and the rows of its particles, or rows alone
     CubeScratch& C = *reinterpret_cast<CubeScratch*>(cube_mem);
-    // [Lmax + 1][CB_T]: keys (wide lists), then candidates: the particle itself is among them
-    float* cube_rows = reinterpret_cast<float*>(&C + 1);
     const int tx = threadIdx.x, lane = tx & 31, warp = tx >> 5;
     const int Lmax = d.Lmax;
-    float* keys = cube_rows + tx;
-    unsigned short* row = (unsigned short*)(cube_rows + (Lmax + 1 > CB_REG ? (Lmax + 1) * CB_T : 0)) + tx;
+    unsigned short* row = (unsigned short*)(&C + 1) + tx;   // [Lmax + 1][CB_T]: the particle itself is among them
     const unsigned left = d.g->left;
     const int nfront = (left >> DIR_CUBE) & 1u ? 0 : (int)(d.g->cubes[DIR_CUBE] >> 32);
     const int ncubes = nfront + ((left >> DIR_SPARSE) & 1u ? 0 : (int)(d.g->cubes[DIR_SPARSE] >> 32));
@@ -1097,7 +1094,7 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
             }
             const bool overflow = nl > Lmax + 1;
             nl = min(nl, Lmax + 1);
-            const int most = __reduce_max_sync(0xffffffffu, nl);   // (at most Lmax + 1: the keys' room)
+            const int most = __reduce_max_sync(0xffffffffu, nl);
             if (!mine) continue;
             auto get = [&](int e, float& key, int& m) {
                 const int t = row[e * CB_T];
@@ -1111,6 +1108,7 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
             else if (most <= 13) row_out<13>(d, s, old, ps, D, c, nl, overflow, get);
             else if (most <= CB_REG) row_out<CB_REG>(d, s, old, ps, D, c, nl, overflow, get);
             else {
+                float keys[MAXL + 1];
                 int nc = 0;                  // without the particle itself
                 for (int e = 0; e < nl; ++e) {
                     float key;
@@ -1118,12 +1116,12 @@ __global__ void __launch_bounds__(CB_T, 5) k_rb_cubes(Dev d)
                     const unsigned short t = row[e * CB_T];
                     get(e, key, m);
                     if (m == ps) continue;
-                    keys[nc * CB_T] = key;
+                    keys[nc] = key;
                     row[nc * CB_T] = t;
                     ++nc;
                 }
                 row_sorted(
-                    d, s, old, D, nc, overflow, [&](int e) -> float& { return keys[e * CB_T]; },
+                    d, s, old, D, nc, overflow, [&](int e) -> float& { return keys[e]; },
                     [&](int e) -> unsigned short& { return row[e * CB_T]; }, [&](int t) { return C.m[t]; });
                 move_state(d, s, old, D, c);
             }
