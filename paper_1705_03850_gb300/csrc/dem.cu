@@ -1548,16 +1548,12 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         jn3 = sub + 3 * LPP < ncnt ? jn3 : s;
         // removed below the removal height: parked until the next list build drops it (tested
         // here, after the row's first loads are in flight, so that live rows do not wait on it)
-        if (idw & GONE_BIT) {
-            if (MODE != 1 && sub == 0) {
+        if (MODE != 2 && (idw & GONE_BIT)) {
+            if (MODE == 0 && sub == 0) {
                 d.pos[cur ^ 1][s] = P;
                 d.vel[cur ^ 1][s] = Vv;
                 d.omg[cur ^ 1][s] = Wv;
-                if (MODE == 2) {
-                    d.hmask[hout][s] = 0u;
-                    d.whist[hout][s] = d.whist[hin][s];
-                }
-            } else if (MODE != 2) {
+            } else {
                 d.outWX[s] = make_float4(0.f, 0.f, 0.f, 0.f);
                 d.cmask[s] = 0ull;
             }
@@ -1590,6 +1586,18 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         // for every lane of a group)
 #pragma unroll
         for (int o = 1; o < LPP; o <<= 1) tm |= __shfl_xor_sync(gmask, tm, o);
+        // (rollouts have few removed particles, none as a rule: parked here, once the velocity has come, as
+        // waiting for it above costs their step 3 %)
+        if (MODE == 2 && (idw & GONE_BIT)) {
+            if (sub == 0) {
+                d.pos[cur ^ 1][s] = P;
+                d.vel[cur ^ 1][s] = Vv;
+                d.omg[cur ^ 1][s] = Wv;
+                d.hmask[hout][s] = 0u;
+                d.whist[hout][s] = d.whist[hin][s];
+            }
+            continue;
+        }
         // entries that left contact get no history (the read-out's contacts are in cmask)
         unsigned clr = MODE != 0 ? 0u : hm & ~tm & submask;
         while (clr) {
