@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace cgdem;
@@ -1175,7 +1176,8 @@ __device__ __forceinline__ Coef<float> coef_of(const InstC& c)
 // MODE 1: forces at the current state only, the outputs named in `want` (WANT_*) written.
 // MODE 2: one step from a saved state to another (rollouts): Dev's buffers 0 hold the state before
 // the step and receive nothing, buffers 1 receive the state after it, with its overlaps and their
-// mask; lists come from the instance's parity.  No displacement bound, no end of step.
+// mask; lists come from the instance's parity.  No displacement bound, no end of step.  PARK: with the
+// test for removed particles (contexts that could hold some: it costs such a step 3 %).
 //
 // Persistent grid: block b owns the contiguous tile range [b T / G, (b+1) T / G)
 // (neighbouring tiles share neighbours, which then hit in L1), one thread per
@@ -1373,7 +1375,7 @@ __device__ __forceinline__ void cp_async4(unsigned dst, const void* src)
 // per launch and then only flips its state buffer (all else in them is constant between list
 // builds).
 constexpr int WANT_F = 1, WANT_T = 2, WANT_V = 4, WANT_W = 8, WANT_WX = 16, WANT_CONTACTS = 32, WANT_XI = 64;
-template <int MODE, bool WALLS, int BS, int LPP, bool FUSED = false>
+template <int MODE, bool WALLS, int BS, int LPP, bool FUSED = false, bool PARK = false>
 __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, InstD& sd, float* smax, int& kstaged,
                                           const int* rows = nullptr, const int* rcnt = nullptr, int want = 0)
 {
@@ -1548,12 +1550,16 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         jn3 = sub + 3 * LPP < ncnt ? jn3 : s;
         // removed below the removal height: parked until the next list build drops it (tested
         // here, after the row's first loads are in flight, so that live rows do not wait on it)
-        if (MODE != 2 && (idw & GONE_BIT)) {
-            if (MODE == 0 && sub == 0) {
+        if ((MODE != 2 || PARK) && (idw & GONE_BIT)) {
+            if (MODE != 1 && sub == 0) {
                 d.pos[cur ^ 1][s] = P;
                 d.vel[cur ^ 1][s] = Vv;
                 d.omg[cur ^ 1][s] = Wv;
-            } else {
+                if (MODE == 2) {
+                    d.hmask[hout][s] = 0u;
+                    d.whist[hout][s] = d.whist[hin][s];
+                }
+            } else if (MODE != 2) {
                 d.outWX[s] = make_float4(0.f, 0.f, 0.f, 0.f);
                 d.cmask[s] = 0ull;
             }
@@ -1586,18 +1592,6 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         // for every lane of a group)
 #pragma unroll
         for (int o = 1; o < LPP; o <<= 1) tm |= __shfl_xor_sync(gmask, tm, o);
-        // (rollouts have few removed particles, none as a rule: parked here, once the velocity has come, as
-        // waiting for it above costs their step 3 %)
-        if (MODE == 2 && (idw & GONE_BIT)) {
-            if (sub == 0) {
-                d.pos[cur ^ 1][s] = P;
-                d.vel[cur ^ 1][s] = Vv;
-                d.omg[cur ^ 1][s] = Wv;
-                d.hmask[hout][s] = 0u;
-                d.whist[hout][s] = d.whist[hin][s];
-            }
-            continue;
-        }
         // entries that left contact get no history (the read-out's contacts are in cmask)
         unsigned clr = MODE != 0 ? 0u : hm & ~tm & submask;
         while (clr) {
@@ -1861,7 +1855,7 @@ struct StepCtl {
     cudaGraphConditionalHandle h_rb, h_loop;
 };
 
-template <int MODE, bool WALLS, int BS = TILE, int LPP = 1>
+template <int MODE, bool WALLS, int BS = TILE, int LPP = 1, bool PARK = false>
 __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int prime, StepCtl ctl)
 {
     __shared__ InstC sc;
@@ -1881,7 +1875,7 @@ __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int 
             return;
         }
     }
-    step_pass<MODE, WALLS, BS, LPP>(d, prime, sc, sd, smax, kstaged, nullptr, nullptr, MODE == 1 ? ctl.counted : 0);
+    step_pass<MODE, WALLS, BS, LPP, false, PARK>(d, prime, sc, sd, smax, kstaged, nullptr, nullptr, MODE == 1 ? ctl.counted : 0);
     if (MODE == 0) {
         // the last block to finish accumulates the bound per instance and decides on rebuilds
         if (threadIdx.x == 0) am_last = add_acq_rel(&d.g->counter) == gridDim.x - 1;
@@ -4249,13 +4243,18 @@ dem_status step_between(dem_ctx* ctx, const Snap& A, const Snap& B, int prime)
         d.hmask[i] = S[i]->hmask;
         d.whist[i] = S[i]->whist;
     }
-    const StepCtl ctl{};
-    switch (ctx->ro.lanes) {
-    case 2: k_step<2, false, TILE, 2><<<ctx->grid_lanes[0], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
-    case 4: k_step<2, false, TILE, 4><<<ctx->grid_lanes[1], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
-    case 8: k_step<2, false, TILE, 8><<<ctx->grid_lanes[2], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
-    default: k_step<2, false><<<ctx->grid_bs[1], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
-    }
+    auto go = [&](auto park) {
+        constexpr bool PARK = decltype(park)::value;
+        const StepCtl ctl{};
+        switch (ctx->ro.lanes) {
+        case 2: k_step<2, false, TILE, 2, PARK><<<ctx->grid_lanes[0], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+        case 4: k_step<2, false, TILE, 4, PARK><<<ctx->grid_lanes[1], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+        case 8: k_step<2, false, TILE, 8, PARK><<<ctx->grid_lanes[2], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+        default: k_step<2, false, TILE, 1, PARK><<<ctx->grid_bs[1], TILE, 0, ctx->stream>>>(d, prime, ctl); break;
+        }
+    };
+    if (ctx->may_remove) go(std::true_type{});
+    else go(std::false_type{});
     CU(cudaGetLastError());
     return DEM_OK;
 }
@@ -4349,6 +4348,7 @@ dem_status dem_set_walls(dem_ctx* ctx, int32_t k, const double* axis, int32_t np
         const double zu = std::ceil((z_remove - h.lo[2]) / q);   // removed: z < z_remove, i.e. z_units < zu
         if (!(zu < 2.0e9)) return fail(ctx, DEM_ERR_ARG, "z_remove above the representable range");
         if (zu > -2.0e9) w.zrem = (int)zu;
+        ctx->may_remove = true;
     }
     c = w;
     bool any = false;

@@ -1453,6 +1453,7 @@ dem_status dem_coupler_create(dem_ctx* coarse, dem_ctx* fine, const dem_coupling
     }
     ctx = fine;
     CU(cudaStreamSynchronize(s));
+    if (cp->g.drain) fine->may_remove = true;
     // first sample of the coarse positions
     cp->g.call = 0;
     cudaStreamSynchronize(coarse->stream);

@@ -44,6 +44,7 @@ struct dem_ctx {
     bool walls = false;               // some instance has axisymmetric walls (step kernel variant)
     bool count_stale = false;         // a coupling call changed the IDs handed out on the device
     bool have_state = false;
+    bool may_remove = false;          // a removal height or drain faces were set: removed particles may sit in slots
     // host knowledge of the lists: lists_ok, no list build can be pending on the device (nothing
     // ran since the last one that could ask for one); must_build, one certainly is (a written state)
     bool lists_ok = false;

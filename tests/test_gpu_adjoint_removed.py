@@ -46,3 +46,22 @@ def test_the_gradients_are_those_of_the_rest():
     # (its KE does not depend on the material): near and far pairs give the block's gradients, up to
     # the order of the slots in the sums (float states, sums in double)
     np.testing.assert_allclose(_rollout(4, 1, False), _rollout(4, 1, True), rtol=1e-12)
+
+
+def test_particles_marked_at_a_drain_face_do_not_enter_the_gradients():
+    # a coupling call marks the top half-layer of the fine level, which touches the layer below it
+    A, _, fine_wl, spec = workloads.coupling_case()
+    out = []
+    for every in (1, 5, 12):
+        coarse = dem.from_workload(A)
+        fine = dem.DEM([dem.desc_from_workload(fine_wl, capacity=fine_wl.n + 4000)])
+        fine.write_state(fine_wl.x, fine_wl.v, fine_wl.w, fine_wl.r, fine_wl.m)
+        cp = dem.Coupler(coarse, fine, **dict(spec, hi=(0.024, 0.024, 0.016), feed_faces=1, drain_faces=1 << 5))
+        fine.step(20)
+        cp.couple()
+        gone = int(np.isnan(fine.read(dem.RADIUS)).sum())
+        assert gone > 20
+        fine.rollout_forward(12, every)
+        out.append(fine.rollout_adjoint(np.array([[1.0, 0.0]]), np.array([[0.0, 0.0]])))
+    assert np.isfinite(out[0]).all() and (out[0] != 0).all()
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
