@@ -185,10 +185,11 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_down(Dev d)
 // takes longer (a call of 532 against 475 us, cells of 3.4), and the few cubes at a bed's rim a round alone.
 // Sparse ones by the time of either way, as a block looks up 216 cells whatever the cube holds: with n
 // particles a cube 5.4 + 0.25 n ns a cube there, on the whole chip, and 0.159 + 0.0048 n ns a particle
-// here, with 20 us for doing both (calls with a build of 300,000 spheres, by cubes and by threads: n = 98
-// 193 and 289 us, 49 202 and 219, 38 204 and 166, 25 238 and 160, 10 401 and 153, 0.6 3230 and 904); from
-// 2,000 cubes, as one or two rounds of blocks are over before (10,000 spheres, n = 25: 73 and 82 us; n = 3: 95
-// and 79).
+// here (calls with a build of 300,000 spheres, by cubes and by threads: n = 98 193 and 289 us, 49 202 and
+// 219, 38 204 and 166, 25 238 and 160, 10 401 and 153, 0.6 3230 and 904).  Doing both costs 20 us more and
+// warps of which few lanes have work, as sparse cubes lie among the others (the ends of 64 columns of 10,000
+// spheres: 320 against 222 us in the kernel), so the others' particles count too.  From 2,000 cubes, as one
+// or two rounds of blocks are over before (10,000 spheres, n = 25: 73 and 82 us; n = 3: 95 and 79).
 __device__ __forceinline__ unsigned cube_route(const Dev& d)
 {
     float N[3], P[3];
@@ -204,7 +205,7 @@ __device__ __forceinline__ unsigned cube_route(const Dev& d)
     auto cube = [&](int i) { return 5.4f * N[i] + 0.25f * P[i]; };
     auto direct = [&](int i) { return 0.159f * P[i] + 0.0048f * P[i] * P[i] / fmaxf(N[i], 1.f); };
     const float all = cube(DIR_CUBE) + cube(DIR_SPARSE);
-    const float both = cube(DIR_CUBE) + direct(DIR_SPARSE) + (pc > 0.f ? 0.f : 20000.f);
+    const float both = cube(DIR_CUBE) + direct(DIR_SPARSE) + 0.159f * P[DIR_CUBE] + 20000.f;
     const float none = direct(DIR_CUBE) + direct(DIR_SPARSE);
     if (none < all && none < both) left = DIR_ALL;
     else if (both < all) left |= 1u << DIR_SPARSE;
@@ -323,8 +324,7 @@ __device__ __forceinline__ unsigned order_contacts(const Dev& d, const InstD& D,
 // order), so that the 32 rows a warp of the step kernel walks together have
 // similar lengths.  Results do not depend on the slot order: every particle sums
 // its own row in the row's order.  Also writes the cell-order copies of
-// positions and IDs that the list build scans.  Results do not depend on the slot order: every particle sums
-// its own row in the row's order.
+// positions and IDs that the list build scans.
 __global__ void __launch_bounds__(TILE) k_rb_tilesort(Dev d)
 {
     if (!d.g->any) return;
@@ -1405,8 +1405,8 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
     // fused steps of one instance deal the slices out to the blocks in turn (slice v to block v mod G):
     // tiles at a wall or in a dense spot, which sit together in the slots' order, would otherwise make
     // a few blocks twice as slow as the rest (28,000 cycles against 13,000 to 17,000 in a discharging
-    // 23,438-sphere silo, 200 steps of which take 2440 us instead of 2940), and there is no locality
-    // in an SM to lose, as fused steps read the neighbours' state from L2
+    // 23,438-sphere silo, which it made 18 % faster), and there is no locality in an SM to lose, as
+    // fused steps read the neighbours' state from L2
     const bool dealt = FUSED && d.B == 1;
     const int u0 = dealt ? 0 : (int)((long long)blockIdx.x * NU / gridDim.x);
     const int u1 = dealt ? (NV + (int)gridDim.x * WPB - 1) / ((int)gridDim.x * WPB)
@@ -1592,7 +1592,9 @@ __device__ __forceinline__ void step_pass(const Dev& d, int prime, InstC& sc, In
         // for every lane of a group)
 #pragma unroll
         for (int o = 1; o < LPP; o <<= 1) tm |= __shfl_xor_sync(gmask, tm, o);
-        // entries that left contact get no history (the read-out's contacts are in cmask)
+        // entries that left contact get no history: their bit goes from the mask, which every reader checks
+        // (the read-out's contacts are in cmask).  Nothing reads the zeros, but leaving them out gained
+        // nothing (-0.3 % on a 1M bed, +0.8 % on the fused silo)
         unsigned clr = MODE != 0 ? 0u : hm & ~tm & submask;
         while (clr) {
             const int e = __ffs(clr) - 1;
@@ -1914,14 +1916,15 @@ __global__ void __launch_bounds__(BS, (step_minb<BS, LPP>())) k_step(Dev d, int 
 //   words alternate by the tag's parity, as a block can be one step ahead, never two.)  With
 //   several instances the last block to arrive ends the step for each and releases the others.
 // - the barrier's cost is its fences and the arrivals at one word: one release and one acquire per
-//   block, by its first thread, and few blocks, one per SM.  A 1,440-sphere box on 96 blocks spent
-//   3,400 cycles of a step there, against 8,000 where each block wrote a word of its own and read
-//   all others', and 10,000 with fences by every warp; the 23,438-sphere silo on 736 blocks of 128
-//   threads 8,000 cycles, against 23,000.
+//   block, by its first thread, and few blocks, one per SM.  A 1,440-sphere box spends 3,400 to 3,900
+//   cycles of a step there, against 8,000 where each block wrote a word of its own and read all
+//   others', and 10,000 with fences by every warp; the 23,438-sphere silo 4,000 to 6,000, on 736 blocks
+//   of 128 threads 8,000, and with fences by every warp 23,000.
 // - a block of one unit keeps its rows and row lengths in shared memory for the launch: they do not
 //   change between list builds, but the barrier's acquires empty the L1.
-// 200 steps of the 1,440-sphere box (8 lanes): 1265 against 1793 us with the counter's last arrival
-// ending the step, of the 23,438-sphere silo (4 lanes, walls) 2763 against 3100 us.
+// 200 steps: the 1,440-sphere box (8 lanes) 1,160 us, the 23,438-sphere silo (4 lanes, walls) 2,650 us,
+// against 1,850 and 2,950 to 3,130 us with the counter's last arrival ending the step, fences by every
+// warp, a block a tile and rows read from L2.
 constexpr unsigned long long BAR_WAIT_NS = 1000000000ull;   // a barrier wait gives up after 1 s
 constexpr unsigned BAR_POLLS = 1u << 24;                     // or after this many polls
 
