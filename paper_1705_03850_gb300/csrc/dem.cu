@@ -883,11 +883,11 @@ __device__ __forceinline__ void rb_finish(const Dev& d)
 // crowded cubes (cube_route) look their cells up one by one, by tiles, after the cubes, and so do at
 // once those of a cube with more than CB_CAP positions around it: a kernel of its own for them made
 // every call that launches the chain without a graph 2 to 4 us longer.
-// Bound by latency: of the 40,000 cycles a block spends on a cube of the 1M bed, half go to the
-// scan (16-byte shared loads at random, four candidates at a time) and a third to the row's way out.
-// One list build of a 1M bed adds 390 us to a step, of a 100,000-sphere bed 55 us, against 575 and
-// 78 us with a thread looking up and scanning its 27 cells in global memory; blocks of 192 threads
-// and 4 to 7 resident blocks of 128 came within 5 % of this.
+// Bound by latency (20 warps an SM, issue 46 % of the time, DRAM 8 %): waits for the gathers of the rows'
+// way out and for the scan's 16-byte shared loads at random, four candidates at a time.  A list build of
+// the settled, sheared 1M bed takes 630 us in all its kernels, 465 of them here, against 900 and 736 with a
+// thread looking up and scanning its 27 cells in global memory; blocks of 192 threads and 4 to 7
+// resident blocks of 128 came within 5 % of this.
 constexpr int CB_T = RB_T;
 static_assert(CB_T == TILE, "a tile a block where cubes are left");
 constexpr int CB_CAP = 800;                  // positions of a cube and around it
